@@ -18,7 +18,8 @@ constexpr int AT = 64;  // head width
 // eight of the head's 64 columns with 16-byte loads.
 __global__ void attn_bwd_dot_kernel(const bf16* __restrict__ dO, const bf16* __restrict__ O,
                                     float* __restrict__ Dout, int rows, int m, int d, int nh) {
-  const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int pz = pdl_enter();
+  const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x + pz) >> 3;
   const int sub = threadIdx.x & 7;
   const long items = (long)rows * nh;
   const bool live = gid < items;
@@ -54,7 +55,8 @@ __global__ void cross_gate_bwd_kernel(const bf16* __restrict__ dAg, const bf16* 
                                       float* __restrict__ Di, bf16* __restrict__ dqa,
                                       float* __restrict__ ga, int ldga, long rows, int L, int d,
                                       int nh) {
-  const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;  // item
+  const int pz = pdl_enter();
+  const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x + pz) >> 3;  // item
   const int sub = threadIdx.x & 7;                                      // lane in the item
   const long items = rows * nh;
   const bool live = gid < items;
@@ -105,9 +107,8 @@ cudaError_t cross_gate_bwd(const bf16* dAg, const bf16* A, const bf16* qa, long 
   LaunchTimer lt("cross_gate_bwd", st, 4.0 * rows * d,
                  6.0 * rows * d + 2.0 * rows * ldq / 8.0 + 8.0 * rows * nh);
   if (((uintptr_t)dAg | (uintptr_t)A | (uintptr_t)dO) & 15) return cudaErrorInvalidValue;
-  cross_gate_bwd_kernel<<<(unsigned)((warps * 8 + 255) / 256), 256, 0, st>>>(
-      dAg, A, qa, ldq, b_a, dO, Di, dqa, ga, ldga, rows, L, d, nh);
-  return cudaGetLastError();
+  return launch_kernel(cross_gate_bwd_kernel, (unsigned)((warps * 8 + 255) / 256), 256, 0, st, dAg,
+                       A, qa, ldq, b_a, dO, Di, dqa, ga, ldga, rows, L, d, nh);
 }
 
 int take_dev_error_attention() { return take_dev_error_tu(); }
@@ -119,9 +120,8 @@ cudaError_t attn_bwd(const bf16* qkv, const bf16* O, const bf16* dO, const float
   {
     LaunchTimer lt("attn_bwd_dot", st, 2.0 * B * m * d, 4.0 * B * m * d + 4.0 * B * nh * m);
     if (((uintptr_t)dO | (uintptr_t)O) & 15) return cudaErrorInvalidValue;
-    attn_bwd_dot_kernel<<<(unsigned)((warps * 8 + 255) / 256), 256, 0, st>>>(dO, O, Di, B * m, m,
-                                                                             d, nh);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(attn_bwd_dot_kernel, (unsigned)((warps * 8 + 255) / 256),
+                                        256, 0, st, dO, O, Di, B * m, m, d, nh);
     if (e != cudaSuccess) return e;
   }
   return attn_bwd_tc(qkv, dO, lse, Di, dqkv, B, m, d, nh, causal, st);

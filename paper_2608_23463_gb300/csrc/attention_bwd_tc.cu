@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_enter();  // the setup above overlaps the kernel before this one
   uint32_t y_issued = 0, x_issued = 0;
 
   if (warp == 0) {
@@ -516,8 +517,7 @@ cudaError_t bw_launch(const CUtensorMap& x1, const CUtensorMap& x2, const CUtens
     return e;
   if (a.n_items == 0) return cudaSuccess;
   const int grid = std::min(a.n_items, num_sms());
-  kern<<<grid, BW_THREADS, BW_SMEM, st>>>(x1, x2, y1, y2, x1c, x2c, y1c, y2c, a);
-  return cudaGetLastError();
+  return launch_kernel(kern, grid, BW_THREADS, BW_SMEM, st, x1, x2, y1, y2, x1c, x2c, y1c, y2c, a);
 }
 
 }  // namespace

@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(FA_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_enter();  // the setup above overlaps the kernel before this one
   uint32_t kv_issued = 0, q_issued = 0;
 
   if (warp == 0 && lane == 0) {
@@ -493,8 +494,7 @@ cudaError_t fa_launch(const CUtensorMap& tq, const CUtensorMap& tkv, FaArgs& a, 
   }
   if (a.n_items == 0) return cudaSuccess;
   const int grid = std::min(a.n_items, num_sms());
-  kern<<<grid, FA_THREADS, FA_SMEM, st>>>(tq, tkv, a);
-  return cudaGetLastError();
+  return launch_kernel(kern, grid, FA_THREADS, FA_SMEM, st, tq, tkv, a);
 }
 
 double cross_pairs(int Lq, int Lk, int P, bool causal) {

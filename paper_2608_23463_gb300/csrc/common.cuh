@@ -59,6 +59,28 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// ------------------------------------------- programmatic dependent launch
+// Every kernel of the library is launched with programmatic stream
+// serialisation (launch_kernel): it starts as soon as the last CTA of the
+// kernel before it in the stream has left, sets up its shared memory, barriers
+// and TMEM while that kernel's writes drain, and waits here, before its first
+// access to global memory, until they are visible.  This takes a dependent
+// launch from about 6.5 us of a stream to 4.5 (a step of 36 small kernels 247
+// -> 175 us; the 262144-token layer, whose 33 launches lie under the power
+// cap, 3430 -> 3347 us).  No kernel lets its successor start any earlier
+// (griddepcontrol.launch_dependents): CTAs that arrive while others still run
+// pack onto the SMs that are free first, and a grid of one CTA per SM then
+// shares some SMs and leaves others idle (fp32 layer 61.7 us so, 69.3 with
+// triggers at the start of every kernel; the 262144-token layer 3435 us).
+// Returns zero, opaque to the compiler: a kernel adds it to an index of its
+// loads through __restrict__ pointers, which could otherwise be moved above
+// the wait (such memory counts as unmodified while the kernel runs).
+__device__ __forceinline__ int pdl_enter() {
+  int z;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(z) : : "memory");
+  return z;
+}
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

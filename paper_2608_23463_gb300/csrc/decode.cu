@@ -76,10 +76,11 @@ struct GemvArgs {
 // tiles are added in shared memory.
 template <int EPI>
 __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_kernel(GemvArgs a) {
+  const int pz = pdl_enter();
   constexpr int U = 4;  // K chunks in flight per warp
   __shared__ float red[GEMV_WARPS][16][GEMV_MAXB];
   __shared__ float s_inv[GEMV_MAXB];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x + pz, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int nt1 = (a.N + 15) / 16;
   // EPI_QKV launches also cover the alpha gate's W_a1 in tiles nt1, nt1+1, ...
@@ -189,11 +190,12 @@ __global__ void __launch_bounds__(512) split_kernel(
     const float* __restrict__ q, const bf16* __restrict__ Kc, const bf16* __restrict__ Vc,
     const int* __restrict__ n_proxy, int cap, int d, int nh, int splits, int R, float sl2,
     float* __restrict__ part, int* __restrict__ n_open, int P, int* __restrict__ valid) {
+  const int pz = pdl_enter();
   constexpr int LPK = DH / 8;  // threads per head
   constexpr int U = 4;
   extern __shared__ __align__(128) unsigned char ring[];  // [stage][K rows | V rows]
   __shared__ __align__(8) uint64_t full[SPLIT_STAGES];
-  const int s = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+  const int s = blockIdx.x + pz, b = blockIdx.y + pz, tid = threadIdx.x;
   const int h = tid / LPK, gl = tid % LPK;
   const bool active = tid * 8 < d;
   const int np = min(max(n_proxy[b], 0), cap);
@@ -323,12 +325,13 @@ __global__ void __launch_bounds__(COMBINE_G * DH) combine_kernel(
     const int* __restrict__ n_open, const int* __restrict__ valid, int P, int d, int nh, float sl2,
     const bf16* __restrict__ u, const bf16* __restrict__ W_a2, const float* __restrict__ b_a2,
     bf16* __restrict__ A) {
+  const int pz = pdl_enter();
   __shared__ float s_p[PF_DECODE_MAX_P];
   __shared__ float s_m[MAX_SPLITS], s_l[MAX_SPLITS];
   __shared__ __align__(16) float s_q[DH];
   __shared__ float s_red[2][COMBINE_G - 1][DH];
   __shared__ float s_alpha;
-  const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+  const int h = blockIdx.x + pz, b = blockIdx.y + pz, tid = threadIdx.x, lane = tid & 31;
   const int g = tid / DH, t = tid % DH;
   if (!valid[b]) return;  // flagged earlier; sequence untouched
   const int n = n_open[b];  // already advanced: open slots 0..n-1 incl. the new token
@@ -401,7 +404,8 @@ __global__ void __launch_bounds__(COMBINE_G * DH) combine_kernel(
 // Append bookkeeping: a sequence is appended iff its block is full and its
 // cache has room; others are flagged.  Runs after the cache rows are written.
 __global__ void append_finish_kernel(int* n_open, int* n_proxy, int B, int P, int cap) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const int b = blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (b >= B) return;
   if (n_open[b] == P && n_proxy[b] >= 0 && n_proxy[b] < cap) {
     n_proxy[b] += 1;
@@ -470,8 +474,8 @@ cudaError_t decode_step_launch(const DecodeLaunch& L, cudaStream_t st) {
     LaunchTimer lt("decode_qkv_alpha", st, 2.0 * nb * (3.0 * d + H) * d,
                    2.0 * (3.0 * d + H) * d + 6.0 * nb * d);
     const int tiles = (3 * d + 15) / 16 + (H + 15) / 16;
-    gemv_kernel<EPI_QKV><<<tiles, GEMV_WARPS * 32, 0, st>>>(g);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_kernel(gemv_kernel<EPI_QKV>, tiles, GEMV_WARPS * 32, 0, st, g);
+    if (e != cudaSuccess) return e;
   }
   {
     dim3 grid(L.splits, B);
@@ -484,22 +488,17 @@ cudaError_t decode_step_launch(const DecodeLaunch& L, cudaStream_t st) {
       return e;
     LaunchTimer lt("decode_split", st, 4.0 * B * (double)L.cap * d,
                    4.0 * B * (double)L.cap * d);  // bytes: upper bound (full cache)
-    k<<<grid, nthr, smem, st>>>(q, L.K_proxy, L.V_proxy, L.n_proxy, L.cap, d, nh, L.splits, R,
-                                sl2, part, L.n_open, L.P, valid);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_kernel(k, grid, nthr, smem, st, q, L.K_proxy, L.V_proxy, L.n_proxy, L.cap, d, nh,
+                      L.splits, R, sl2, part, L.n_open, L.P, valid);
+    if (e != cudaSuccess) return e;
   }
   {
     dim3 grid(nh, B);
     LaunchTimer lt("decode_combine", st, 4.0 * B * d * L.P, 4.0 * B * d * L.P);
-    if (dh == 128)
-      combine_kernel<128><<<grid, COMBINE_G * 128, 0, st>>>(part, L.splits, q, L.K_open, L.V_open,
-                                                            L.n_open, valid, L.P, d, nh, sl2, u,
-                                                            L.W_a2, L.b_a2, A);
-    else
-      combine_kernel<64><<<grid, COMBINE_G * 64, 0, st>>>(part, L.splits, q, L.K_open, L.V_open,
-                                                          L.n_open, valid, L.P, d, nh, sl2, u,
-                                                          L.W_a2, L.b_a2, A);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_kernel(dh == 128 ? combine_kernel<128> : combine_kernel<64>, grid, COMBINE_G * dh, 0,
+                      st, part, L.splits, q, L.K_open, L.V_open, L.n_open, valid, L.P, d, nh, sl2,
+                      u, L.W_a2, L.b_a2, A);
+      if (e != cudaSuccess) return e;
   }
   for (int b0 = 0; b0 < B; b0 += GEMV_MAXB) {
     GemvArgs o{};
@@ -512,15 +511,16 @@ cudaError_t decode_step_launch(const DecodeLaunch& L, cudaStream_t st) {
     o.y = L.y + (size_t)b0 * d;
     o.valid = valid + b0;
     LaunchTimer lt("decode_out", st, 2.0 * o.B * d * (double)d, 2.0 * d * (double)d + 6.0 * o.B * d);
-    gemv_kernel<EPI_OUT><<<(d + 15) / 16, GEMV_WARPS * 32, 0, st>>>(o);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_kernel(gemv_kernel<EPI_OUT>, (d + 15) / 16, GEMV_WARPS * 32, 0, st, o);
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
 // Prefill: every sequence's cache holds m proxies and r open tokens.
 __global__ void prefill_counts_kernel(int* n_open, int* n_proxy, int B, int m, int r) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const int b = blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (b < B) {
     n_proxy[b] = m;
     n_open[b] = r;
@@ -529,14 +529,14 @@ __global__ void prefill_counts_kernel(int* n_open, int* n_proxy, int B, int m, i
 
 cudaError_t prefill_counts(int* n_open, int* n_proxy, int B, int m, int r, cudaStream_t st) {
   LaunchTimer lt("prefill_counts", st, 0.0, 8.0 * B);
-  prefill_counts_kernel<<<(B + 127) / 128, 128, 0, st>>>(n_open, n_proxy, B, m, r);
-  return cudaGetLastError();
+  return launch_kernel(prefill_counts_kernel, (B + 127) / 128, 128, 0, st, n_open, n_proxy, B, m,
+                       r);
 }
 
 cudaError_t append_finish(int* n_open, int* n_proxy, int B, int P, int cap, cudaStream_t st) {
   LaunchTimer lt("append_finish", st, 0.0, 16.0 * B);
-  append_finish_kernel<<<1, 32 * ((B + 31) / 32), 0, st>>>(n_open, n_proxy, B, P, cap);
-  return cudaGetLastError();
+  return launch_kernel(append_finish_kernel, 1, 32 * ((B + 31) / 32), 0, st, n_open, n_proxy, B, P,
+                       cap);
 }
 
 }  // namespace pf

@@ -13,7 +13,8 @@ constexpr int EW_THREADS = 256;
 
 __global__ void copy_block0_kernel(const bf16* __restrict__ src, long Ls, bf16* __restrict__ dst,
                                    long Ld, int d, long per_seq_vec) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
   const int b = blockIdx.y;
   if (i >= per_seq_vec) return;
   *reinterpret_cast<uint4*>(dst + (long)b * Ld * d + i * 8) =
@@ -22,7 +23,8 @@ __global__ void copy_block0_kernel(const bf16* __restrict__ src, long Ls, bf16* 
 
 __global__ void pad_rows_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst, long L,
                                 long Lp, int d) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;  // vector index in [Lp*d/8]
+  const int pz = pdl_enter();
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;  // vector index in [Lp*d/8]
   const int b = blockIdx.y;
   if (i >= Lp * d / 8) return;
   const long tok = i * 8 / d;
@@ -53,14 +55,15 @@ struct RowIdx {  // row r = (b*m + i)*k2 + grp
 
 __global__ void __launch_bounds__(EW_THREADS, 2) inj_bwd_kernel(InjBwdArgs a, float* __restrict__ part,
                                                                 long M, int N, long rows_per_chunk) {
-  const int col = (blockIdx.x * EW_THREADS + threadIdx.x) * INJ_COLS;
+  const int pz = pdl_enter();
+  const int col = (blockIdx.x * EW_THREADS + threadIdx.x + pz) * INJ_COLS;
   if (col >= N) return;
   const bf16* __restrict__ G = a.G;
   const bf16* __restrict__ X = a.X;
   const bf16* __restrict__ D = a.D;
   bf16* __restrict__ dD = a.dD;
   bf16* __restrict__ dX = a.dX;
-  const long r0 = (long)blockIdx.y * rows_per_chunk;
+  const long r0 = (long)blockIdx.y * rows_per_chunk + pz;
   const long r1 = min(M, r0 + rows_per_chunk);
   const int P = a.k1 * a.k2;
   const int ch = col % a.d, tq = col / a.d;
@@ -199,9 +202,10 @@ __device__ __forceinline__ IbRow ib_row(const InjBwdArgs& a, const RowIdx& ix, i
 __global__ void __launch_bounds__(256, 2) inj_bwd_stream_kernel(InjBwdArgs a,
                                                                float* __restrict__ part, long M,
                                                                int N, long rows_per_chunk) {
+  const int pz = pdl_enter();
   extern __shared__ __align__(128) uint8_t ib_smem[];
   __shared__ __align__(8) uint64_t full[IB_STAGES];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x + pz;
   const int col0 = blockIdx.x * IB_W, col = col0 + tid * 8;
   const long r0 = (long)blockIdx.y * rows_per_chunk;
   const long r1 = min(M, r0 + rows_per_chunk);
@@ -365,7 +369,8 @@ __device__ __forceinline__ float warp_sum(float v) {
 // q = 1..3 are left in chunk 0's slots of part for the gate reduction below.
 __global__ void inj_bwd_colsum_kernel(float* __restrict__ part, int n_chunks, int N,
                                       float* __restrict__ db_d1, int gates) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
   const int nq = gates ? 4 : 1;
   if (i >= (long)nq * N) return;
   const int q = (int)(i / N), col = (int)(i % N);
@@ -382,7 +387,8 @@ __global__ void inj_bwd_colsum_kernel(float* __restrict__ part, int n_chunks, in
 // totals of quantity q (q = 1: w_x, 2: w_dlt, 3: b_g).
 __global__ void inj_bwd_gates_kernel(const float* __restrict__ part, int N, int d, float* gw_x,
                                      float* gw_dlt, float* gb_g) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (i >= 3 * d) return;
   const int q = 1 + i / d, ch = i % d, T = N / d;
   float s = 0.f;
@@ -412,8 +418,9 @@ template <typename T>
 __global__ void __launch_bounds__(EW_THREADS) colsum_part_kernel(const T* __restrict__ X, long R,
                                                                  int C, int CG, long rows_per_chunk,
                                                                  float* __restrict__ part) {
+  const int pz = pdl_enter();
   __shared__ float s_acc[EW_THREADS * 8];
-  const int RL = EW_THREADS / CG, cg = threadIdx.x % CG, rl = threadIdx.x / CG;
+  const int RL = EW_THREADS / CG, cg = threadIdx.x % CG + pz, rl = threadIdx.x / CG;
   const int col = (blockIdx.x * CG + cg) * 8;
   const long r0 = (long)blockIdx.y * rows_per_chunk, r1 = min(R, r0 + rows_per_chunk);
   float acc[8] = {};
@@ -455,8 +462,9 @@ constexpr int CS_WARPS = 16;
 __global__ void __launch_bounds__(32 * CS_WARPS)
     colsum_final_kernel(const float* __restrict__ part, int n_chunks, int C,
                         float* __restrict__ out) {
+  const int pz = pdl_enter();
   __shared__ float s_w[CS_WARPS][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = (threadIdx.x & 31) + pz, w = threadIdx.x >> 5;
   const int col = blockIdx.x * 32 + lane;
   float a = 0.f;
   if (col < C)
@@ -507,13 +515,12 @@ cudaError_t colsum_impl(const T* X, long R, int C, float* out, float* part, cuda
   dim3 grid((C + cg * 8 - 1) / (cg * 8), nc);
   {
     LaunchTimer lt("colsum", st, (double)R * C, (double)R * C * sizeof(T));
-    colsum_part_kernel<T><<<grid, EW_THREADS, 0, st>>>(X, R, C, cg, rpc, part);
+    const cudaError_t e = launch_kernel(colsum_part_kernel<T>, grid, EW_THREADS, 0, st, X, R, C, cg,
+                                        rpc, part);
+    if (e != cudaSuccess) return e;
   }
-  {
-    LaunchTimer lt("colsum_final", st, (double)nc * C, 4.0 * nc * C);
-    colsum_final_kernel<<<(C + 31) / 32, 32 * CS_WARPS, 0, st>>>(part, nc, C, out);
-  }
-  return cudaGetLastError();
+  LaunchTimer lt("colsum_final", st, (double)nc * C, 4.0 * nc * C);
+  return launch_kernel(colsum_final_kernel, (C + 31) / 32, 32 * CS_WARPS, 0, st, part, nc, C, out);
 }
 
 }  // namespace
@@ -523,16 +530,14 @@ cudaError_t copy_block0(const bf16* src, long Ls, bf16* dst, long Ld, int B, int
   const long nvec = (long)rows * d / 8;
   dim3 grid((unsigned)((nvec + 255) / 256), B);
   LaunchTimer lt("copy_block0", st, 0.0, 32.0 * nvec * B);
-  copy_block0_kernel<<<grid, 256, 0, st>>>(src, Ls, dst, Ld, d, nvec);
-  return cudaGetLastError();
+  return launch_kernel(copy_block0_kernel, grid, 256, 0, st, src, Ls, dst, Ld, d, nvec);
 }
 
 cudaError_t pad_rows(const bf16* src, bf16* dst, int B, long L, long Lp, int d, cudaStream_t st) {
   const long nvec = Lp * d / 8;
   dim3 grid((unsigned)((nvec + 255) / 256), B);
   LaunchTimer lt("pad_rows", st, 0.0, 2.0 * B * (L + Lp) * d);
-  pad_rows_kernel<<<grid, 256, 0, st>>>(src, dst, L, Lp, d);
-  return cudaGetLastError();
+  return launch_kernel(pad_rows_kernel, grid, 256, 0, st, src, dst, L, Lp, d);
 }
 
 // The streaming form needs whole IB_W slices and enough rows per CTA to fill
@@ -561,12 +566,10 @@ cudaError_t inj_bwd_1d(const InjBwdArgs& a, float* part, int n_chunks, cudaStrea
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, IB_SMEM);
     if (e != cudaSuccess) return e;
     dim3 grid(N / IB_W, n_chunks);
-    inj_bwd_stream_kernel<<<grid, 256, IB_SMEM, st>>>(a, part, M, N, rpc);
-    return cudaGetLastError();
+    return launch_kernel(inj_bwd_stream_kernel, grid, 256, IB_SMEM, st, a, part, M, N, rpc);
   }
   dim3 grid((N / INJ_COLS + EW_THREADS - 1) / EW_THREADS, n_chunks);
-  inj_bwd_kernel<<<grid, EW_THREADS, 0, st>>>(a, part, M, N, rpc);
-  return cudaGetLastError();
+  return launch_kernel(inj_bwd_kernel, grid, EW_THREADS, 0, st, a, part, M, N, rpc);
 }
 
 cudaError_t inj_bwd_finalize(const float* part, int n_chunks, int N, int d, float* db_d1,
@@ -575,10 +578,11 @@ cudaError_t inj_bwd_finalize(const float* part, int n_chunks, int N, int d, floa
   const int gates = gw_x != nullptr ? 1 : 0;
   const long n = (long)(gates ? 4 : 1) * N;
   float* pw = const_cast<float*>(part);  // the column totals reuse chunk 0's slots
-  inj_bwd_colsum_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(pw, n_chunks, N, db_d1, gates);
-  if (gates)
-    inj_bwd_gates_kernel<<<(3 * d + 255) / 256, 256, 0, st>>>(part, N, d, gw_x, gw_dlt, gb_g);
-  return cudaGetLastError();
+  const cudaError_t e = launch_kernel(inj_bwd_colsum_kernel, (unsigned)((n + 255) / 256), 256, 0, st,
+                                      pw, n_chunks, N, db_d1, gates);
+  if (e != cudaSuccess || !gates) return e;
+  return launch_kernel(inj_bwd_gates_kernel, (3 * d + 255) / 256, 256, 0, st, part, N, d, gw_x,
+                       gw_dlt, gb_g);
 }
 
 namespace {
@@ -587,7 +591,8 @@ namespace {
 // formed and reduced modulo 2 pi in double precision, (cos, sin) stored in
 // single precision.  Shared by every sequence, head and by Q and K.
 __global__ void rope_table_kernel(float2* __restrict__ tab, int m) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (t >= m * 32) return;
   const int i = t >> 5, j = t & 31;
   const double theta = exp2(-(double)(2 * j) / 64.0 * 13.287712379549449);  // log2(10000)
@@ -601,7 +606,8 @@ __global__ void rope_table_kernel(float2* __restrict__ tab, int m) {
 // RoPE on Q | K in place, one thread per rotated pair, angles from the table.
 __global__ void rope_qk_kernel(bf16* __restrict__ qk, long ld, long rows, int m, int d,
                                const float2* __restrict__ tab, float sgn) {
-  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (t >= rows * d) return;  // d pairs per row: d / 2 in Q, d / 2 in K
   const long row = t / d;
   const int col = 2 * (int)(t % d);
@@ -614,7 +620,8 @@ __global__ void rope_qk_kernel(bf16* __restrict__ qk, long ld, long rows, int m,
 
 __global__ void add_f32_bf16_kernel(const bf16* __restrict__ a, const float* __restrict__ b,
                                     float* __restrict__ of, bf16* __restrict__ ob, long n4) {
-  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (t >= n4) return;
   const uint2 u = reinterpret_cast<const uint2*>(a)[t];
   const float2 x = unpack_bf16(u.x), y = unpack_bf16(u.y);
@@ -635,12 +642,12 @@ cudaError_t rope_qk(bf16* qk, long ld, int B, int m, int d, float2* tab, bool in
   const long rows = (long)B * m, n = rows * d;
   {
     LaunchTimer lt("rope_table", st, 0.0, 8.0 * m * 32);
-    rope_table_kernel<<<(m * 32 + 255) / 256, 256, 0, st>>>(tab, m);
+    const cudaError_t e = launch_kernel(rope_table_kernel, (m * 32 + 255) / 256, 256, 0, st, tab, m);
+    if (e != cudaSuccess) return e;
   }
   LaunchTimer lt("rope_qk", st, 6.0 * n, 8.0 * n);
-  rope_qk_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(qk, ld, rows, m, d, tab,
-                                                              inverse ? -1.f : 1.f);
-  return cudaGetLastError();
+  return launch_kernel(rope_qk_kernel, (unsigned)((n + 255) / 256), 256, 0, st, qk, ld, rows, m, d,
+                       tab, inverse ? -1.f : 1.f);
 }
 
 cudaError_t add_f32_bf16(const bf16* a, const float* b, float* out_f, bf16* out_b, long n,
@@ -648,8 +655,8 @@ cudaError_t add_f32_bf16(const bf16* a, const float* b, float* out_f, bf16* out_
   if (n % 4) return cudaErrorInvalidValue;
   const long n4 = n / 4;
   LaunchTimer lt("add_f32_bf16", st, (double)n, 2.0 * n + (b ? 4.0 : 0.0) * n + 6.0 * n);
-  add_f32_bf16_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(a, b, out_f, out_b, n4);
-  return cudaGetLastError();
+  return launch_kernel(add_f32_bf16_kernel, (unsigned)((n4 + 255) / 256), 256, 0, st, a, b, out_f,
+                       out_b, n4);
 }
 
 long colsum_part_elems(long R, int C) { return (long)colsum_chunks(R, C) * C; }

@@ -45,9 +45,10 @@ __global__ void __launch_bounds__(FTHREADS) gemm_f32_kernel(const float* __restr
                                                            const float* __restrict__ bias,
                                                            const float* __restrict__ addend,
                                                            long ld_add, int vec, InjF32 inj) {
+  const int pz = pdl_enter();
   __shared__ __align__(16) float As[2][FK][FT + 4], Bs[2][FK][FT + 4];
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int m0 = blockIdx.y * FT, n0 = blockIdx.x * FT;
+  const int m0 = blockIdx.y * FT + pz, n0 = blockIdx.x * FT + pz;
   const int kbeg = blockIdx.z * Kc, kend = min(K, kbeg + Kc);
   C += (long)blockIdx.z * M * ldc;
   // thread t loads rows r = t / 8 + 32 i (i = 0, 1) and k = (t % 8) * 4 .. + 4
@@ -174,11 +175,12 @@ __global__ void __launch_bounds__(FTHREADS, 2) gemm_f32_cp_kernel(
     const float* __restrict__ A, long lda, const float* __restrict__ Bm, long ldb,
     float* __restrict__ C, long ldc, int M, int N, int K, int Kc, const float* __restrict__ bias,
     const float* __restrict__ addend, long ld_add, InjF32 inj) {
+  const int pz = pdl_enter();
   extern __shared__ __align__(16) float cps[];
   float* As = cps;                              // [stage][FT][CP_LD]
   float* Bs = cps + CP_STAGES * FT * CP_LD;     // [stage][FT][CP_LD]
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int m0 = blockIdx.y * FT, n0 = blockIdx.x * FT;
+  const int m0 = blockIdx.y * FT + pz, n0 = blockIdx.x * FT + pz;
   const int kbeg = blockIdx.z * Kc, kend = min(K, kbeg + Kc);
   const int nslab = kend > kbeg ? (kend - kbeg + FK - 1) / FK : 0;
   C += (long)blockIdx.z * M * ldc;
@@ -300,11 +302,12 @@ constexpr int ATT_Q = 8;  // one query per warp: 4x the CTAs of 32, a quarter of
 __global__ void __launch_bounds__(256) attn_f32_kernel(const float* __restrict__ qkv,
                                                        float* __restrict__ out, int m, int d,
                                                        int causal, float scale) {
+  const int pz = pdl_enter();
   __shared__ float Kt[64][65];                  // [dim][key]
   __shared__ __align__(16) float Vs[64][64];    // [key][dim]
   __shared__ __align__(16) float Qs[ATT_Q][64];
   __shared__ float Ps[8][64];    // per warp: the chunk's probabilities
-  const int b = blockIdx.z, h = blockIdx.y, q0 = blockIdx.x * ATT_Q;
+  const int b = blockIdx.z + pz, h = blockIdx.y, q0 = blockIdx.x * ATT_Q;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const long ld = 3L * d, rb = (long)b * m;
   for (int i = tid; i < ATT_Q * 16; i += 256) {
@@ -398,7 +401,8 @@ __global__ void inject_f32_kernel(const float* __restrict__ X, const float* __re
                                   const float* __restrict__ w_dlt, const float* __restrict__ b_g,
                                   long L, int d, int P, int k1, int k2, int m, int shift, int gated,
                                   long total4) {
-  const long e4 = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const long e4 = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (e4 >= total4) return;
   const int d4 = d >> 2;
   const long tokg = e4 / d4;  // global token (b * L + t)
@@ -430,7 +434,8 @@ __global__ void inject_f32_kernel(const float* __restrict__ X, const float* __re
 
 __global__ void pad_f32_kernel(const float* __restrict__ src, float* __restrict__ dst, long L,
                                long Lp, int d, long total) {
-  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (e >= total) return;
   const long b = e / (Lp * d), r = e % (Lp * d);
   dst[e] = (r < L * d) ? src[b * L * d + r] : 0.f;
@@ -447,10 +452,11 @@ __global__ void __launch_bounds__(256) splitk_f32_reduce(const float* __restrict
                                                          const float* __restrict__ bias,
                                                          const float* __restrict__ addend,
                                                          long ld_add) {
+  const int pz = pdl_enter();
   __shared__ float4 sums[RED_G][32];
   const int g = threadIdx.x >> 5, l = threadIdx.x & 31;
   const long n4 = (long)(N + 3) / 4;
-  const long q = (long)blockIdx.x * 32 + l;  // four-column group over [M, N / 4]
+  const long q = (long)blockIdx.x * 32 + l + pz;  // four-column group over [M, N / 4]
   const bool in = q < (long)M * n4;
   const long r = in ? q / n4 : 0;
   const int c = in ? (int)(q % n4) * 4 : 0;
@@ -517,13 +523,11 @@ cudaError_t launch_f32(dim3 grid, int vec, const float* A, long lda, const float
     static const cudaError_t attr = cudaFuncSetAttribute(
         gemm_f32_cp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CP_SMEM);
     if (attr != cudaSuccess) return attr;
-    gemm_f32_cp_kernel<<<grid, FTHREADS, CP_SMEM, st>>>(A, lda, B, ldb, C, ldc, M, N, K, Kc, bias,
-                                                        addend, ld_add, inj);
-  } else {
-    gemm_f32_kernel<<<grid, FTHREADS, 0, st>>>(A, lda, B, ldb, C, ldc, M, N, K, Kc, bias, addend,
-                                               ld_add, 0, inj);
+    return launch_kernel(gemm_f32_cp_kernel, grid, FTHREADS, CP_SMEM, st, A, lda, B, ldb, C, ldc, M,
+                         N, K, Kc, bias, addend, ld_add, inj);
   }
-  return cudaGetLastError();
+  return launch_kernel(gemm_f32_kernel, grid, FTHREADS, 0, st, A, lda, B, ldb, C, ldc, M, N, K, Kc,
+                       bias, addend, ld_add, 0, inj);
 }
 }  // namespace
 
@@ -540,9 +544,8 @@ cudaError_t gemm_f32(int M, int N, int K, const float* A, long lda, const float*
                                0, InjF32{}, st);
     if (e != cudaSuccess) return e;
     const long groups = (long)M * ((N + 3) / 4);
-    splitk_f32_reduce<<<(unsigned)((groups + 31) / 32), 256, 0, st>>>(scratch, S, M, N, C, ldc, bias,
-                                                                     addend, ld_add);
-    return cudaGetLastError();
+    return launch_kernel(splitk_f32_reduce, (unsigned)((groups + 31) / 32), 256, 0, st, scratch, S,
+                         M, N, C, ldc, bias, addend, ld_add);
   }
   dim3 grid((N + FT - 1) / FT, (M + FT - 1) / FT, 1);
   return launch_f32(grid, vec, A, lda, B, ldb, C, ldc, M, N, K, K, bias, addend, ld_add, InjF32{},
@@ -580,8 +583,8 @@ cudaError_t attn_f32(const float* qkv, float* out, int B, int m, int d, int nh, 
   const double pairs = (double)B * nh * (causal ? 0.5 * m * (m + 1.0) : (double)m * m);
   LaunchTimer lt("attn_f32", st, 4.0 * 64 * pairs, 4.0 * B * m * 4.0 * d);
   dim3 grid((m + ATT_Q - 1) / ATT_Q, nh, B);
-  attn_f32_kernel<<<grid, 256, 0, st>>>(qkv, out, m, d, causal ? 1 : 0, 1.0f / sqrtf(64.0f));
-  return cudaGetLastError();
+  return launch_kernel(attn_f32_kernel, grid, 256, 0, st, qkv, out, m, d, causal ? 1 : 0,
+                       1.0f / sqrtf(64.0f));
 }
 
 cudaError_t inject_f32(const float* X, const float* D, float* Xo, const float* w_x,
@@ -589,16 +592,15 @@ cudaError_t inject_f32(const float* X, const float* D, float* Xo, const float* w
                        int k2, int m, int shift, int gated, cudaStream_t st) {
   const long total4 = (long)B * L * d / 4;
   LaunchTimer lt("inject_f32", st, 0.0, 48.0 * total4);
-  inject_f32_kernel<<<(unsigned)((total4 + 255) / 256), 256, 0, st>>>(
-      X, D, Xo, w_x, w_dlt, b_g, L, d, P, k1, k2, m, shift, gated, total4);
-  return cudaGetLastError();
+  return launch_kernel(inject_f32_kernel, (unsigned)((total4 + 255) / 256), 256, 0, st, X, D, Xo,
+                       w_x, w_dlt, b_g, L, d, P, k1, k2, m, shift, gated, total4);
 }
 
 cudaError_t pad_f32(const float* src, float* dst, int B, long L, long Lp, int d, cudaStream_t st) {
   const long total = (long)B * Lp * d;
   LaunchTimer lt("pad_rows", st, 0.0, 4.0 * B * (L + Lp) * d);
-  pad_f32_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(src, dst, L, Lp, d, total);
-  return cudaGetLastError();
+  return launch_kernel(pad_f32_kernel, (unsigned)((total + 255) / 256), 256, 0, st, src, dst, L,
+                       Lp, d, total);
 }
 
 }  // namespace pf

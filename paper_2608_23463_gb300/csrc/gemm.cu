@@ -100,21 +100,8 @@ cudaError_t launch(int M, int N, int K, const CUtensorMap& ta, const CUtensorMap
     const long pair_tiles =
         (long)((N + BN - 1) / BN) * ((M + 2 * GEMM_BM - 1) / (2 * GEMM_BM)) * splits;
     if (pairs > 0 && pair_tiles >= pairs) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(2 * (unsigned)std::min<long>(pair_tiles, pairs));
-      cfg.blockDim = dim3(threads);
-      cfg.dynamicSmemBytes = smem2;
-      cfg.stream = st;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 2;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      e = cudaLaunchKernelEx(&cfg, kern2, ta, tb, tx, M, N, K, splits, epi);
-      if (e != cudaSuccess) return e;
-      return cudaGetLastError();
+      return launch_clusters(2, kern2, 2 * (unsigned)std::min<long>(pair_tiles, pairs), threads,
+                             smem2, st, ta, tb, tx, M, N, K, splits, epi);
     }
   }
   auto kern = gemm_tc_kernel<BN, AMN, BMN, Epi>;
@@ -123,8 +110,8 @@ cudaError_t launch(int M, int N, int K, const CUtensorMap& ta, const CUtensorMap
   if (e != cudaSuccess) return e;
   const long tiles = (long)((N + BN - 1) / BN) * ((M + GEMM_BM - 1) / GEMM_BM) * splits;
   const int grid = (int)std::min<long>(tiles, num_sms());
-  kern<<<grid, GemmRoles<Epi>::kThreads, smem, st>>>(ta, tb, tx, M, N, K, splits, epi);
-  return cudaGetLastError();
+  return launch_kernel(kern, grid, GemmRoles<Epi>::kThreads, smem, st, ta, tb, tx, M, N, K, splits,
+                       epi);
 }
 
 template <int BN, class Epi>
@@ -176,7 +163,8 @@ cudaError_t gemm_dispatch(int M, int N, int K, Operand A, Operand B, const Epi& 
 // out = sum_s part[s] (+ bias) (+ addend) -> fp32 and/or bf16, 4 columns per thread.
 __global__ void splitk_reduce_kernel(const float* __restrict__ part, int S, int M, int N,
                                      EpiLinearArgs e) {
-  const long i = ((long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  const int pz = pdl_enter();
+  const long i = ((long)blockIdx.x * blockDim.x + threadIdx.x + pz) * 4;
   if (i >= (long)M * N) return;
   const long row = i / N;
   const int col = (int)(i % N);
@@ -253,9 +241,8 @@ cudaError_t gemm_linear(int M, int N, int K, Operand A, Operand B, const EpiLine
     }
     LaunchTimer lt("splitk_reduce", st, (double)S * M * N, 4.0 * (S + 1.0) * M * N);
     const long quads = (long)M * N / 4;
-    splitk_reduce_kernel<<<(unsigned)((quads + 255) / 256), 256, 0, st>>>(e.splitk_scratch, S, M,
-                                                                          N, e);
-    return cudaGetLastError();
+    return launch_kernel(splitk_reduce_kernel, (unsigned)((quads + 255) / 256), 256, 0, st,
+                         e.splitk_scratch, S, M, N, e);
   }
   if ((e.add_bf16 && ((uintptr_t)e.add_bf16 & 15)) || (e.add_bf16 && e.ld_add_bf16 % 8))
     return cudaErrorInvalidValue;

@@ -250,6 +250,7 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
   if (PAIR) cluster_sync_all();  // both CTAs' barriers exist before any remote arrival
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_enter();  // the setup above overlaps the kernel before this one
   uint32_t issued = 0;
   bool x_pending = false;
   uint32_t x_parity = 0;

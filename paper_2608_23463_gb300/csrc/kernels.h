@@ -5,6 +5,39 @@
 
 namespace pf {
 
+// Launch with programmatic stream serialisation (pdl_enter in common.cuh,
+// which every kernel calls before it touches global memory).
+// launch_clusters: clusters of that many CTAs along x.
+template <class... P, class... A>
+cudaError_t launch_clusters(int cluster, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cluster > 1) {
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+  const cudaError_t last = cudaGetLastError();  // (also clears it)
+  return e != cudaSuccess ? e : last;
+}
+template <class... P, class... A>
+cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                          A&&... args) {
+  return launch_clusters(1, kern, grid, block, smem, st, args...);
+}
+
 // ------------------------------------------------------------------ GEMM
 // Operand of D[M,N] = sum_k A[m,k] B[n,k]: `mn` = 0 for K-major storage
 // ([rows=M or N, K], leading dimension ld >= K), 1 for MN-major storage

@@ -26,7 +26,8 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 __global__ void __launch_bounds__(256) patch_gather_stats_kernel(
     const bf16* __restrict__ X, bf16* __restrict__ Xp, float* __restrict__ stats, long T, int d,
     int patch, int gh, int gw) {
-  const long t = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int pz = pdl_enter();
+  const long t = ((long)blockIdx.x * blockDim.x + threadIdx.x + pz) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= T) return;
   const long HW = (long)gh * gw;
@@ -83,10 +84,11 @@ __global__ void __launch_bounds__(256) temb_fwd_kernel(const float* __restrict__
                                                        float* __restrict__ a1_out,
                                                        float* __restrict__ u_out,
                                                        float* __restrict__ gb_out) {
+  const int pz = pdl_enter();
   extern __shared__ float sm[];  // e [256], u [d]
   float* e = sm;
   float* u = sm + 256;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x + pz, tid = threadIdx.x + pz, lane = tid & 31, warp = tid >> 5;
   const float tb = 1000.f * t[b];
   if (tid < 128) {
     const float w = expf(-(float)tid * (9.210340371976184f / 128.f));  // ln(10000)/128
@@ -122,7 +124,8 @@ __global__ void __launch_bounds__(256) temb_fwd_kernel(const float* __restrict__
 __global__ void adaln_fwd_kernel(const float* __restrict__ H, const float* __restrict__ gb,
                                  float* __restrict__ n_out, float* __restrict__ rstd_out,
                                  bf16* __restrict__ Hq, long R, int d, int m) {
-  const long r = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int pz = pdl_enter();
+  const long r = ((long)blockIdx.x * blockDim.x + threadIdx.x + pz) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= R) return;
   const float* h = H + r * d;
@@ -156,8 +159,9 @@ __global__ void __launch_bounds__(256) inj_bwd_2d_kernel(
     const bf16* __restrict__ G, const bf16* __restrict__ X, const float* __restrict__ stats,
     const bf16* __restrict__ S, bf16* __restrict__ dD, bf16* __restrict__ dXd,
     float* __restrict__ part, long R, int d, int patch, int gh, int gw) {
+  const int pz = pdl_enter();
   __shared__ float red[8][2 * 256 * IB2_MAXI];
-  const int p = blockIdx.y, chunk = blockIdx.x;
+  const int p = blockIdx.y + pz, chunk = blockIdx.x + pz;
   const int py = p / patch, px = p % patch;
   const int npw = gw / patch, m = (gh / patch) * npw, P = patch * patch;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -240,7 +244,8 @@ __global__ void __launch_bounds__(256) inj_bwd_2d_kernel(
 // per column, chunks in order.
 __global__ void colsum_chunks_kernel(const float* __restrict__ part, int n_chunks, long C,
                                      float* __restrict__ out) {
-  const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const long c = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (c >= C) return;
   float v = 0.f;
   for (int k = 0; k < n_chunks; ++k) v += part[(long)k * C + c];
@@ -253,7 +258,8 @@ __global__ void adaln_bwd_kernel(const float* __restrict__ dHq, const float* __r
                                  const float* __restrict__ rstd, const float* __restrict__ gb,
                                  const float* __restrict__ dH_out, float* __restrict__ dHf,
                                  bf16* __restrict__ dHb, long R, int d, int m) {
-  const long r = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int pz = pdl_enter();
+  const long r = ((long)blockIdx.x * blockDim.x + threadIdx.x + pz) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= R) return;
   const float* gam = gb + (r / m) * 2 * d;
@@ -278,7 +284,8 @@ __global__ void adaln_bwd_kernel(const float* __restrict__ dHq, const float* __r
 // over a chunk of rows: part[b][chunk][0..d) and [d..2d).
 __global__ void adaln_param_part_kernel(const float* __restrict__ dHq, const float* __restrict__ nH,
                                         float* __restrict__ part, int d, int m, int chunks) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const int c = blockIdx.x * blockDim.x + threadIdx.x + pz;
   const int ck = blockIdx.y, b = blockIdx.z;
   if (c >= d) return;
   const int rows = (m + chunks - 1) / chunks;
@@ -296,7 +303,8 @@ __global__ void adaln_param_part_kernel(const float* __restrict__ dHq, const flo
 
 __global__ void adaln_param_final_kernel(const float* __restrict__ part, float* __restrict__ dgb,
                                          int d, int chunks, int B) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x + pz;
   if (i >= B * 2 * d) return;
   const int b = i / (2 * d), j = i % (2 * d);
   float s = 0.f;
@@ -307,7 +315,8 @@ __global__ void adaln_param_final_kernel(const float* __restrict__ part, float* 
 // du = W_t2^T dgb, da1 = du * SiLU'(a1), per image (thread per column i).
 __global__ void temb_bwd_du_kernel(const float* __restrict__ dgb, const bf16* __restrict__ W_t2,
                                    const float* __restrict__ a1, float* __restrict__ da1, int d) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
+  const int pz = pdl_enter();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x + pz, b = blockIdx.y;
   if (i >= d) return;
   float du = 0.f;
   for (int o = 0; o < 2 * d; ++o) du = fmaf(__bfloat162float(W_t2[(long)o * d + i]), dgb[(long)b * 2 * d + o], du);
@@ -322,7 +331,8 @@ __global__ void temb_wgrad_kernel(const float* __restrict__ dgb, const float* __
                                   const float* __restrict__ da1, const float* __restrict__ e,
                                   float* gW_t2, float* gb_t2, float* gW_t1, float* gb_t1, int d,
                                   int B) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pz = pdl_enter();
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
   const long n_w2 = 2L * d * d, n_b2 = 2L * d, n_w1 = (long)d * 256, n_b1 = d;
   float s = 0.f;
   if (i < n_w2) {
@@ -351,25 +361,23 @@ cudaError_t patch_gather_stats(const bf16* X, bf16* Xp, float* stats, int B, int
   if (d > 512 || d % 8 != 0) return cudaErrorInvalidValue;
   const long T = (long)B * gh * gw;
   LaunchTimer lt("patch_gather_stats", st, 0.0, 4.0 * T * d + 8.0 * T);
-  patch_gather_stats_kernel<<<(unsigned)((T * 32 + 255) / 256), 256, 0, st>>>(X, Xp, stats, T, d,
-                                                                             patch, gh, gw);
-  return cudaGetLastError();
+  return launch_kernel(patch_gather_stats_kernel, (unsigned)((T * 32 + 255) / 256), 256, 0, st, X,
+                       Xp, stats, T, d, patch, gh, gw);
 }
 
 cudaError_t temb_fwd(const float* t, int B, int d, const bf16* W_t1, const float* b_t1,
                      const bf16* W_t2, const float* b_t2, float* e, float* a1, float* u, float* gb,
                      cudaStream_t st) {
   LaunchTimer lt("temb_fwd", st, 2.0 * B * (256.0 * d + 2.0 * d * d), 2.0 * (256.0 * d + 2.0 * d * d));
-  temb_fwd_kernel<<<B, 256, (256 + d) * sizeof(float), st>>>(t, d, W_t1, b_t1, W_t2, b_t2, e, a1,
-                                                             u, gb);
-  return cudaGetLastError();
+  return launch_kernel(temb_fwd_kernel, B, 256, (256 + d) * sizeof(float), st, t, d, W_t1, b_t1,
+                       W_t2, b_t2, e, a1, u, gb);
 }
 
 cudaError_t adaln_fwd(const float* H, const float* gb, float* nH, float* rstd, bf16* Hq, long R,
                       int d, int m, cudaStream_t st) {
   LaunchTimer lt("adaln_fwd", st, 0.0, 10.0 * R * d);
-  adaln_fwd_kernel<<<(unsigned)((R * 32 + 255) / 256), 256, 0, st>>>(H, gb, nH, rstd, Hq, R, d, m);
-  return cudaGetLastError();
+  return launch_kernel(adaln_fwd_kernel, (unsigned)((R * 32 + 255) / 256), 256, 0, st, H, gb, nH,
+                       rstd, Hq, R, d, m);
 }
 
 long inj_bwd_2d_part_elems(long R, int d, int patch) {
@@ -385,23 +393,22 @@ cudaError_t inj_bwd_2d(const bf16* G, const bf16* X, const float* stats, const b
   {
     LaunchTimer lt("inj_bwd_2d", st, 0.0, 12.0 * R * P * (double)d);
     dim3 grid(n_chunks, P);
-    inj_bwd_2d_kernel<<<grid, 256, 0, st>>>(G, X, stats, S, dD, dXd, part, R, d, patch, gh, gw);
+    const cudaError_t e = launch_kernel(inj_bwd_2d_kernel, grid, 256, 0, st, G, X, stats, S, dD, dXd,
+                                        part, R, d, patch, gh, gw);
+    if (e != cudaSuccess || !db_d1) return e;
   }
-  if (db_d1) {
-    const long C = 2L * P * d;
-    LaunchTimer lt("colsum_final", st, (double)n_chunks * C, 4.0 * n_chunks * C);
-    colsum_chunks_kernel<<<(unsigned)((C + 255) / 256), 256, 0, st>>>(part, n_chunks, C, db_d1);
-  }
-  return cudaGetLastError();
+  const long C = 2L * P * d;
+  LaunchTimer lt("colsum_final", st, (double)n_chunks * C, 4.0 * n_chunks * C);
+  return launch_kernel(colsum_chunks_kernel, (unsigned)((C + 255) / 256), 256, 0, st, part, n_chunks,
+                       C, db_d1);
 }
 
 cudaError_t adaln_bwd(const float* dHq, const float* nH, const float* rstd, const float* gb,
                       const float* dH_out, float* dHf, bf16* dHb, long R, int d, int m,
                       cudaStream_t st) {
   LaunchTimer lt("adaln_bwd", st, 0.0, 18.0 * R * d);
-  adaln_bwd_kernel<<<(unsigned)((R * 32 + 255) / 256), 256, 0, st>>>(dHq, nH, rstd, gb, dH_out, dHf,
-                                                                    dHb, R, d, m);
-  return cudaGetLastError();
+  return launch_kernel(adaln_bwd_kernel, (unsigned)((R * 32 + 255) / 256), 256, 0, st, dHq, nH,
+                       rstd, gb, dH_out, dHf, dHb, R, d, m);
 }
 
 int adaln_param_chunks(int m) { return m < 64 ? 1 : (m < 4096 ? m / 64 : 64); }
@@ -412,10 +419,12 @@ cudaError_t adaln_param_grads(const float* dHq, const float* nH, float* part, fl
   {
     LaunchTimer lt("adaln_param", st, 0.0, 8.0 * B * m * (double)d);
     dim3 grid((d + 255) / 256, chunks, B);
-    adaln_param_part_kernel<<<grid, 256, 0, st>>>(dHq, nH, part, d, m, chunks);
+    const cudaError_t e =
+        launch_kernel(adaln_param_part_kernel, grid, 256, 0, st, dHq, nH, part, d, m, chunks);
+    if (e != cudaSuccess) return e;
   }
-  adaln_param_final_kernel<<<(B * 2 * d + 255) / 256, 256, 0, st>>>(part, dgb, d, chunks, B);
-  return cudaGetLastError();
+  return launch_kernel(adaln_param_final_kernel, (B * 2 * d + 255) / 256, 256, 0, st, part, dgb, d,
+                       chunks, B);
 }
 
 cudaError_t temb_bwd(const float* dgb, const bf16* W_t2, const float* a1, const float* u,
@@ -423,11 +432,11 @@ cudaError_t temb_bwd(const float* dgb, const bf16* W_t2, const float* a1, const 
                      cudaStream_t st) {
   LaunchTimer lt("temb_bwd", st, 0.0, 8.0 * d * d);
   dim3 g1((d + 255) / 256, B);
-  temb_bwd_du_kernel<<<g1, 256, 0, st>>>(dgb, W_t2, a1, da1, d);
+  const cudaError_t err = launch_kernel(temb_bwd_du_kernel, g1, 256, 0, st, dgb, W_t2, a1, da1, d);
+  if (err != cudaSuccess) return err;
   const long total = 2L * d * d + 2L * d + (long)d * 256 + d;
-  temb_wgrad_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(dgb, u, da1, e, g.W_t2, g.b_t2,
-                                                                    g.W_t1, g.b_t1, d, B);
-  return cudaGetLastError();
+  return launch_kernel(temb_wgrad_kernel, (unsigned)((total + 255) / 256), 256, 0, st, dgb, u, da1,
+                       e, g.W_t2, g.b_t2, g.W_t1, g.b_t1, d, B);
 }
 
 }  // namespace pf
