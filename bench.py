@@ -246,7 +246,7 @@ def kernel_files(label: str):
         return ["attention_bwd_tc.cu", "attention.cu", "common.cuh"]
     if label.startswith("decode_"):
         return ["decode.cu", "common.cuh"]
-    if label.startswith(("inj_bwd", "colsum", "copy_block0", "pad_rows")):
+    if label.startswith(("inj_bwd", "colsum", "pad_rows")):
         return ["elementwise.cu", "common.cuh"]
     return ["gemm_tc.cuh", "gemm.cu", "common.cuh"]
 

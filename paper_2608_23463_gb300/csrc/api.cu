@@ -194,7 +194,7 @@ FwdWs carve_fwd(Carve& wc, const pf_layer_desc& s, const Dims& g, void* saved) {
 }
 
 struct BwdWs {
-  bf16 *Xpad, *dXpad, *dD, *dZ, *dHbar, *dA, *dQKV, *dHb, *dY;
+  bf16 *Xpad, *dD, *dZ, *dHbar, *dA, *dQKV, *dHb, *dY;
   float *Di, *dHf, *part, *sk;
   long part_elems;
   size_t skb;
@@ -210,7 +210,6 @@ struct BwdWs {
 BwdWs carve_bwd(Carve& c, const pf_layer_desc& s, const Dims& g) {
   BwdWs w{};
   w.Xpad = g.ragged ? c.take<bf16>(g.B * g.Lp * g.df) : nullptr;
-  w.dXpad = g.ragged ? c.take<bf16>(g.B * g.Lp * g.df) : nullptr;
   if (g.cross) {
     w.Wqa = c.take<bf16>(g.ldq * g.d);
     w.dAg = c.take<bf16>(g.T * g.d);
@@ -495,7 +494,7 @@ pf_status layer_fwd_2d(const pf_layer_desc& s, const Dims& g, const pf_layer_par
     PF_CUDA(gemm_linear((int)g.R, d, d, {sv.Aatt, d, 0}, {static_cast<const bf16*>(p.W_o), d, 0}, with_sk(eo, sk, skb), cs));
   }
   {
-    EpiAffine2DArgs e{p.b_d1, sv.S, static_cast<bf16*>(X_out), sv.stats, sv.Xp, d, patch, gh, gw,
+    EpiAffine2DArgs e{p.b_d1, sv.S, static_cast<bf16*>(X_out), sv.stats, X, d, patch, gh, gw,
                       (int)g.m};
     set_gemm_tag("decompress_affine", (double)g.R * N1 * 8.0);
     PF_CUDA(gemm_affine2d((int)g.R, 2 * N1, d, {sv.Hbar, d, 0},
@@ -807,7 +806,7 @@ pf_status proxy_layer_fwd(const pf_layer_desc* desc, const pf_layer_params* prm,
     Zsrc = sv.Z;
   }
   {
-    EpiInjectArgs e{prm->b_d1, sv.D, Xsrc, Xo,
+    EpiInjectArgs e{prm->b_d1, sv.D, Xb, Xo,
                     prm->w_x, prm->w_dlt, prm->b_g,
                     df, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L, g.causal ? 1 : 0,
                     s.inject == PF_INJ_GATED ? 1 : 0};
@@ -815,7 +814,6 @@ pf_status proxy_layer_fwd(const pf_layer_desc* desc, const pf_layer_params* prm,
     PF_CUDA(gemm_inject1d((int)g.rows1, (int)g.N1, d, {Zsrc, d, 0},
                           {static_cast<const bf16*>(prm->W_d1), d, 0}, e, cs));
   }
-  if (g.causal) PF_CUDA(copy_block0(Xb, g.L, Xo, g.L, (int)g.B, df, (int)std::min(g.P, g.L), cs));
   return PF_OK;
 }
 
@@ -866,9 +864,7 @@ pf_status proxy_layer_bwd(const pf_layer_desc* desc, const pf_layer_params* prm,
     PF_CUDA(pad_rows(Xb, w.Xpad, (int)g.B, g.L, g.Lp, df, cs));
     Xsrc = w.Xpad;
   }
-  // direct injection gradient: written into dX, or into a block-padded buffer
-  // when L % P != 0 so the dX GEMM epilogue can prefetch it as whole tiles
-  bf16* dXd = g.ragged ? w.dXpad : dXb;
+  // the direct injection gradient goes into dX; the dX GEMM adds to it
   if (g.cross) {
     // the gated cross injection backward: output projection, gate, the
     // cross-attention (dQ of the tokens, dK / dV of the proxies), then the
@@ -924,31 +920,23 @@ pf_status proxy_layer_bwd(const pf_layer_desc* desc, const pf_layer_params* prm,
       PF_CUDA(gemm_linear((int)g.R, d, 2 * d, {w.dKVx, 2 * d, 0}, {W_kvx, d, 1},
                           with_sk(e, w.sk, w.skb), cs));
     }
-    // direct dX, in the block-padded layout when L % P != 0 (per sequence
-    // then, as the rows of different sequences are spaced differently)
-    const bool per_seq = g.ragged && g.B > 1;
-    for (long b = 0; b < (per_seq ? g.B : 1); ++b) {
+    {
       EpiLinearArgs e;
-      e.add_bf16 = G + b * g.L * d;
+      e.add_bf16 = G;
       e.ld_add_bf16 = d;
-      e.out_bf16 = dXd + b * (g.ragged ? g.Lp : g.L) * d;
+      e.out_bf16 = dXb;
       e.ld_bf16 = d;
-      const int rows = per_seq ? (int)g.L : T;
-      set_gemm_tag("bwd_dX_direct", (double)rows * (q + 2 * d) * 2.0);
-      PF_CUDA(gemm_linear(rows, d, q, {w.dQA + b * g.L * q, q, 0}, {w.Wqa, d, 1},
-                          with_sk(e, w.sk, w.skb), cs));
+      set_gemm_tag("bwd_dX_direct", (double)T * (q + 2 * d) * 2.0);
+      PF_CUDA(gemm_linear(T, d, q, {w.dQA, q, 0}, {w.Wqa, d, 1}, with_sk(e, w.sk, w.skb), cs));
     }
   } else {
     // injection backward: dD (proxy order), direct dX, gate and b_d1 gradients
     {
       const int nch = inj_bwd_chunks(g.rows1, N1);
-      InjBwdArgs a{G, Xb, sv.D, w.dD, dXd, g.ragged ? g.Lp : g.L, prm->w_x, prm->w_dlt, prm->b_g,
+      InjBwdArgs a{G, Xb, sv.D, w.dD, dXb, prm->w_x, prm->w_dlt, prm->b_g,
                    df, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L, (int)g.B, g.causal ? 1 : 0,
                    gated ? 1 : 0};
       PF_CUDA(inj_bwd_1d(a, w.part, nch, cs));
-      if (g.causal)
-        PF_CUDA(copy_block0(G, g.L, dXd, g.ragged ? g.Lp : g.L, (int)g.B, df,
-                            (int)std::min(g.P, g.L), cs));
       PF_CUDA(inj_bwd_finalize(w.part, nch, N1, df, grads->b_d1, gated ? grads->w_x : nullptr,
                                gated ? grads->w_dlt : nullptr, gated ? grads->b_g : nullptr, cs));
     }
@@ -1096,7 +1084,7 @@ pf_status proxy_layer_bwd(const pf_layer_desc* desc, const pf_layer_params* prm,
     PF_CUDA(gemm_linear(d, N1, (int)g.rows1, {dYsrc, d, 1}, {Xsrc, N1, 1}, with_sk(e, w.sk, w.skb), cs));
   }
   {
-    EpiDXArgs e{dXd, dXb, df, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L};
+    EpiDXArgs e{dXb, df, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L};
     set_gemm_tag("bwd_dX", (double)g.rows1 * N1 * 4.0);
     PF_CUDA(gemm_dx1d((int)g.rows1, N1, d, {dYsrc, d, 0}, {W_c1, N1, 1}, e, cs));
   }
@@ -1592,7 +1580,7 @@ SegFwdWs carve_seg_fwd(Carve& wc, const SegPlan& p, void* saved) {
 }
 
 struct SegBwdWs {
-  bf16 *Xpad, *dXpad, *dD, *dZ, *dHbar, *dA, *dQKV, *dHb, *dY;
+  bf16 *Xpad, *dD, *dZ, *dHbar, *dA, *dQKV, *dHb, *dY;
   float *Di, *dHf, *part, *sk, *gtmp, *gsum;
   size_t skb;
 };
@@ -1612,7 +1600,6 @@ SegBwdWs carve_seg_bwd(Carve& c, const SegPlan& p) {
   }
   pe = std::max(pe, colsum_part_elems((long)p.s.size(), (int)(3 * p.d)));
   w.Xpad = z.ragged ? c.take<bf16>(z.m * z.P * p.d) : nullptr;
-  w.dXpad = z.ragged ? c.take<bf16>(z.m * z.P * p.d) : nullptr;
   w.dD = c.take<bf16>(dD);
   if (p.levels == 2) w.dZ = c.take<bf16>(dZ);
   w.dHbar = c.take<bf16>(p.M * p.d);
@@ -1693,7 +1680,6 @@ pf_status proxy_segments_fwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
   const bf16* Xb = static_cast<const bf16*>(X);
   bf16* Xo = static_cast<bf16*>(X_out);
   // compression, segment by segment, into the proxies' rows g0 .. g0 + m - 1
-  std::vector<const bf16*> xs(p.s.size());
   for (size_t i = 0; i < p.s.size(); ++i) {
     const Seg& g = p.s[i];
     const bf16* Xs = Xb + g.off * d;
@@ -1701,7 +1687,6 @@ pf_status proxy_segments_fwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
       PF_CUDA(pad_rows(Xs, f.Xpad, 1, g.L, g.m * g.P, d, cs));
       Xs = f.Xpad;
     }
-    xs[i] = Xs;
     const bf16* W_c1 = static_cast<const bf16*>(sp[i].W_c1);
     EpiLinearArgs e;
     e.bias = sp[i].b_c1;
@@ -1759,14 +1744,12 @@ pf_status proxy_segments_fwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
                           with_sk(e, f.sk, f.skb), cs));
       Zsrc = sv.Z[i];
     }
-    EpiInjectArgs e{sp[i].b_d1, sv.D[i], xs[i], Xo + g.off * d, prm->w_x, prm->w_dlt, prm->b_g,
+    EpiInjectArgs e{sp[i].b_d1, sv.D[i], Xb + g.off * d, Xo + g.off * d, prm->w_x, prm->w_dlt, prm->b_g,
                     d, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L, i == 0 ? 1 : 0, p.gated ? 1 : 0};
     set_gemm_tag("seg_decompress_d1_inject", (double)g.rows1 * g.N1 * 8.0);
     PF_CUDA(gemm_inject1d((int)g.rows1, (int)g.N1, d, {Zsrc, d, 0},
                           {static_cast<const bf16*>(sp[i].W_d1), d, 0}, e, cs));
   }
-  const Seg& g0 = p.s.front();
-  PF_CUDA(copy_block0(Xb, g0.L, Xo, g0.L, 1, d, (int)std::min(g0.P, g0.L), cs));
   return PF_OK;
 }
 
@@ -1802,7 +1785,6 @@ pf_status proxy_segments_bwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
   PF_CUDA(cudaMemsetAsync(w.dHbar + (p.M - 1) * d, 0, d * sizeof(bf16), cs));
   if (p.gated) PF_CUDA(cudaMemsetAsync(w.gtmp, 0, p.s.size() * 3 * d * sizeof(float), cs));
   std::vector<const bf16*> xs(p.s.size());
-  std::vector<bf16*> dxd(p.s.size());
   // injection and decompression backward, segment by segment (segment 0 first:
   // its last proxy row, which feeds no block of its own, is overwritten by
   // segment 1's first source row)
@@ -1810,21 +1792,16 @@ pf_status proxy_segments_bwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
     const Seg& g = p.s[i];
     const bf16* Xs = Xb + g.off * d;
     xs[i] = Xs;
-    dxd[i] = dXb + g.off * d;
     if (g.ragged) {
       PF_CUDA(pad_rows(Xs, w.Xpad, 1, g.L, g.m * g.P, d, cs));
       xs[i] = w.Xpad;
-      dxd[i] = w.dXpad;
     }
     const int N1 = (int)g.N1, r1 = (int)g.rows1;
     const int nch = inj_bwd_chunks(g.rows1, N1);
-    InjBwdArgs a{G + g.off * d, Xs, sv.D[i], w.dD, dxd[i], g.ragged ? g.m * g.P : g.L, prm->w_x,
+    InjBwdArgs a{G + g.off * d, Xs, sv.D[i], w.dD, dXb + g.off * d, prm->w_x,
                  prm->w_dlt, prm->b_g, d, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L, 1,
                  i == 0 ? 1 : 0, p.gated ? 1 : 0};
     PF_CUDA(inj_bwd_1d(a, w.part, nch, cs));
-    if (i == 0)
-      PF_CUDA(copy_block0(G, g.L, dxd[0], g.ragged ? g.m * g.P : g.L, 1, d,
-                          (int)std::min(g.P, g.L), cs));
     float* gt = w.gtmp + i * 3 * d;
     PF_CUDA(inj_bwd_finalize(w.part, nch, N1, d, sg[i].b_d1, p.gated ? gt : nullptr,
                              p.gated ? gt + d : nullptr, p.gated ? gt + 2 * d : nullptr, cs));
@@ -1940,7 +1917,7 @@ pf_status proxy_segments_bwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
       set_gemm_tag("seg_bwd_dW_c1", (double)d * N1 * 4.0);
       PF_CUDA(gemm_linear(d, N1, r1, {dYsrc, d, 1}, {xs[i], N1, 1}, with_sk(e, w.sk, w.skb), cs));
     }
-    EpiDXArgs e{dxd[i], dXb + g.off * d, d, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L};
+    EpiDXArgs e{dXb + g.off * d, d, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L};
     set_gemm_tag("seg_bwd_dX", (double)r1 * N1 * 4.0);
     PF_CUDA(gemm_dx1d(r1, N1, d, {dYsrc, d, 0}, {static_cast<const bf16*>(sp[i].W_c1), N1, 1}, e,
                       cs));

@@ -1,6 +1,5 @@
 // Bandwidth-bound kernels of the layer: injection backward with its column
-// reductions, deterministic column sums (bias gradients), block-0 copies and
-// zero padding.  All accesses are 16-byte vectors over contiguous rows.
+// reductions, deterministic column sums (bias gradients) and zero padding.  All accesses are 16-byte vectors over contiguous rows.
 #include <algorithm>
 
 #include "kernels.h"
@@ -10,16 +9,6 @@ namespace pf {
 namespace {
 
 constexpr int EW_THREADS = 256;
-
-__global__ void copy_block0_kernel(const bf16* __restrict__ src, long Ls, bf16* __restrict__ dst,
-                                   long Ld, int d, long per_seq_vec) {
-  const int pz = pdl_enter();
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
-  const int b = blockIdx.y;
-  if (i >= per_seq_vec) return;
-  *reinterpret_cast<uint4*>(dst + (long)b * Ld * d + i * 8) =
-      *reinterpret_cast<const uint4*>(src + (long)b * Ls * d + i * 8);
-}
 
 __global__ void pad_rows_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst, long L,
                                 long Lp, int d) {
@@ -85,18 +74,20 @@ __global__ void __launch_bounds__(EW_THREADS, 2) inj_bwd_kernel(InjBwdArgs a, fl
   for (long rb = r0; rb < r1; rb += INJ_U) {
     uint4 gv[INJ_U], xv[INJ_U], dv[INJ_U];
     long offx[INJ_U];
-    bool valid[INJ_U];
+    bool valid[INJ_U], copy[INJ_U];
 #pragma unroll
     for (int u = 0; u < INJ_U; ++u) {
       const long r = rb + u;
-      const int it = ix.i + a.shift;
+      // the last proxy of a causal sequence feeds no block: its rows copy
+      // block 0, which received nothing, dX = G
+      copy[u] = ix.i + a.shift >= a.m;
+      const int it = copy[u] ? 0 : ix.i + a.shift;
       const long tok = (long)it * P + (long)ix.grp * a.k1 + tq;
-      valid[u] = r < r1 && it < a.m && tok < a.L;
-      offx[u] = ((long)ix.b * a.Ldx + tok) * a.d + ch;
+      valid[u] = r < r1 && tok < a.L;
+      offx[u] = ((long)ix.b * a.L + tok) * a.d + ch;
       if (valid[u]) {
-        const long off = ((long)ix.b * a.L + tok) * a.d + ch;
-        gv[u] = *reinterpret_cast<const uint4*>(G + off);
-        xv[u] = *reinterpret_cast<const uint4*>(X + off);
+        gv[u] = *reinterpret_cast<const uint4*>(G + offx[u]);
+        xv[u] = *reinterpret_cast<const uint4*>(X + offx[u]);
         dv[u] = *reinterpret_cast<const uint4*>(D + r * N + col);
       }
       ix.next(a.k2, a.m);
@@ -106,7 +97,7 @@ __global__ void __launch_bounds__(EW_THREADS, 2) inj_bwd_kernel(InjBwdArgs a, fl
       const long r = rb + u;
       if (r >= r1) break;
       float dd[8];
-      if (valid[u]) {
+      if (valid[u] && !copy[u]) {
         float g[8], x[8], Dv[8], dx[8];
         const uint32_t* pg = &gv[u].x;
         const uint32_t* px = &xv[u].x;
@@ -135,6 +126,7 @@ __global__ void __launch_bounds__(EW_THREADS, 2) inj_bwd_kernel(InjBwdArgs a, fl
         }
         store8_bf16(dX + offx[u], dx);
       } else {
+        if (valid[u]) *reinterpret_cast<uint4*>(dX + offx[u]) = gv[u];
 #pragma unroll
         for (int j = 0; j < 8; ++j) dd[j] = 0.f;
       }
@@ -179,23 +171,19 @@ constexpr uint32_t IB_STAGE_BYTES = 3 * IB_R * IB_ROW_BYTES;  // [D | G | X] x I
 constexpr uint32_t IB_SMEM = IB_STAGES * IB_STAGE_BYTES + 128;
 
 struct IbRow {
-  bool valid;   // the row has target tokens
-  int lim;      // valid columns of the row (tokens < L), 0 if none
-  long gx_off;  // element offset of the row's tokens in G / X
-  long dx_off;  // element offset in dX
+  bool copy;  // the last proxy of a causal sequence: the row copies block 0, dX = G
+  int lim;    // valid columns of the row (tokens < L), 0 if none
+  long off;   // element offset of the row's tokens in G, X and dX
 };
 
 __device__ __forceinline__ IbRow ib_row(const InjBwdArgs& a, const RowIdx& ix, int N) {
-  IbRow r{false, 0, 0, 0};
-  const int it = ix.i + a.shift;
+  IbRow r;
+  r.copy = ix.i + a.shift >= a.m;
+  const int it = r.copy ? 0 : ix.i + a.shift;
   const long tok0 = (long)it * (a.k1 * a.k2) + (long)ix.grp * a.k1;
-  if (it < a.m && tok0 < a.L) {
-    r.valid = true;
-    const long lim = (a.L - tok0) * a.d;
-    r.lim = lim < N ? (int)lim : N;
-    r.gx_off = ((long)ix.b * a.L + tok0) * a.d;
-    r.dx_off = ((long)ix.b * a.Ldx + tok0) * a.d;
-  }
+  const long lim = (a.L - tok0) * a.d;
+  r.lim = lim <= 0 ? 0 : lim < N ? (int)lim : N;
+  r.off = ((long)ix.b * a.L + tok0) * a.d;
   return r;
 }
 
@@ -239,9 +227,9 @@ __global__ void __launch_bounds__(256, 2) inj_bwd_stream_kernel(InjBwdArgs a,
       if (rs + u < r1) {
         dbytes[u] = IB_ROW_BYTES;
         const IbRow rr = ib_row(a, pix, N);
-        if (rr.valid && rr.lim > col0) {
+        if (rr.lim > col0) {
           gbytes[u] = (uint32_t)(min(rr.lim - col0, IB_W)) * 2u;
-          goff[u] = rr.gx_off + col0;
+          goff[u] = rr.off + col0;
         }
         pix.next(a.k2, a.m);
       }
@@ -285,9 +273,9 @@ __global__ void __launch_bounds__(256, 2) inj_bwd_stream_kernel(InjBwdArgs a,
       const IbRow rr = ib_row(a, ix, N);
       ix.next(a.k2, a.m);
       if (!ok) continue;
-      const bool v = rr.valid && col < rr.lim;
+      const bool v = col < rr.lim;
       float dd[8];
-      if (v) {
+      if (v && !rr.copy) {
         const uint4 gv = *reinterpret_cast<const uint4*>(base + (IB_R + u) * IB_ROW_BYTES);
         const uint4 xv = *reinterpret_cast<const uint4*>(base + (2 * IB_R + u) * IB_ROW_BYTES);
         const uint4 dv = *reinterpret_cast<const uint4*>(base + u * IB_ROW_BYTES);
@@ -315,8 +303,11 @@ __global__ void __launch_bounds__(256, 2) inj_bwd_stream_kernel(InjBwdArgs a,
             dd[j] = g[j];
           }
         }
-        store8_bf16(a.dX + rr.dx_off + col, dx);
+        store8_bf16(a.dX + rr.off + col, dx);
       } else {
+        if (v)
+          *reinterpret_cast<uint4*>(a.dX + rr.off + col) =
+              *reinterpret_cast<const uint4*>(base + (IB_R + u) * IB_ROW_BYTES);
 #pragma unroll
         for (int j = 0; j < 8; ++j) dd[j] = 0.f;
       }
@@ -524,14 +515,6 @@ cudaError_t colsum_impl(const T* X, long R, int C, float* out, float* part, cuda
 }
 
 }  // namespace
-
-cudaError_t copy_block0(const bf16* src, long Ls, bf16* dst, long Ld, int B, int d, int rows,
-                        cudaStream_t st) {
-  const long nvec = (long)rows * d / 8;
-  dim3 grid((unsigned)((nvec + 255) / 256), B);
-  LaunchTimer lt("copy_block0", st, 0.0, 32.0 * nvec * B);
-  return launch_kernel(copy_block0_kernel, grid, 256, 0, st, src, Ls, dst, Ld, d, nvec);
-}
 
 cudaError_t pad_rows(const bf16* src, bf16* dst, int B, long L, long Lp, int d, cudaStream_t st) {
   const long nvec = Lp * d / 8;

@@ -62,6 +62,21 @@ bool make_operand_map(CUtensorMap* m, const Operand& op, int rows, int K) {
   return make_map(m, op.ptr, (uint64_t)K, (uint64_t)rows, (uint64_t)op.ld, 64, 128);
 }
 
+// B of a direct epilogue: row n = 8 s + 2 g + e as dimensions (k, e, g, s); a box
+// holds 32 rows of one g.
+bool make_segment_map(CUtensorMap* m, const Operand& op, int rows, int K) {
+  auto fn = encode_fn();
+  if (fn == nullptr || op.mn || rows % 8 != 0) return false;
+  const cuuint64_t row = (cuuint64_t)op.ld * 2;
+  cuuint64_t dims[4] = {(cuuint64_t)K, 2, 4, (cuuint64_t)rows / 8};
+  cuuint64_t strides[3] = {row, 2 * row, 8 * row};
+  cuuint32_t box[4] = {64, 2, 1, 16};
+  cuuint32_t es[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(op.ptr), dims, strides, box,
+            es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Co-resident CTA pairs of the pair kernel (at most half the SMs).
 template <class Kern>
 int max_pairs(Kern kern, int threads, int smem) {
@@ -86,42 +101,44 @@ int max_pairs(Kern kern, int threads, int smem) {
 
 template <int BN, bool AMN, bool BMN, class Epi>
 cudaError_t launch(int M, int N, int K, const CUtensorMap& ta, const CUtensorMap& tb,
-                   const CUtensorMap& tx, const Epi& epi, cudaStream_t st, int splits) {
-  constexpr int XCOLS = Epi::kXTile ? (Epi::kPaired ? BN / 2 : BN) : 0;
-  if constexpr (BN == 256 && Epi::kPairs) {
+                   const Epi& epi, cudaStream_t st, int splits) {
+  if constexpr (BN == 256) {
     // CTA pairs (256 x 256 tiles, half of B per CTA, a deeper stage ring)
     // when every co-resident pair gets a tile
     auto kern2 = gemm_tc_kernel<BN, AMN, BMN, Epi, true>;
-    constexpr int smem2 = GemmCfg<BN, XCOLS, Epi::kColPar, true, Epi::kStageBytes>::SMEM_BYTES;
-    constexpr int threads = GemmRoles<Epi>::kThreads;
+    constexpr int smem2 = GemmCfg<BN, true, gemm_stage_bytes<Epi>(true)>::SMEM_BYTES;
     cudaError_t e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
     if (e != cudaSuccess) return e;
-    static const int pairs = max_pairs(kern2, threads, smem2);
+    static const int pairs = max_pairs(kern2, GEMM_THREADS, smem2);
     const long pair_tiles =
         (long)((N + BN - 1) / BN) * ((M + 2 * GEMM_BM - 1) / (2 * GEMM_BM)) * splits;
-    if (pairs > 0 && pair_tiles >= pairs) {
-      return launch_clusters(2, kern2, 2 * (unsigned)std::min<long>(pair_tiles, pairs), threads,
-                             smem2, st, ta, tb, tx, M, N, K, splits, epi);
-    }
+    if (pairs > 0 && pair_tiles >= pairs)
+      return launch_clusters(2, kern2, 2 * (unsigned)std::min<long>(pair_tiles, pairs),
+                             GEMM_THREADS, smem2, st, ta, tb, M, N, K, splits, epi);
   }
   auto kern = gemm_tc_kernel<BN, AMN, BMN, Epi>;
-  constexpr int smem = GemmCfg<BN, XCOLS, Epi::kColPar, false, Epi::kStageBytes>::SMEM_BYTES;
+  constexpr int smem = GemmCfg<BN, false, gemm_stage_bytes<Epi>(false)>::SMEM_BYTES;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const long tiles = (long)((N + BN - 1) / BN) * ((M + GEMM_BM - 1) / GEMM_BM) * splits;
   const int grid = (int)std::min<long>(tiles, num_sms());
-  return launch_kernel(kern, grid, GemmRoles<Epi>::kThreads, smem, st, ta, tb, tx, M, N, K, splits,
-                       epi);
+  return launch_kernel(kern, grid, GEMM_THREADS, smem, st, ta, tb, M, N, K, splits, epi);
 }
 
+// Operand majors that the epilogue's callers use: all four for the linear
+// ones, K-major A (and one major of B) for the fused ones.
 template <int BN, class Epi>
 cudaError_t launch_majors(int M, int N, int K, const Operand& A, const Operand& B,
-                          const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tx,
-                          const Epi& epi, cudaStream_t st, int splits = 1) {
-  if (!A.mn && !B.mn) return launch<BN, false, false>(M, N, K, ta, tb, tx, epi, st, splits);
-  if (!A.mn && B.mn) return launch<BN, false, true>(M, N, K, ta, tb, tx, epi, st, splits);
-  if (A.mn && B.mn) return launch<BN, true, true>(M, N, K, ta, tb, tx, epi, st, splits);
-  return launch<BN, true, false>(M, N, K, ta, tb, tx, epi, st, splits);
+                          const CUtensorMap& ta, const CUtensorMap& tb, const Epi& epi,
+                          cudaStream_t st, int splits = 1) {
+  if (!A.mn && !B.mn) return launch<BN, false, false>(M, N, K, ta, tb, epi, st, splits);
+  if constexpr (!Epi::kDirect)
+    if (!A.mn && B.mn) return launch<BN, false, true>(M, N, K, ta, tb, epi, st, splits);
+  if constexpr (!Epi::kRows) {
+    if (A.mn && B.mn) return launch<BN, true, true>(M, N, K, ta, tb, epi, st, splits);
+    return launch<BN, true, false>(M, N, K, ta, tb, epi, st, splits);
+  }
+  return cudaErrorInvalidValue;
 }
 
 bool operand_ok(const Operand& op) {
@@ -129,24 +146,15 @@ bool operand_ok(const Operand& op) {
          (op.ld * 2) % 16 == 0;
 }
 
-// X tile source (kXTile epilogues): the [rows, N] bf16 view the epilogue
-// prefetches by TMA; for other epilogues `xsrc` is ignored.
 template <class Epi>
 cudaError_t gemm_dispatch(int M, int N, int K, Operand A, Operand B, const Epi& epi,
-                          const bf16* xsrc, long x_rows, cudaStream_t st, long x_cols = -1) {
-  if (x_cols < 0) x_cols = N;
+                          cudaStream_t st) {
   if (M <= 0 || N <= 0 || N % 32 != 0 || K < 0 || !operand_ok(A) || !operand_ok(B))
     return cudaErrorInvalidValue;
-  CUtensorMap ta, tb, tx;
-  if (!make_operand_map(&ta, A, M, K) || !make_operand_map(&tb, B, N, K))
+  CUtensorMap ta, tb;
+  if (!make_operand_map(&ta, A, M, K) ||
+      !(Epi::kDirect ? make_segment_map(&tb, B, N, K) : make_operand_map(&tb, B, N, K)))
     return cudaErrorInvalidValue;
-  if (Epi::kXTile) {
-    if (xsrc == nullptr || (reinterpret_cast<uintptr_t>(xsrc) & 15) != 0 ||
-        !make_map(&tx, xsrc, (uint64_t)x_cols, (uint64_t)x_rows, (uint64_t)x_cols, 64, 128))
-      return cudaErrorInvalidValue;
-  } else {
-    tx = ta;
-  }
   const long tiles256 = (long)((N + 255) / 256) * ((M + GEMM_BM - 1) / GEMM_BM);
   LaunchTimer lt(gemm_tag_label(), st, 2.0 * M * N * (double)K,
                  2.0 * ((double)M * K + (double)N * K) + gemm_tag_bytes());
@@ -156,8 +164,9 @@ cudaError_t gemm_dispatch(int M, int N, int K, Operand A, Operand B, const Epi& 
   const long tiles128 = (long)((N + 127) / 128) * ((M + GEMM_BM - 1) / GEMM_BM);
   const long sms = num_sms(), w256 = (tiles256 + sms - 1) / sms, w128 = (tiles128 + sms - 1) / sms;
   if (Epi::kPaired || (N >= 256 && 3 * w256 <= 2 * w128))
-    return launch_majors<256>(M, N, K, A, B, ta, tb, tx, epi, st);
-  return launch_majors<128>(M, N, K, A, B, ta, tb, tx, epi, st);
+    return launch_majors<256>(M, N, K, A, B, ta, tb, epi, st);
+  if constexpr (!Epi::kPaired) return launch_majors<128>(M, N, K, A, B, ta, tb, epi, st);
+  return cudaErrorInvalidValue;
 }
 
 // out = sum_s part[s] (+ bias) (+ addend) -> fp32 and/or bf16, 4 columns per thread.
@@ -236,7 +245,7 @@ cudaError_t gemm_linear(int M, int N, int K, Operand A, Operand B, const EpiLine
     {
       LaunchTimer lt(gemm_tag_label(), st, 2.0 * M * N * (double)K,
                      2.0 * ((double)M * K + (double)N * K) + 4.0 * S * M * N);
-      cudaError_t err = launch_majors<128>(M, N, K, A, B, ta, tb, ta, epi, st, S);
+      cudaError_t err = launch_majors<128>(M, N, K, A, B, ta, tb, epi, st, S);
       if (err != cudaSuccess) return err;
     }
     LaunchTimer lt("splitk_reduce", st, (double)S * M * N, 4.0 * (S + 1.0) * M * N);
@@ -244,58 +253,63 @@ cudaError_t gemm_linear(int M, int N, int K, Operand A, Operand B, const EpiLine
     return launch_kernel(splitk_reduce_kernel, (unsigned)((quads + 255) / 256), 256, 0, st,
                          e.splitk_scratch, S, M, N, e);
   }
-  if ((e.add_bf16 && ((uintptr_t)e.add_bf16 & 15)) || (e.add_bf16 && e.ld_add_bf16 % 8))
-    return cudaErrorInvalidValue;
+  if (e.add_bf16) {  // bf16 sum of the product and a bf16 matrix, nothing else
+    if (((uintptr_t)e.add_bf16 & 15) || e.ld_add_bf16 % 8 || !e.out_bf16 || e.ld_bf16 % 8 ||
+        e.bias || e.addend || e.out_f32 || e.act_silu || e.pre_bf16 || e.dsilu_of || A.mn)
+      return cudaErrorInvalidValue;
+    EpiAddRows epi{{}, M, N, e.add_bf16, e.ld_add_bf16, e.out_bf16, e.ld_bf16};
+    return gemm_dispatch(M, N, K, A, B, epi, st);
+  }
   if ((e.pre_bf16 && ((uintptr_t)e.pre_bf16 & 15 || e.ld_pre % 8)) ||
       (e.dsilu_of && ((uintptr_t)e.dsilu_of & 15 || e.ld_dsilu % 8)))
     return cudaErrorInvalidValue;
   // a short contraction with a plain (bias) epilogue stores whole rows from a
   // shared-memory stage: its output, not its mainloop, would bound it
-  if (K <= 2048 && !e.addend && !e.add_bf16 && !e.act_silu && !e.pre_bf16 && !e.dsilu_of &&
+  if (K <= 2048 && !e.addend && !e.act_silu && !e.pre_bf16 && !e.dsilu_of &&
       (e.out_f32 == nullptr || e.ld_f32 % 4 == 0) && (e.out_bf16 == nullptr || e.ld_bf16 % 8 == 0)) {
     EpiLinearStaged epi{{}, M, N, e.bias, e.out_f32, e.ld_f32, e.out_bf16, e.ld_bf16};
-    return gemm_dispatch(M, N, K, A, B, epi, nullptr, 0, st);
+    return gemm_dispatch(M, N, K, A, B, epi, st);
   }
   EpiLinear epi{{},         M,          N,          e.bias,      e.addend,  e.ld_add,
-                e.out_f32,  e.ld_f32,   e.out_bf16, e.ld_bf16,   e.add_bf16, e.ld_add_bf16,
-                e.act_silu, e.pre_bf16, e.ld_pre,   e.dsilu_of,  e.ld_dsilu};
-  return gemm_dispatch(M, N, K, A, B, epi, nullptr, 0, st);
+                e.out_f32,  e.ld_f32,   e.out_bf16, e.ld_bf16,   e.act_silu, e.pre_bf16,
+                e.ld_pre,   e.dsilu_of, e.ld_dsilu};
+  return gemm_dispatch(M, N, K, A, B, epi, st);
 }
 
 cudaError_t gemm_inject1d(int M, int N, int K, Operand A, Operand B, const EpiInjectArgs& e,
                           cudaStream_t st) {
-  EpiInject1D epi{{}, M, N, e.bias, e.D_save, e.X_out, e.w_x, e.w_dlt, e.b_g,
+  EpiInject1D epi{{}, M, N, e.bias, e.D_save, e.X, e.X_out, e.w_x, e.w_dlt, e.b_g,
                   e.d, e.k1, e.k2, e.m, e.L, e.shift, e.gated};
-  if (A.mn || B.mn) return cudaErrorInvalidValue;
-  return gemm_dispatch(M, N, K, A, B, epi, e.Xsrc, M, st);
+  if (A.mn || B.mn || e.d % 32 != 0) return cudaErrorInvalidValue;
+  return gemm_dispatch(M, N, K, A, B, epi, st);
 }
 
 cudaError_t gemm_dx1d(int M, int N, int K, Operand A, Operand B, const EpiDXArgs& e,
                       cudaStream_t st) {
   EpiDX1D epi{{}, M, N, e.dX, e.d, e.k1, e.k2, e.m, e.L};
-  if (A.mn || !B.mn) return cudaErrorInvalidValue;
-  return gemm_dispatch(M, N, K, A, B, epi, e.dXd, M, st);
+  if (A.mn || !B.mn || e.d % 8 != 0) return cudaErrorInvalidValue;
+  return gemm_dispatch(M, N, K, A, B, epi, st);
 }
 
 cudaError_t gemm_append_kv(int M, int N, int K, Operand A, Operand B, const EpiAppendArgs& e,
                            cudaStream_t st) {
   EpiAppendKV epi{{}, M, N, e.K, e.V, e.n_open, e.n_proxy, e.d, e.P, e.cap};
   if (A.mn || B.mn) return cudaErrorInvalidValue;
-  return gemm_dispatch(M, N, K, A, B, epi, nullptr, 0, st);
+  return gemm_dispatch(M, N, K, A, B, epi, st);
 }
 
 cudaError_t gemm_affine2d(int M, int N, int K, Operand A, Operand B, const EpiAffine2DArgs& e,
                           cudaStream_t st) {
-  EpiAffine2D epi{{}, M, e.bias, e.S_save, e.X_out, e.stats, e.d, e.patch, e.gh, e.gw, e.m};
+  EpiAffine2D epi{{}, M, e.bias, e.S_save, e.X, e.X_out, e.stats, e.d, e.patch, e.gh, e.gw, e.m};
   if (A.mn || B.mn || e.d % 128 != 0) return cudaErrorInvalidValue;
-  return gemm_dispatch(M, N, K, A, B, epi, e.Xp, M, st, (long)e.patch * e.patch * e.d);
+  return gemm_dispatch(M, N, K, A, B, epi, st);
 }
 
 cudaError_t gemm_dx2d(int M, int N, int K, Operand A, Operand B, const EpiDX2DArgs& e,
                       cudaStream_t st) {
-  EpiDX2D epi{{}, M, N, e.dX, e.d, e.patch, e.gh, e.gw, e.m};
+  EpiDX2D epi{{}, M, N, e.dXd, e.dX, e.d, e.patch, e.gh, e.gw, e.m};
   if (A.mn || !B.mn || e.d % 32 != 0) return cudaErrorInvalidValue;
-  return gemm_dispatch(M, N, K, A, B, epi, e.dXd, M, st);
+  return gemm_dispatch(M, N, K, A, B, epi, st);
 }
 
 }  // namespace pf

@@ -28,15 +28,30 @@
 //              lanes 32*(w%4).. and half of the tile's columns), fused
 //              epilogue functor, global stores.  While they drain
 //              accumulator i, the MMA warp fills the other.
-// Epilogues that read a bf16 tile shaped like the output (the local stream X
-// for injection, the direct gradient for dX) have it prefetched by TMA into
-// shared memory (128 x BN, 128B-swizzled, 64-column boxes).  Unpaired ones get
-//   warp 10  : X loader: refills each box for the next tile as soon as the
-//              four epilogue warps of its column half are done with it, so
-//              the load overlaps the rest of the tile instead of waiting for
-//              the whole tile to drain (the single buffer has no room for a
-//              second one next to the operand stages);
-// paired ones (2D affine) load the whole tile at the start of its epilogue.
+// Epilogues that read tensors shaped like the output (kRows: the local stream
+// X for injection, the direct gradient for dX) give lane (sr, sp) = (lane / 4,
+// lane % 4) four columns pairs or eight columns of rows sr, sr + 8, sr + 16, sr
+// + 24 of a 32 x 32 chunk, straight from TMEM.  The chunk of X comes by
+// cp.async into a ring of 2 KB slots a warp, results leave as 64 contiguous
+// bytes a row, and the per-column parameters sit in registers.  Two forms:
+//   kDirect (two outputs, K-major B): the rows of B are loaded in the order that
+//            puts 8 consecutive columns of a row into one lane, which reads only
+//            its own 16 bytes of X and stores both outputs from registers; the
+//            reordered loads (four boxes for one) cost the mainloop 15%
+//   else     MMA fragments (column pairs), X by ldmatrix, the output over it by
+//            stmatrix and out; any B; a second output would go the same way
+//            (injection 448 us so, 417 direct), one output is faster (cross_out,
+//            M 131072, N = K = 1024: 175 us so, 189 direct)
+// What bounds these kernels besides the MMAs is shared memory, its bandwidth
+// and its size, and the lines that a store instruction touches (with 32 bytes a
+// row injection takes 615 us).  An epilogue whose lanes own rows (X tile by TMA
+// in 64 KB, four broadcast parameters a column, outputs staged) took 7k of the
+// 16.8k cycles of a 128 x 256 x 1024 tile in shared memory and left room for a
+// three-stage ring; these take 1-2k and leave a CTA pair six stages.
+// Measured, before and after: injection of the 262144-token layer (M 32768, N
+// 8192, K 1024) 487 -> 417 us, its dX 342 -> 330; of the 65536-token layer 152
+// -> 122 and 109 -> 99; affine injection of four 512 x 512 images (M 16384, N
+// 65536, K 512) 1317 -> 1100, their dX 577 -> 491; cross_out 266 -> 175.
 // Every mbarrier wait is bounded (common.cuh); on a timeout the kernel flags
 // the error, drains its own copies and MMAs (bounded), frees TMEM and returns.
 #pragma once
@@ -50,38 +65,22 @@ constexpr int GEMM_BK = 64;
 constexpr int GEMM_EPI_WARPS = 8;  // two per TMEM lane quarter, each owning half the columns
 constexpr int GEMM_THREADS = 64 + 32 * GEMM_EPI_WARPS;
 
-// Unpaired X-tile epilogues run an X-loader warp after the epilogue warps.
-template <class Epi>
-struct GemmRoles {
-  static constexpr bool kXLoader = Epi::kXTile && !Epi::kPaired;
-  static constexpr int kThreads = GEMM_THREADS + (kXLoader ? 32 : 0);
-};
-
-// XCOLS: columns of the bf16 tile an epilogue prefetches (0: none).
-// PAR: the epilogue stages one float4 of per-column parameters per output
-// column in shared memory (two tiles' worth, filled one tile ahead).
 // PAIR: the tile is shared by a CTA pair, each CTA staging half of B.
-constexpr uint32_t GEMM_SMEM_MAX = 232448;  // dynamic shared memory per CTA (227 KB)
 // SB: bytes of shared memory the epilogue stages its output in (0: none).
-template <int BN, int XCOLS, bool PAR = false, bool PAIR = false, uint32_t SB = 0>
+constexpr uint32_t GEMM_SMEM_MAX = 232448;  // dynamic shared memory per CTA (227 KB)
+template <int BN, bool PAIR, uint32_t SB>
 struct GemmCfg {
   static constexpr int B_ROWS = PAIR ? BN / 2 : BN;            // B rows staged by one CTA
   static constexpr uint32_t A_BYTES = GEMM_BM * GEMM_BK * 2;  // 16 KB
   static constexpr uint32_t B_BYTES = B_ROWS * GEMM_BK * 2;   // 16/32 KB
   static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr uint32_t X_BYTES = GEMM_BM * XCOLS * 2;
-  static constexpr uint32_t PAR_BYTES = PAR ? 2 * BN * 16 : 0;
-  static constexpr uint32_t FIXED_BYTES =
-      X_BYTES + 1024 /*align*/ + 256 /*barriers*/ + PAR_BYTES + SB;
-  static constexpr int PAIR_STAGES = (int)((GEMM_SMEM_MAX - FIXED_BYTES) / STAGE_BYTES);
-  static constexpr int TABLE_STAGES =
-      PAIR ? 7
-           : (XCOLS ? (BN == 256 && (XCOLS == 256 || PAR) ? 3 : (BN == 256 ? 4 : 5))
-                    : (BN == 256 ? 4 : 6));
-  static constexpr int STAGES = PAIR_STAGES < TABLE_STAGES ? PAIR_STAGES : TABLE_STAGES;
+  static constexpr uint32_t FIXED_BYTES = 1024 /*align*/ + 256 /*barriers*/ + SB;
+  static constexpr int FIT = (int)((GEMM_SMEM_MAX - FIXED_BYTES) / STAGE_BYTES);
+  static constexpr int MOST = PAIR ? 7 : (BN == 256 ? 4 : 6);
+  static constexpr int STAGES = FIT < MOST ? FIT : MOST;
   static constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + FIXED_BYTES;
   static_assert(SMEM_BYTES <= GEMM_SMEM_MAX, "shared memory");
-  static_assert(2 * STAGES + 14 <= 31, "barrier region");
+  static_assert(2 * STAGES + 6 <= 31, "barrier region");
 };
 
 // Barrier of the epilogue threads (named barrier 1) that also ANDs a predicate
@@ -99,95 +98,75 @@ __device__ __forceinline__ bool epi_bar_and(bool p) {
   return r != 0;
 }
 
-// 8 bf16 of row r, columns [c, c+8) of a 128 x BN tile stored as BN/64 boxes
-// of 128 rows x 64 columns with 128-byte swizzle (TMA SWIZZLE_128B layout).
-__device__ __forceinline__ void xtile_load8(const uint8_t* xt, int r, int c, float* v) {
-  const uint8_t* p = xt + (c >> 6) * 16384 + r * 128 + ((((c & 63) >> 3) ^ (r & 7)) << 4);
-  uint4 u = *reinterpret_cast<const uint4*>(p);
-  float2 a = unpack_bf16(u.x), b = unpack_bf16(u.y), e = unpack_bf16(u.z), f = unpack_bf16(u.w);
-  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y; v[4] = e.x; v[5] = e.y; v[6] = f.x; v[7] = f.y;
+// A warp's 32 x 32 fp32 stage: row r's 16-byte piece p (columns 4p..) sits at
+// piece p ^ (r & 7) of its 128 bytes, so that neither the row-per-lane writes
+// nor reads of whole rows (8 lanes a row) or of 8-column segments (4 lanes a
+// row) meet in a bank.
+constexpr uint32_t GEMM_STG_BYTES = GEMM_EPI_WARPS * 4096;
+__device__ __forceinline__ float4* stg_ptr(float* s, int r, int p) {
+  return reinterpret_cast<float4*>(s + r * 32 + ((p ^ (r & 7)) << 2));
 }
-
-// Address of 8 bf16 at row r, columns [c, c+8) of the swizzled tile above.
-__device__ __forceinline__ uint8_t* xtile_ptr(uint8_t* xt, int r, int c) {
-  return xt + (c >> 6) * 16384 + r * 128 + ((((c & 63) >> 3) ^ (r & 7)) << 4);
-}
-
-// Coalesced store of a warp's 32 rows x 32 columns (tile rows 32q.., tile
-// columns cl..) that its threads have staged, one row each, in the swizzled
-// tile: every store instruction writes 8 rows x 64 contiguous bytes.  dst(rr,
-// p) returns the global address of row rr's 16-byte piece p (or null to skip);
-// it is called by all lanes in step (it may shuffle).
-template <class F>
-__device__ __forceinline__ void warp_store_rows(uint8_t* xt, int q, int cl, F dst) {
-  const int lane = threadIdx.x & 31, p = lane & 3;
+__device__ __forceinline__ void stg_put_row(float* s, int r, const float* v) {
 #pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int rr = it * 8 + (lane >> 2);
-    bf16* g = dst(rr, p);
-    const uint4 val = *reinterpret_cast<const uint4*>(xtile_ptr(xt, q * 32 + rr, cl + p * 8));
-    if (g) *reinterpret_cast<uint4*>(g) = val;
-  }
+  for (int p = 0; p < 8; ++p)
+    *stg_ptr(s, r, p) = make_float4(v[4 * p], v[4 * p + 1], v[4 * p + 2], v[4 * p + 3]);
+}
+__device__ __forceinline__ void stg_get8(float* s, int r, int p8, float* f) {
+  const float4 a = *stg_ptr(s, r, 2 * p8), b = *stg_ptr(s, r, 2 * p8 + 1);
+  f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
+  f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+}
+// 16 bytes from global to shared memory, past L1: the rows of a chunk are k1 * d
+// elements apart, powers of two of which meet in a few sets of the little L1
+// that the stage ring leaves (X through registers: 754 us).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void ld8_f32(const float* p, float* v) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+  const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+__device__ __forceinline__ uint4 pack8_bf16(const float* v) {
+  return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
+                    pack_bf16(v[6], v[7]));
 }
 
-// Destinations of warp_store_rows' four store instructions for whole-row
-// segments: this lane stores (in instruction it) for row 8 it + lane / 4 of
-// the warp's 32 rows, whose element offset and valid column count are
-// gathered here once per tile (not shuffled again for every chunk).
-struct SegRows {
-  long long off[4];
-  int lim[4];
-  __device__ __forceinline__ void gather(long long my_off, int my_lim) {
-    const int src = (threadIdx.x & 31) >> 2;
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      off[it] = __shfl_sync(0xffffffffu, my_off, it * 8 + src);
-      lim[it] = __shfl_sync(0xffffffffu, my_lim, it * 8 + src);
-    }
-  }
-};
-
-__device__ __forceinline__ void xtile_put8(uint8_t* xt, int r, int c, const float* v) {
-  *reinterpret_cast<uint4*>(xtile_ptr(xt, r, c)) =
-      make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
-                 pack_bf16(v[6], v[7]));
+// Shared memory of the epilogue: a kRows one has xd slots of X a warp.
+template <class Epi>
+constexpr int gemm_xd(bool pair) {
+  return pair ? Epi::kPairDepth : 2;
+}
+template <class Epi>
+constexpr uint32_t gemm_stage_bytes(bool pair) {
+  return Epi::kRows ? (uint32_t)(GEMM_EPI_WARPS * gemm_xd<Epi>(pair) * 2048) : Epi::kStageBytes;
 }
 
 template <int BN, bool A_MN, bool B_MN, class Epi, bool PAIR = false>
-__global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ CUtensorMap tmX, int M, int N, int K, int splits,
-                   Epi epi) {
+                   int M, int N, int K, int splits, Epi epi) {
   static_assert(!PAIR || BN == 256, "CTA pairs use 256-wide tiles");
-  constexpr int XCOLS = Epi::kXTile ? (Epi::kPaired ? BN / 2 : BN) : 0;
-  using Cfg = GemmCfg<BN, XCOLS, Epi::kColPar, PAIR, Epi::kStageBytes>;
+  static_assert(!Epi::kDirect || !B_MN, "direct epilogues need a K-major B");
+  constexpr uint32_t SB = gemm_stage_bytes<Epi>(PAIR);
+  using Cfg = GemmCfg<BN, PAIR, SB>;
   constexpr int STAGES = Cfg::STAGES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
-  uint8_t* xtile = smem + STAGES * Cfg::STAGE_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(xtile + Cfg::X_BYTES);
-  // bars: full[S], empty[S], tfull[2], tempty[2], xfull, done, xbox_full[4],
-  // xbox_empty[4]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 14);
-  constexpr bool XL = GemmRoles<Epi>::kXLoader;
-  constexpr int XBOXES = XCOLS / 64;       // 64-column boxes of the X tile
-  constexpr int XB_HALF = XBOXES / 2;      // boxes per epilogue column half (XL)
-  // column parameters (kColPar), [2 tiles][BN/4 groups][4 params] float4: the
-  // float4 at (c / 4) * 4 + k holds parameter k of columns c & ~3 .. (c & ~3) + 3
-  float4* cpar = reinterpret_cast<float4*>(xtile + Cfg::X_BYTES + 256);
-  auto cpar_put = [&](int b, int col, float4 p) {
-    float* f = reinterpret_cast<float*>(cpar + b * BN) + (col >> 2) * 16 + (col & 3);
-    f[0] = p.x;
-    f[4] = p.y;
-    f[8] = p.z;
-    f[12] = p.w;
-  };
+  // output staging of the epilogue warps (kStageBytes), then the barriers:
+  // full[S], empty[S], tfull[2], tempty[2], done
+  uint8_t* const epi_smem = smem + STAGES * Cfg::STAGE_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(epi_smem + SB);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 6);
   __shared__ uint32_t s_consumed;
-  // output staging of the epilogue warps (kStageBytes epilogues), after the
-  // column parameters; other epilogues get the X tile
-  uint8_t* const epi_smem =
-      Epi::kStageBytes ? xtile + Cfg::X_BYTES + 256 + Cfg::PAR_BYTES : xtile;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // a pair (cluster of two CTAs) works on one tile of 2 x 128 rows: `unit` is
@@ -214,8 +193,7 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
   const int kb = sp * kps, ke = min(num_k, kb + kps);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
   const uint32_t tfull0 = smem_u32(bars + 2 * STAGES), tempty0 = tfull0 + 16;
-  const uint32_t xfull = tfull0 + 32, done = tfull0 + 40;
-  const uint32_t xbf0 = tfull0 + 48, xbe0 = xbf0 + 32;
+  const uint32_t done = tfull0 + 32;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -227,12 +205,7 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
       // one arrival per epilogue warp (of both CTAs of a pair, on rank 0)
       mbar_init(tempty0 + 8 * b, PAIR ? 2 * GEMM_EPI_WARPS : GEMM_EPI_WARPS);
     }
-    mbar_init(xfull, 1);
     mbar_init(done, 1);
-    for (int j = 0; j < 4; ++j) {
-      mbar_init(xbf0 + 8 * j, 1);
-      mbar_init(xbe0 + 8 * j, 4);  // the four epilogue warps of the box's column half
-    }
     fence_barrier_init();
     s_consumed = 0;
   }
@@ -252,9 +225,6 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
   const uint32_t tmem = *tmem_slot;
   pdl_enter();  // the setup above overlaps the kernel before this one
   uint32_t issued = 0;
-  bool x_pending = false;
-  uint32_t x_parity = 0;
-  uint32_t xb_issued[4] = {0, 0, 0, 0};  // X loader: loads issued per box
 
   if (warp == 0 && lane == 0) {
     // ---------------------------------------------------------- producer
@@ -297,7 +267,21 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
           ld(a_dst + 8192, &tmA, m0 + 64, k0);
         }
         // this CTA's B rows: all of them, or (a pair) its half of the columns
-        if (!B_MN) {
+        if (Epi::kDirect) {
+          // box row 32 g + 2 s + e of a 128-row box holds B row 8 s + 2 g + e
+          constexpr int JB = Cfg::B_ROWS / 128;
+#pragma unroll
+          for (int j = 0; j < JB; ++j) {
+            const int s8 = epi.b_row(n0, j + (int)rank * JB) >> 3;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              if (PAIR)
+                tma_load_4d_pair(b_dst + j * 16384 + g * 4096, &tmB, fb, k0, 0, g, s8);
+              else
+                tma_load_4d(b_dst + j * 16384 + g * 4096, &tmB, fb, k0, 0, g, s8);
+            }
+          }
+        } else if (!B_MN) {
           constexpr int JB = Cfg::B_ROWS / 128;
 #pragma unroll
           for (int j = 0; j < JB; ++j)
@@ -377,92 +361,170 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
         tc_commit(done);
     }
     __syncwarp();
-  } else if (XL && warp == 2 + GEMM_EPI_WARPS) {
-    // ---------------------------------------------------------- X loader
-    if (lane == 0) {
-      prefetch_tmap(&tmX);
-      uint32_t lt = 0;
-      bool ok = true;
-      for (int tile = unit; tile < tiles && ok; tile += n_units, ++lt) {
-        PF_TILE_DECODE(tile)
-        (void)sp;
-        (void)kb;
-        (void)ke;
-        const int xr = epi.x_row(m0);
-        // in the order the halves free them: box i of each half, then box i+1
-        for (int i = 0; i < XB_HALF && ok; ++i) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int j = h * XB_HALF + i;
-            if (!mbar_wait(xbe0 + 8 * j, (lt & 1) ^ 1)) {
-              ok = false;
-              break;
-            }
-            mbar_arrive_expect_tx(xbf0 + 8 * j, 16384);
-            tma_load_2d(smem_u32(xtile) + j * 16384, &tmX, xbf0 + 8 * j, epi.x_col(n0, j), xr);
-            xb_issued[j] = lt + 1;
-          }
-        }
-      }
-    }
   } else if (warp >= 2) {
     // ---------------------------------------------------------- epilogue
-    const int et = threadIdx.x - 64;
     const int q = warp & 3;                               // TMEM lane quarter
     const int c_begin = ((warp - 2) >> 2) * (BN / 2);     // this warp's column half
-    auto tile_n0 = [&](int t) {
-      const int r = t % mn_tiles;
-      return (m_fast ? r / num_m : r % num_n) * BN;
+    // the accumulator has been read: rank 0's MMA warp may fill it again
+    auto release = [&](uint32_t buf) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (PAIR && rank == 1)
+          mbar_arrive_remote_relaxed(smem_map_rank(tempty0 + 8 * buf, 0));
+        else
+          mbar_arrive(tempty0 + 8 * buf);
+      }
     };
-    if constexpr (Epi::kColPar) {  // parameters of the first tile
-      if (unit < tiles && et < BN) cpar_put(0, et, epi.col_param(tile_n0(unit), et));
-      epi_bar_and(true);
-    }
     uint32_t lt = 0;
-    for (int tile = unit; tile < tiles; tile += n_units, ++lt) {
-      PF_TILE_DECODE(tile)
-      const bool no_k = ke <= kb;
-      const uint32_t buf = lt & 1, use = lt >> 1;
-      if (Epi::kXTile && !XL && et == 0) {
-        mbar_arrive_expect_tx(xfull, Cfg::X_BYTES);
-        const int xr = epi.x_row(m0);
+    if constexpr (Epi::kRows) {
+      // No barrier couples the warps: one that sees a wait run out leaves alone.
+      constexpr int NCH = Epi::kPaired ? BN / 128 : BN / 64;  // 32-column chunks per warp
+      constexpr int XD = gemm_xd<Epi>(PAIR), AHEAD = XD - 1 < NCH ? XD - 1 : NCH;
+      const int cb = Epi::kPaired ? c_begin / 2 : c_begin;
+      const int sr = lane >> 2, sp = lane & 3;
+      typename Epi::Rows rows, nrows;
+      // A slot holds the chunk's 32 rows x 64 bytes of X.  Lane (sr, sp) copies
+      // pieces sp (16 bytes) of rows sr + 8 it to `mine`.  Fragments: row r's piece
+      // p sits at piece p ^ (r / 2 % 4), so that neither a matrix's eight rows nor
+      // the lanes' pieces meet in a bank; lane names row lane % 8 of matrix lane / 8.
+      uint8_t* const slots = epi_smem + (warp - 2) * (XD * 2048);
+      const uint32_t slots0 = smem_u32(slots);
+      const uint32_t mine = Epi::kDirect ? lane * 16 : sr * 64 + ((sp ^ ((sr >> 1) & 3)) << 4);
+      const uint32_t mrow = (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4);
+      auto info = [&](int t, typename Epi::Rows& r) -> int {  // rows of tile t; returns its n0
+        const int rem = t % mn_tiles;
+        const int m0 = (m_fast ? rem % num_m : rem / num_n) * TILE_M + (int)rank * GEMM_BM;
+        const int n0 = (m_fast ? rem / num_m : rem % num_n) * BN;
+        epi.rows_info(r, m0 + q * 32 + sr, n0);
+        return n0;
+      };
+      auto load = [&](uint32_t trow, int c, uint32_t* r) {
+        if constexpr (Epi::kDirect) {
 #pragma unroll
-        for (int j = 0; j < XCOLS / 64; ++j)
-          tma_load_2d(smem_u32(xtile) + j * 16384, &tmX, xfull, epi.x_col(n0, j), xr);
-        x_pending = true;
-        x_parity = lt & 1;
-      }
-      // next tile's column parameters: loaded now, stored after this tile
-      const int ntile = tile + n_units;
-      float4 npar = make_float4(0.f, 0.f, 0.f, 0.f);
-      if constexpr (Epi::kColPar)
-        if (ntile < tiles && et < BN) npar = epi.col_param(tile_n0(ntile), et);
-      const float4* cp = cpar + (lt & 1) * BN;
-      bool ok = mbar_wait(tfull0 + 8 * buf, use & 1);
-      tc_fence_after();
-      if (Epi::kXTile && !XL) {
-        mbar_wait(xfull, lt & 1);
-        x_pending = false;
-      }
-      const int rl = q * 32 + lane;
-      // split-K partial epilogues address row (split * M + row); -1 = out of range
-      const int erow = Epi::kSplitRows ? (m0 + rl < M ? sp * M + m0 + rl : -1) : m0 + rl;
-      const typename Epi::Row ri = epi.row_info(erow, n0);
-      const uint32_t trow = tmem + buf * BN + ((uint32_t)(q * 32) << 16);
-      if constexpr (Epi::kPaired) {
-        // columns c and c + BN/2 belong together (e.g. s and t of one channel)
-#pragma unroll 1
-        for (int c = c_begin / 2; c < c_begin / 2 + BN / 4; c += 32) {
-          float v[32], w[32];
-          tmem_ld32(trow + (uint32_t)c, v);
-          tmem_ld32(trow + (uint32_t)(c + BN / 2), w);
-          if (no_k) {
+          for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = w[i] = 0.f;
-          }
-          epi.apply_pair(ri, erow, n0, c, v, w, xtile, rl, cp);
+            for (int g = 0; g < 4; ++g)
+              tmem_ld_16x8_async(trow + ((uint32_t)(16 * h) << 16) +
+                                     (uint32_t)((c & ~127) + 32 * g + ((c & 127) >> 2)),
+                                 r + 16 * h + 4 * g);
+        } else {
+          tmem_ld_frag_async(trow + (uint32_t)c, r);
+          tmem_ld_frag_async(trow + (16u << 16) + (uint32_t)c, r + 16);
         }
-      } else {
+        tmem_wait_ld(r);
+      };
+      uint32_t put = 0, get = 0;  // pieces of how many chunks were requested / used
+      auto fetch = [&](const typename Epi::Rows& r, int n0, int ci) {
+        const int c = cb + 32 * ci;
+        if (n0 + c < N) {  // uniform
+#pragma unroll
+          for (int it = 0; it < 4; ++it)
+            cp_async16(slots0 + (put % XD) * 2048 + it * 512 + mine,
+                       epi.src(r, it, n0, c + 8 * sp));
+        }
+      };
+      int n0 = 0, nn0 = 0;
+      if (unit < tiles) {
+        n0 = info(unit, rows);
+#pragma unroll
+        for (int ci = 0; ci < AHEAD; ++ci, ++put) {
+          fetch(rows, n0, ci);
+          cp_async_commit();
+        }
+      }
+      for (int tile = unit; tile < tiles; tile += n_units, ++lt) {
+        const uint32_t buf = lt & 1, use = lt >> 1;
+        const bool more = tile + n_units < tiles;
+        if (more) {
+          nn0 = info(tile + n_units, nrows);
+        }
+        if (!mbar_wait_warp(tfull0 + 8 * buf, use & 1)) break;
+        tc_fence_after();
+        const uint32_t trow = tmem + buf * BN + ((uint32_t)(q * 32) << 16);
+#pragma unroll 1
+        for (int ci = 0; ci < NCH; ++ci, ++put, ++get) {
+          const int c = cb + 32 * ci;
+          const bool live = n0 + c < N;  // uniform
+          typename Epi::Par par;
+          if (live) epi.params(par, n0, c + (Epi::kDirect ? 8 : 2) * sp);
+          // the pieces of the chunk AHEAD of this one
+          if (ci + AHEAD < NCH)
+            fetch(rows, n0, ci + AHEAD);
+          else if (more)
+            fetch(nrows, nn0, ci + AHEAD - NCH);
+          cp_async_commit();
+          // r[16 h + 4 g + 2 k + e]: row sr + 16 h + 8 k, column 8 g + 2 sp + e (direct:
+          // column 8 sp + 2 g + e)
+          const uint32_t slot = (get % XD) * 2048;
+          uint32_t r[32];
+          load(trow, c, r);
+          if constexpr (Epi::kDirect) {
+            uint32_t r2[32];
+            if (Epi::kPaired) load(trow, c + BN / 2, r2);  // belong to columns c..
+            if (ci == NCH - 1) release(buf);
+            cp_async_wait<AHEAD>();  // this chunk's pieces have landed
+            if (live) {
+#pragma unroll
+              for (int it = 0; it < 4; ++it) {
+                float f[8], ft[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const int i = 16 * (it >> 1) + 4 * (j >> 1) + 2 * (it & 1) + (j & 1);
+                  f[j] = __uint_as_float(r[i]);
+                  if (Epi::kPaired) ft[j] = __uint_as_float(r2[i]);
+                }
+                const uint4 x = *reinterpret_cast<const uint4*>(slots + slot + it * 512 + mine);
+                if constexpr (Epi::kPaired)
+                  epi.apply(rows, par, it, n0, c + 8 * sp, f, ft, x);
+                else
+                  epi.apply(rows, par, it, n0, c + 8 * sp, f, x);
+              }
+            }
+          } else {
+            if (ci == NCH - 1) release(buf);
+            cp_async_wait<AHEAD>();
+            __syncwarp();  // the warp's pieces of this chunk have landed
+            uint32_t o[4][4];
+#pragma unroll
+            for (int it = 0; it < 4; ++it) {
+              uint32_t x[4];
+              ldmatrix_x4(slots0 + slot + it * 512 + mrow, x);
+              const uint32_t* a = r + 16 * (it >> 1) + 2 * (it & 1);
+#pragma unroll
+              for (int g = 0; g < 4; ++g)
+                o[it][g] = epi.apply(
+                    make_float2(__uint_as_float(a[4 * g]), __uint_as_float(a[4 * g + 1])), x[g]);
+            }
+            __syncwarp();  // the slot's readers are done: the output takes its place
+#pragma unroll
+            for (int it = 0; it < 4; ++it) stmatrix_x4(slots0 + slot + it * 512 + mrow, o[it]);
+            __syncwarp();
+            if (live) {
+#pragma unroll
+              for (int it = 0; it < 4; ++it) {
+                const uint4 w = *reinterpret_cast<const uint4*>(slots + slot + it * 512 + mine);
+                if (bf16* d = epi.dst(rows, it, n0, c + 8 * sp)) *reinterpret_cast<uint4*>(d) = w;
+              }
+            }
+          }
+        }
+        rows = nrows;
+        n0 = nn0;
+      }
+      cp_async_wait<0>();
+    } else {
+      for (int tile = unit; tile < tiles; tile += n_units, ++lt) {
+        PF_TILE_DECODE(tile)
+        const bool no_k = ke <= kb;
+        const uint32_t buf = lt & 1, use = lt >> 1;
+        const bool ok = mbar_wait(tfull0 + 8 * buf, use & 1);
+        tc_fence_after();
+        const int rl = q * 32 + lane;
+        // split-K partial epilogues address row (split * M + row); -1 = out of range
+        const int erow = Epi::kSplitRows ? (m0 + rl < M ? sp * M + m0 + rl : -1) : m0 + rl;
+        const typename Epi::Row ri = epi.row_info(erow, n0);
+        const uint32_t trow = tmem + buf * BN + ((uint32_t)(q * 32) << 16);
         // 32-column chunks, the TMEM load of chunk i+1 in flight while chunk i
         // is processed
         constexpr int NCH = BN / 64;
@@ -474,7 +536,7 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
           float v[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-          epi.apply(ri, erow, n0 + c, v, epi_smem, rl, c, cp);
+          epi.apply(ri, erow, n0 + c, v, epi_smem, rl);
         };
         uint32_t ra[32], rb[32];
         tmem_ld32_async(trow + (uint32_t)c_begin, ra);
@@ -482,37 +544,17 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
 #pragma unroll 1
         for (int ci = 0; ci < NCH; ci += 2) {
           const int c = c_begin + ci * 32;
-          const int xb = c >> 6;  // the X box of this chunk pair (XL)
-          if (XL) ok = mbar_wait(xbf0 + 8 * xb, lt & 1) && ok;
           tmem_ld32_async(trow + (uint32_t)(c + 32), rb);
           run(ra, c);
           tmem_wait_ld(rb);
           if (ci + 2 < NCH) tmem_ld32_async(trow + (uint32_t)(c + 64), ra);
           run(rb, c + 32);
-          if (XL) {  // this warp is done with the box: staging writes before the refill
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(xbe0 + 8 * xb);
-          }
           if (ci + 2 < NCH) tmem_wait_ld(ra);
         }
+        release(buf);
+        // leave together if any epilogue thread saw a wait run out
+        if (!epi_bar_and(ok)) break;
       }
-      if constexpr (Epi::kColPar)
-        if (ntile < tiles && et < BN) cpar_put((lt + 1) & 1, et, npar);
-      // staging writes into the X tile are ordered before the next tile's
-      // TMA load of it
-      if (Epi::kXTile && !XL) fence_proxy_async_smem();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        if (PAIR && rank == 1)
-          mbar_arrive_remote(smem_map_rank(tempty0 + 8 * buf, 0));
-        else
-          mbar_arrive(tempty0 + 8 * buf);
-      }
-      // all epilogue threads are done with the X tile (free for the next
-      // prefetch); leave together if any of them saw a wait run out
-      if (!epi_bar_and(ok)) break;
     }
   }
   tc_fence_before();
@@ -529,11 +571,6 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
         for (uint32_t it = s_consumed; it < issued; ++it)
           mbar_wait_drain(full0 + 8 * (it % STAGES), (it / STAGES) & 1);
       }
-    }
-    if (warp == 2 && lane == 0 && x_pending) mbar_wait_drain(xfull, x_parity);
-    if (XL && warp == 2 + GEMM_EPI_WARPS && lane == 0) {
-      for (int j = 0; j < XBOXES; ++j)
-        if (xb_issued[j]) mbar_wait_drain(xbf0 + 8 * j, (xb_issued[j] - 1) & 1);
     }
     if (warp == 1 && lane == 0) mbar_wait_drain(done, 0);
     __syncthreads();
@@ -554,33 +591,39 @@ __global__ void __launch_bounds__(GemmRoles<Epi>::kThreads, 1)
 }
 
 // ------------------------------------------------------------------ epilogues
-// row_info(row, n0) is evaluated once per tile and output row; apply(ri, row,
-// col, v, xt, rl, cl) then receives 32 consecutive accumulator columns [col,
-// col+32) of that row, with rl / cl the row and column inside the tile and xt
-// the prefetched bf16 tile (kXTile epilogues: x_row(m0) / x_col(n0, j) give the
-// coordinates of the tile's 64-column boxes in the X tensor map).  kPaired
-// epilogues receive columns c and c + BN/2 together through apply_pair, and
-// prefetch BN/2 columns.  b_row(n0, j) is the first row of B (K-major) loaded
-// for 128-row box j of the tile starting at output column n0.  N is a
-// multiple of 32.
+// Row-per-lane epilogues: row_info(row, n0) is evaluated once per tile and
+// output row; apply(ri, row, col, v, stg, rl) then receives 32 consecutive
+// accumulator columns [col, col+32) of that row (rl: the row inside the tile).
+// kRows epilogues: rows_info(r, row, n0) describes a lane's rows row, row + 8,
+// row + 16, row + 24 of the tile that starts at output column n0; src(r, it, n0,
+// c) is the address of the 16 bytes that its it-th row needs for columns n0 + c
+// .. + 7 (where there are none: of any 16 bytes that can be read, so that the
+// copies need no branch).  kDirect: params(par, n0, c) reads the parameters of
+// columns n0 + c .. + 7 and apply(r, par, it, n0, c, f, x) stores them (kPaired:
+// with columns c + BN/2 in ft).  Else apply(f, x) gives an output pair and dst
+// the address of 8 output columns of a row, or null.  b_row(n0, j) is the first
+// row of B (K-major) loaded for 128-row box j of the tile starting at output
+// column n0.  N is a multiple of 32.
 struct EpiBase {
-  static constexpr bool kXTile = false;
+  static constexpr bool kRows = false;
+  static constexpr bool kDirect = false;
+  static constexpr int kPairDepth = 0;
   static constexpr bool kPaired = false;
   static constexpr bool kSplitRows = false;
-  static constexpr bool kColPar = false;
-  // may run on CTA pairs (256-wide tiles with enough of them); an epilogue
-  // slower than its mainloop does better on single CTAs, whose tiles do not
-  // wait for the other CTA's epilogue
-  static constexpr bool kPairs = true;
   // shared memory for staging the output (0: the epilogue stores from registers)
   static constexpr uint32_t kStageBytes = 0;
-  __device__ __forceinline__ float4 col_param(int, int) const { return make_float4(0, 0, 0, 0); }
-  __device__ __forceinline__ int x_row(int m0) const { return m0; }
-  __device__ __forceinline__ int x_col(int n0, int j) const { return n0 + 64 * j; }
   __device__ __forceinline__ int b_row(int n0, int j) const { return n0 + 128 * j; }
-  template <class R>
-  __device__ __forceinline__ void apply_pair(const R&, int, int, int, float*, float*, uint8_t*,
-                                             int, const float4*) const {}
+};
+struct EpiRowsBase : EpiBase {
+  static constexpr bool kRows = true;
+  static constexpr int kPairDepth = 2;  // gemm_xd of a CTA pair
+  struct Par {};
+  __device__ __forceinline__ void params(Par&, int, int) const {}
+  // acc + X (the sums of a product and a bf16 matrix)
+  __device__ __forceinline__ uint32_t apply(float2 f, uint32_t x) const {
+    const float2 a = unpack_bf16(x);
+    return pack_bf16(f.x + a.x, f.y + a.y);
+  }
 };
 
 // v = acc (+ bias[col]) (+ addend[row, col]); stored as fp32 and/or bf16.
@@ -596,16 +639,14 @@ struct EpiLinear : EpiBase {
   long ld_f32;
   bf16* out_bf16;
   long ld_bf16;
-  const bf16* add_bf16;
-  long ld_add_bf16;
   int act_silu;
   bf16* pre_bf16;
   long ld_pre;
   const bf16* dsilu_of;
   long ld_dsilu;
   __device__ __forceinline__ Row row_info(int row, int) const { return Row{row < M}; }
-  __device__ __forceinline__ void apply(const Row& ri, int row, int col, float* v, const uint8_t*,
-                                        int, int, const float4*) const {
+  __device__ __forceinline__ void apply(const Row& ri, int row, int col, float* v, uint8_t*,
+                                        int) const {
     if (!ri.ok || col >= N) return;
     if (bias) {
 #pragma unroll
@@ -620,20 +661,6 @@ struct EpiLinear : EpiBase {
       for (int i = 0; i < 32; i += 4) {
         float4 b = *reinterpret_cast<const float4*>(a + i);
         v[i] += b.x; v[i + 1] += b.y; v[i + 2] += b.z; v[i + 3] += b.w;
-      }
-    }
-    if (add_bf16) {
-      const bf16* a = add_bf16 + (long)row * ld_add_bf16 + col;
-#pragma unroll
-      for (int i = 0; i < 32; i += 8) {
-        const uint4 u = *reinterpret_cast<const uint4*>(a + i);
-        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float2 f = unpack_bf16(w[j]);
-          v[i + 2 * j] += f.x;
-          v[i + 2 * j + 1] += f.y;
-        }
       }
     }
     if (pre_bf16) {
@@ -675,14 +702,12 @@ struct EpiLinear : EpiBase {
 };
 
 // A linear epilogue (v = acc + bias, fp32 and / or bf16 out) that stores
-// whole rows: each warp stages its 32 x 32 chunk in shared memory (rows 36
-// floats apart, so neither the row-per-lane writes nor the row reads conflict)
-// and writes it back row by row, 128 contiguous bytes of fp32 per row.
-// Used where the output is large next to the contraction (short K), so that
-// the stores from one row per lane would bound the epilogue.
+// whole rows: each warp stages its 32 x 32 chunk in shared memory and writes
+// it back row by row, 128 contiguous bytes of fp32 per row.  Used where the
+// output is large next to the contraction (short K), so that the stores from
+// one row per lane would bound the epilogue.
 struct EpiLinearStaged : EpiBase {
-  static constexpr int kRowF = 36;  // floats per staged row
-  static constexpr uint32_t kStageBytes = GEMM_EPI_WARPS * 32 * kRowF * 4;
+  static constexpr uint32_t kStageBytes = GEMM_STG_BYTES;
   struct Row {
     bool ok;
   };
@@ -694,10 +719,10 @@ struct EpiLinearStaged : EpiBase {
   long ld_bf16;
   __device__ __forceinline__ Row row_info(int row, int) const { return Row{row < M}; }
   __device__ __forceinline__ void apply(const Row&, int row, int col, float* v, uint8_t* stg,
-                                        int rl, int, const float4*) const {
+                                        int rl) const {
     if (col >= N) return;  // uniform across the warp
     const int lane = threadIdx.x & 31, ew = (threadIdx.x >> 5) - 2;
-    float* s = reinterpret_cast<float*>(stg) + ew * (32 * kRowF);
+    float* s = reinterpret_cast<float*>(stg) + ew * 1024;
     if (bias) {
 #pragma unroll
       for (int i = 0; i < 32; i += 4) {
@@ -705,33 +730,52 @@ struct EpiLinearStaged : EpiBase {
         v[i] += b.x; v[i + 1] += b.y; v[i + 2] += b.z; v[i + 3] += b.w;
       }
     }
-#pragma unroll
-    for (int i = 0; i < 32; i += 4)
-      *reinterpret_cast<float4*>(s + lane * kRowF + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    stg_put_row(s, lane, v);
     __syncwarp();
     const int rfirst = row - (rl & 31);
     if (out_f32) {  // 8 lanes per row, 4 rows per instruction
 #pragma unroll
       for (int it = 0; it < 8; ++it) {
-        const int rr = it * 4 + (lane >> 3), pc = (lane & 7) * 4;
-        const float4 val = *reinterpret_cast<const float4*>(s + rr * kRowF + pc);
+        const int rr = it * 4 + (lane >> 3), p = lane & 7;
+        const float4 val = *stg_ptr(s, rr, p);
         if (rfirst + rr < M)
-          *reinterpret_cast<float4*>(out_f32 + (long)(rfirst + rr) * ld_f32 + col + pc) = val;
+          *reinterpret_cast<float4*>(out_f32 + (long)(rfirst + rr) * ld_f32 + col + 4 * p) = val;
       }
     }
     if (out_bf16) {  // 4 lanes per row (8 values each), 8 rows per instruction
 #pragma unroll
       for (int it = 0; it < 4; ++it) {
-        const int rr = it * 8 + (lane >> 2), pc = (lane & 3) * 8;
-        const float4 a = *reinterpret_cast<const float4*>(s + rr * kRowF + pc);
-        const float4 b = *reinterpret_cast<const float4*>(s + rr * kRowF + pc + 4);
+        const int rr = it * 8 + (lane >> 2), p = lane & 3;
+        float f[8];
+        stg_get8(s, rr, p, f);
         if (rfirst + rr < M)
-          *reinterpret_cast<uint4*>(out_bf16 + (long)(rfirst + rr) * ld_bf16 + col + pc) =
-              make_uint4(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w), pack_bf16(b.x, b.y),
-                         pack_bf16(b.z, b.w));
+          *reinterpret_cast<uint4*>(out_bf16 + (long)(rfirst + rr) * ld_bf16 + col + 8 * p) =
+              pack8_bf16(f);
       }
     }
     __syncwarp();  // the staging is reused by the next chunk
+  }
+};
+
+// out = acc + add, bf16, row strides ld and ld_add (the residual and direct
+// gradient sums of the cross injection).
+struct EpiAddRows : EpiRowsBase {
+  struct Rows {
+    int row;
+  };
+  int M, N;
+  const bf16* add;
+  long ld_add;
+  bf16* out;
+  long ld;
+  __device__ __forceinline__ void rows_info(Rows& r, int row, int) const { r.row = row; }
+  __device__ __forceinline__ const bf16* src(const Rows& r, int it, int n0, int c) const {
+    const int row = r.row + 8 * it;
+    return add + (row < M ? (long)row * ld_add + n0 + c : 0);
+  }
+  __device__ __forceinline__ bf16* dst(const Rows& r, int it, int n0, int c) const {
+    const int row = r.row + 8 * it;
+    return row < M ? out + (long)row * ld + n0 + c : nullptr;
   }
 };
 
@@ -743,182 +787,122 @@ struct EpiLinearStaged : EpiBase {
 // (i+shift)*P + a*k1 + c/d:
 //   gated: X_out = X + sigmoid(w_x X + w_dlt D + b_g) D    (Eq. inj-gate)
 //   add:   X_out = X + D                                    (Eq. inj-add)
-// X is read from the prefetched tile: rows r + shift*k2 of the view
-// [B*m*k2, k1*d] of X (zero-padded to whole blocks when L % P != 0).
-struct EpiInject1D : EpiBase {
-  static constexpr bool kXTile = true;
-  static constexpr bool kPairs = false;  // epilogue-bound (measured slower on pairs)
-  struct Row {
-    bool ok;    // row < M
-    long off0;  // element offset of the group's first token in X_out
-    int lim;    // columns < lim belong to tokens < L of a target block
-    SegRows seg;
+// With shift = 1 the last proxy of a sequence feeds no block; its rows copy
+// the sequence's block 0, which receives nothing, X_out = X.
+struct EpiInject1D : EpiRowsBase {
+  static constexpr bool kDirect = true;
+  struct Rows {
+    long off[4];  // element offset of the row's first token in X and X_out
+    int lim[4];   // columns < lim belong to tokens < L of the row's block (0: none)
+    int row;
+    uint32_t copy;  // bit it: row it copies block 0
+  };
+  struct Par {
+    float b[8], wx[8], wd[8], bg[8];
   };
   int M, N;
   const float* bias;
   bf16* D_save;
+  const bf16* X;
   bf16* X_out;
   const float *w_x, *w_dlt, *b_g;
   int d, k1, k2, m, L, shift, gated;
-  __device__ __forceinline__ int x_row(int m0) const { return m0 + shift * k2; }
-  __device__ __forceinline__ Row row_info(int row, int) const {
-    Row r{row < M, 0, 0};
-    const int a = row % k2, prox = row / k2;
-    const int b = prox / m, i = prox % m;
-    const int it = i + shift;
-    const long tok0 = (long)it * (k1 * k2) + (long)a * k1;
-    if (r.ok && it < m && tok0 < L) {
-      r.off0 = ((long)b * L + tok0) * d;
-      const long lim = (L - tok0) * d;
-      r.lim = lim < N ? (int)lim : N;
-    }
-    r.seg.gather(r.off0, r.ok ? r.lim : 0);
-    return r;
-  }
-  // staged per column: (bias, w_x, w_dlt, b_g)
-  static constexpr bool kColPar = true;
-  __device__ __forceinline__ float4 col_param(int n0, int cl) const {
-    const int col = n0 + cl;
-    if (col >= N) return make_float4(0.f, 0.f, 0.f, 0.f);
-    const float b = bias[col];
-    if (!gated) return make_float4(b, 0.f, 0.f, 0.f);
-    const int ch = col % d;
-    return make_float4(b, w_x[ch], w_dlt[ch], b_g[ch]);
-  }
-  // The warp's 32 x 32 chunk of X_out and then of D is staged in the X tile
-  // cells it has just read and stored with whole-row segments.  cp: the
-  // staged parameters, one float4 per (4-column group, parameter).  The gate
-  // arithmetic runs on column pairs with packed fp32x2 FMAs (each lane an
-  // IEEE fp32 FMA, as the scalar form), and the cell addresses are formed
-  // once per chunk.
-  __device__ __forceinline__ void apply(const Row& ri, int row, int col, float* v, uint8_t* xt,
-                                        int rl, int cl, const float4* cp) const {
-    if (col >= N) return;  // uniform across the warp
-    const int lane = threadIdx.x & 31, q = rl >> 5;
-    const float4* cg = cp + (cl >> 2) * 4;
-    // this row's four 16-byte cells of the chunk (128-byte swizzle)
-    const int c8 = (cl & 63) >> 3, sw = rl & 7;
-    uint8_t* const rowp = xt + (cl >> 6) * 16384 + rl * 128;
-    uint4* cell[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) cell[j] = reinterpret_cast<uint4*>(rowp + (((c8 | j) ^ sw) << 4));
-    uint32_t dpk[16];  // D = acc + bias, bf16 pairs
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint4 xu = *cell[j];
-      const uint32_t xw[4] = {xu.x, xu.y, xu.z, xu.w};
-      uint32_t ow[4];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int g4 = 2 * j + h;  // 4-column group of the chunk
-        const float4 b = cg[g4 * 4];
-        const float bb[4] = {b.x, b.y, b.z, b.w};
-        float wx[4], wd[4], bg[4];
-        if (gated) {
-          const float4 a = cg[g4 * 4 + 1], dd = cg[g4 * 4 + 2], e = cg[g4 * 4 + 3];
-          wx[0] = a.x; wx[1] = a.y; wx[2] = a.z; wx[3] = a.w;
-          wd[0] = dd.x; wd[1] = dd.y; wd[2] = dd.z; wd[3] = dd.w;
-          bg[0] = e.x; bg[1] = e.y; bg[2] = e.z; bg[3] = e.w;
-        }
-#pragma unroll
-        for (int pr = 0; pr < 2; ++pr) {
-          const int e0 = 8 * j + 4 * h + 2 * pr, k = 2 * pr;
-          const float2 x2 = unpack_bf16(xw[2 * h + pr]);
-          const float2 d2 = __fadd2_rn(make_float2(v[e0], v[e0 + 1]), make_float2(bb[k], bb[k + 1]));
-          float2 o2;
-          if (gated) {
-            const float2 g2 = __ffma2_rn(make_float2(wx[k], wx[k + 1]), x2,
-                                         __ffma2_rn(make_float2(wd[k], wd[k + 1]), d2,
-                                                    make_float2(bg[k], bg[k + 1])));
-            const float2 hg = __fmul2_rn(g2, make_float2(0.5f, 0.5f));
-            const float2 t2 = make_float2(tanh_approx(hg.x), tanh_approx(hg.y));
-            const float2 s2 = __ffma2_rn(make_float2(0.5f, 0.5f), t2, make_float2(0.5f, 0.5f));
-            o2 = __ffma2_rn(s2, d2, x2);
-          } else {
-            o2 = __fadd2_rn(x2, d2);
-          }
-          ow[2 * h + pr] = pack_bf16(o2.x, o2.y);
-          dpk[(e0 >> 1)] = pack_bf16(d2.x, d2.y);
-        }
-      }
-      *cell[j] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-    }
-    __syncwarp();
-    // whole-row stores: instruction it writes rows 8 it + lane / 4 of the warp,
-    // 16-byte piece p = lane % 4; the swizzle phase of those rows is lane / 4
-    const int p = lane & 3, rq = lane >> 2;
-    const uint8_t* srow = xt + (cl >> 6) * 16384 + (q * 32 + rq) * 128 + (((c8 | p) ^ rq) << 4);
+  __device__ __forceinline__ void rows_info(Rows& r, int row, int) const {
+    r.row = row;
+    r.copy = 0;
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
-      const uint4 val = *reinterpret_cast<const uint4*>(srow + it * 8 * 128);
-      if (col + p * 8 < ri.seg.lim[it])
-        *reinterpret_cast<uint4*>(X_out + ri.seg.off[it] + col + p * 8) = val;
-    }
-    __syncwarp();
-    if (D_save) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        *cell[j] = make_uint4(dpk[4 * j], dpk[4 * j + 1], dpk[4 * j + 2], dpk[4 * j + 3]);
-      __syncwarp();
-      const int rfirst = row - (rl & 31);
-      bf16* dbase = D_save + (long)(rfirst + rq) * N + col + p * 8;
-#pragma unroll
-      for (int it = 0; it < 4; ++it) {
-        const uint4 val = *reinterpret_cast<const uint4*>(srow + it * 8 * 128);
-        if (rfirst + rq + 8 * it < M) *reinterpret_cast<uint4*>(dbase + (long)it * 8 * N) = val;
+      const int rr = row + 8 * it;
+      const int a = rr % k2, prox = rr / k2;
+      const int b = prox / m, i = prox % m;
+      int blk = i + shift;
+      if (blk >= m) {
+        blk = 0;
+        r.copy |= 1u << it;
       }
-      __syncwarp();
+      const long tok0 = (long)blk * (k1 * k2) + (long)a * k1;
+      const long lim = (L - tok0) * d;
+      r.off[it] = ((long)b * L + tok0) * d;
+      r.lim[it] = rr < M && lim > 0 ? (lim < N ? (int)lim : N) : 0;
     }
+  }
+  __device__ __forceinline__ const bf16* src(const Rows& r, int it, int n0, int c) const {
+    return X + (n0 + c < r.lim[it] ? r.off[it] + n0 + c : 0);
+  }
+  __device__ __forceinline__ void params(Par& p, int n0, int c) const {
+    const int col = n0 + c;
+    ld8_f32(bias + col, p.b);
+    if (gated) {
+      const int ch = col % d;
+      ld8_f32(w_x + ch, p.wx);
+      ld8_f32(w_dlt + ch, p.wd);
+      ld8_f32(b_g + ch, p.bg);
+    }
+  }
+  // the gate arithmetic runs on column pairs with packed fp32x2 FMAs (each
+  // lane an IEEE fp32 FMA, as the scalar form)
+  __device__ __forceinline__ void apply(const Rows& r, const Par& p, int it, int n0, int c,
+                                        const float* f, uint4 x) const {
+    const int col = n0 + c;
+    const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+    uint32_t ow[4], dw[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int k = 2 * j;
+      const float2 x2 = unpack_bf16(xw[j]);
+      const float2 d2 = __fadd2_rn(make_float2(f[k], f[k + 1]), make_float2(p.b[k], p.b[k + 1]));
+      float2 o2;
+      if (gated) {
+        const float2 g2 = __ffma2_rn(make_float2(p.wx[k], p.wx[k + 1]), x2,
+                                     __ffma2_rn(make_float2(p.wd[k], p.wd[k + 1]), d2,
+                                                make_float2(p.bg[k], p.bg[k + 1])));
+        const float2 hg = __fmul2_rn(g2, make_float2(0.5f, 0.5f));
+        const float2 t2 = make_float2(tanh_approx(hg.x), tanh_approx(hg.y));
+        const float2 s2 = __ffma2_rn(make_float2(0.5f, 0.5f), t2, make_float2(0.5f, 0.5f));
+        o2 = __ffma2_rn(s2, d2, x2);
+      } else {
+        o2 = __fadd2_rn(x2, d2);
+      }
+      ow[j] = pack_bf16(o2.x, o2.y);
+      dw[j] = pack_bf16(d2.x, d2.y);
+    }
+    if (col < r.lim[it])
+      *reinterpret_cast<uint4*>(X_out + r.off[it] + col) =
+          (r.copy >> it) & 1u ? x : make_uint4(ow[0], ow[1], ow[2], ow[3]);
+    const int row = r.row + 8 * it;
+    if (D_save && row < M)
+      *reinterpret_cast<uint4*>(D_save + (long)row * N + col) =
+          make_uint4(dw[0], dw[1], dw[2], dw[3]);
   }
 };
 
 // First compression level's input gradient added to the direct injection
-// gradient: rows r = (b*m + i)*k2 + a, columns (token c/d of the group, channel
-// c%d) -> token i*P + a*k1 + c/d of sequence b.  The direct gradient is read
-// from the prefetched tile of dXd, the view [B*m*k2, k1*d] of a buffer padded
-// to whole blocks (dX itself when L % P == 0); the sum is written to dX.
-struct EpiDX1D : EpiBase {
-  static constexpr bool kXTile = true;
-  struct Row {
-    bool ok;
-    long off0;
-    int lim;
-    SegRows seg;
+// gradient that dX already holds: rows r = (b*m + i)*k2 + a, columns (token
+// c/d of the group, channel c%d) -> token i*P + a*k1 + c/d of sequence b.
+// Each element of dX is read and written by one lane.
+struct EpiDX1D : EpiRowsBase {
+  struct Rows {
+    long off[4];
+    int lim[4];
   };
   int M, N;
   bf16* dX;
   int d, k1, k2, m, L;
-  __device__ __forceinline__ Row row_info(int row, int) const {
-    Row r{row < M, 0, 0};
+  __device__ __forceinline__ void rows_info(Rows& r, int row, int) const {
     const int per_seq = m * k2;
-    const int b = row / per_seq, rr = row % per_seq;
-    const long tok0 = (long)rr * k1;
-    if (r.ok && tok0 < L) {
-      r.off0 = ((long)b * L + tok0) * d;
-      const long lim = (L - tok0) * d;
-      r.lim = lim < N ? (int)lim : N;
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+      const int rr = row + 8 * it, b = rr / per_seq;
+      const long tok0 = (long)(rr % per_seq) * k1, lim = (L - tok0) * d;
+      r.off[it] = ((long)b * L + tok0) * d;
+      r.lim[it] = rr < M && lim > 0 ? (lim < N ? (int)lim : N) : 0;
     }
-    r.seg.gather(r.off0, r.ok ? r.lim : 0);
-    return r;
   }
-  // staged in the tile cells just read, stored with whole-row segments
-  __device__ __forceinline__ void apply(const Row& ri, int, int col, float* v, uint8_t* xt,
-                                        int rl, int cl, const float4*) const {
-    if (col >= N) return;  // uniform across the warp
-#pragma unroll
-    for (int i8 = 0; i8 < 32; i8 += 8) {
-      float x[8];
-      xtile_load8(xt, rl, cl + i8, x);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) x[j] += v[i8 + j];
-      xtile_put8(xt, rl, cl + i8, x);
-    }
-    __syncwarp();
-    warp_store_rows(xt, rl >> 5, cl, [&](int rr, int p) -> bf16* {
-      const int it = rr >> 3;
-      return col + p * 8 < ri.seg.lim[it] ? dX + ri.seg.off[it] + col + p * 8 : nullptr;
-    });
-    __syncwarp();
+  __device__ __forceinline__ const bf16* src(const Rows& r, int it, int n0, int c) const {
+    return dX + (n0 + c < r.lim[it] ? r.off[it] + n0 + c : 0);
+  }
+  __device__ __forceinline__ bf16* dst(const Rows& r, int it, int n0, int c) const {
+    return n0 + c < r.lim[it] ? dX + r.off[it] + n0 + c : nullptr;
   }
 };
 
@@ -943,8 +927,8 @@ struct EpiAppendKV : EpiBase {
     }
     return r;
   }
-  __device__ __forceinline__ void apply(const Row& ri, int, int col, float* v, const uint8_t*, int,
-                                        int, const float4*) const {
+  __device__ __forceinline__ void apply(const Row& ri, int, int col, float* v, uint8_t*,
+                                        int) const {
     if (!ri.ok || col >= N) return;
     bf16* o = col < d ? K + ri.off + col : V + ri.off + (col - d);
 #pragma unroll
@@ -957,22 +941,26 @@ struct EpiAppendKV : EpiBase {
 // W_d1 [2*P*d, d] holds s for token p of a patch at rows [2pd, 2pd+d) and t at
 // [2pd+d, 2(p+1)d).  Output tile n0 = 256*nt covers token p = nt / (d/128) and
 // channels [cb, cb+128), cb = 128 * (nt % (d/128)): its B rows are loaded as
-// s (columns 0..127) then t (128..255), so each thread holds matching s and t.
-// X comes from the prefetched tile of the patch-ordered copy Xp [B*m, P*d];
+// s (columns 0..127) then t (128..255), so each lane holds matching s and t.
 // LayerNorm statistics per token from `stats` (mean, 1/std).  s is saved in
 // patch order [B*m, P*d] for the backward.
-struct EpiAffine2D : EpiBase {
-  static constexpr bool kXTile = true;
+struct EpiAffine2D : EpiRowsBase {
+  static constexpr bool kDirect = true;
   static constexpr bool kPaired = true;
-  struct Row {
-    bool ok;
-    long xoff;  // element offset of (token, channel cb) in X_out
-    float mu, rs;
-    SegRows seg;  // X_out offsets of the rows this lane stores (lim 1: row exists)
+  // two chunks ahead of X (K = d <= 512: the epilogue, not the ring, bounds it)
+  static constexpr int kPairDepth = 4;
+  struct Rows {
+    long off[4];  // element offset of (token, channel cb) in X and X_out
+    float2 st[4];
+    int row;
+  };
+  struct Par {
+    float bs[8], bt[8];
   };
   int M;
   const float* bias;
   bf16* S_save;
+  const bf16* X;
   bf16* X_out;
   const float* stats;
   int d, patch, gh, gw, m;
@@ -981,121 +969,82 @@ struct EpiAffine2D : EpiBase {
   __device__ __forceinline__ int b_row(int n0, int j) const {
     return ptok(n0) * 2 * d + j * d + cbase(n0);
   }
-  __device__ __forceinline__ int x_col(int n0, int j) const {
-    return ptok(n0) * d + cbase(n0) + 64 * j;
-  }
-  __device__ __forceinline__ Row row_info(int row, int n0) const {
-    Row r{row < M, 0, 0.f, 0.f};
-    if (r.ok) {
-      const int npw = gw / patch;
-      const int b = row / m, pr = row % m, by = pr / npw, bx = pr % npw;
-      const int p = ptok(n0), py = p / patch, px = p % patch;
-      const long tok = (long)b * gh * gw + (long)(by * patch + py) * gw + bx * patch + px;
-      r.xoff = tok * d + cbase(n0);
-      r.mu = stats[2 * tok];
-      r.rs = stats[2 * tok + 1];
-    }
-    r.seg.gather(r.xoff, r.ok ? 1 : 0);
-    return r;
-  }
-  // staged per column c of the s half: (bias of s, bias of t)
-  static constexpr bool kColPar = true;
-  __device__ __forceinline__ float4 col_param(int n0, int cl) const {
-    if (cl >= 128) return make_float4(0.f, 0.f, 0.f, 0.f);
-    const float* bs = bias + (long)ptok(n0) * 2 * d + cbase(n0) + cl;
-    return make_float4(bs[0], bs[d], 0.f, 0.f);
-  }
-  // The warp's 32 x 32 chunk of X_out and then of S is staged in the X tile
-  // cells it has just read and stored with whole-row segments.
-  __device__ __forceinline__ void apply_pair(const Row& ri, int row, int n0, int c, float* vs,
-                                             float* vt, uint8_t* xt, int rl,
-                                             const float4* cp) const {
-    const int q = rl >> 5, p = ptok(n0), ch0 = cbase(n0) + c;
-    const float4* cg = cp + (c >> 2) * 4;
+  __device__ __forceinline__ void rows_info(Rows& r, int row, int n0) const {
+    const int npw = gw / patch, p = ptok(n0), py = p / patch, px = p % patch, cb = cbase(n0);
+    r.row = row;
 #pragma unroll
-    for (int i8 = 0; i8 < 32; i8 += 8) {
-      float x[8], o[8];
-      xtile_load8(xt, rl, c + i8, x);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int g4 = (i8 >> 2) + h;
-        const float4 bs = cg[g4 * 4], bt = cg[g4 * 4 + 1];
-        const float bsa[4] = {bs.x, bs.y, bs.z, bs.w}, bta[4] = {bt.x, bt.y, bt.z, bt.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int e = h * 4 + j;
-          const float sv = vs[i8 + e] + bsa[j];
-          vs[i8 + e] = sv;
-          o[e] = fmaf(1.f + sv, (x[e] - ri.mu) * ri.rs, vt[i8 + e] + bta[j]);
-        }
+    for (int it = 0; it < 4; ++it) {
+      const int rr = row + 8 * it;
+      r.off[it] = 0;
+      r.st[it] = make_float2(0.f, 0.f);
+      if (rr < M) {
+        const int b = rr / m, pr = rr % m, by = pr / npw, bx = pr % npw;
+        const long tok = (long)b * gh * gw + (long)(by * patch + py) * gw + bx * patch + px;
+        r.off[it] = tok * d + cb;
+        r.st[it] = __ldg(reinterpret_cast<const float2*>(stats) + tok);
       }
-      xtile_put8(xt, rl, c + i8, o);
     }
-    __syncwarp();
-    warp_store_rows(xt, q, c, [&](int rr, int pc) -> bf16* {
-      const int it = rr >> 3;
-      return ri.seg.lim[it] ? X_out + ri.seg.off[it] + c + pc * 8 : nullptr;
-    });
-    __syncwarp();
+  }
+  __device__ __forceinline__ const bf16* src(const Rows& r, int it, int, int c) const {
+    return X + (r.row + 8 * it < M ? r.off[it] + c : 0);
+  }
+  __device__ __forceinline__ void params(Par& p, int n0, int c) const {
+    const float* bs = bias + (long)ptok(n0) * 2 * d + cbase(n0) + c;
+    ld8_f32(bs, p.bs);
+    ld8_f32(bs + d, p.bt);
+  }
+  __device__ __forceinline__ void apply(const Rows& r, const Par& p, int it, int n0, int c, float* fs,
+                                        const float* ft, uint4 x) const {
+    const int row = r.row + 8 * it;
+    if (row >= M) return;
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+    float o[8];
 #pragma unroll
-    for (int i8 = 0; i8 < 32; i8 += 8) xtile_put8(xt, rl, c + i8, vs + i8);
-    __syncwarp();
-    const int rfirst = row - (rl & 31);
+    for (int j = 0; j < 8; ++j) {
+      const float2 x2 = unpack_bf16(w[j >> 1]);
+      const float xe = j & 1 ? x2.y : x2.x;
+      const float sv = fs[j] + p.bs[j];
+      fs[j] = sv;
+      o[j] = fmaf(1.f + sv, (xe - r.st[it].x) * r.st[it].y, ft[j] + p.bt[j]);
+    }
+    *reinterpret_cast<uint4*>(X_out + r.off[it] + c) = pack8_bf16(o);
     const long pd = (long)patch * patch * d;
-    warp_store_rows(xt, q, c, [&](int rr, int pc) -> bf16* {
-      const int r2 = rfirst + rr;
-      return r2 < M ? S_save + (long)r2 * pd + (long)p * d + ch0 + pc * 8 : nullptr;
-    });
-    __syncwarp();
+    *reinterpret_cast<uint4*>(S_save + (long)row * pd + (long)ptok(n0) * d + cbase(n0) + c) =
+        pack8_bf16(fs);
   }
 };
 
 // Compression input gradient of the 2D layer: rows are patches, columns
 // (token p = c / d of the patch, channel c % d); the direct gradient comes from
-// the prefetched tile of dXd (same patch order) and the sum is written to dX
-// at the token's raster position.
-struct EpiDX2D : EpiBase {
-  static constexpr bool kXTile = true;
-  struct Row {
-    bool ok;
-    long base;  // offset of the patch's top-left token in dX
-    SegRows seg;
+// dXd (same patch order) and the sum is written to dX at the token's raster
+// position (a 32-column chunk is 32 channels of one token: d % 32 == 0).
+struct EpiDX2D : EpiRowsBase {
+  struct Rows {
+    long base[4];  // offset of the patch's top-left token in dX
+    int row;
   };
   int M, N;
+  const bf16* dXd;
   bf16* dX;
   int d, patch, gh, gw, m;
-  __device__ __forceinline__ Row row_info(int row, int) const {
-    Row r{row < M, 0};
-    if (r.ok) {
-      const int npw = gw / patch;
-      const int b = row / m, pr = row % m, by = pr / npw, bx = pr % npw;
-      r.base = ((long)b * gh * gw + (long)by * patch * gw + bx * patch) * d;
+  __device__ __forceinline__ void rows_info(Rows& r, int row, int) const {
+    const int npw = gw / patch;
+    r.row = row;
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+      const int rr = row + 8 * it;
+      const int b = rr / m, pr = rr % m, by = pr / npw, bx = pr % npw;
+      r.base[it] = ((long)b * gh * gw + (long)by * patch * gw + bx * patch) * d;
     }
-    r.seg.gather(r.base, r.ok ? N : 0);
-    return r;
   }
-  // staged in the tile cells just read, stored with whole-row segments: a
-  // 32-column chunk is 32 channels of one token of the patch (d is a multiple
-  // of 32), 64 contiguous bytes of dX per row
-  __device__ __forceinline__ void apply(const Row& ri, int, int col, float* v, uint8_t* xt,
-                                        int rl, int cl, const float4*) const {
-    if (col >= N) return;  // uniform across the warp
-#pragma unroll
-    for (int i8 = 0; i8 < 32; i8 += 8) {
-      float x[8];
-      xtile_load8(xt, rl, cl + i8, x);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) x[j] += v[i8 + j];
-      xtile_put8(xt, rl, cl + i8, x);
-    }
-    __syncwarp();
-    const int p = col / d, ch = col - p * d, py = p / patch, px = p - py * patch;
-    const long colofs = ((long)py * gw + px) * d + ch;
-    warp_store_rows(xt, rl >> 5, cl, [&](int rr, int q) -> bf16* {
-      const int it = rr >> 3;
-      return col + q * 8 < ri.seg.lim[it] ? dX + ri.seg.off[it] + colofs + q * 8 : nullptr;
-    });
-    __syncwarp();
+  __device__ __forceinline__ const bf16* src(const Rows& r, int it, int n0, int c) const {
+    const int row = r.row + 8 * it;
+    return dXd + (row < M ? (long)row * N + n0 + c : 0);
+  }
+  __device__ __forceinline__ bf16* dst(const Rows& r, int it, int n0, int c) const {
+    const int col = n0 + c, p = col / d, py = p / patch;
+    const long ofs = ((long)py * gw + (p - py * patch)) * d + (col - p * d);
+    return r.row + 8 * it < M ? dX + r.base[it] + ofs : nullptr;
   }
 };
 
@@ -1111,8 +1060,8 @@ struct EpiPartial : EpiBase {
   __device__ __forceinline__ Row row_info(int erow, int) const {
     return Row{erow < 0 ? -1L : (long)erow * N};
   }
-  __device__ __forceinline__ void apply(const Row& ri, int, int col, float* v, const uint8_t*, int,
-                                        int, const float4*) const {
+  __device__ __forceinline__ void apply(const Row& ri, int, int col, float* v, uint8_t*,
+                                        int) const {
     if (ri.off < 0 || col >= N) return;
     float* o = part + ri.off + col;
 #pragma unroll

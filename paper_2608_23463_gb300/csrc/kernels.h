@@ -52,8 +52,8 @@ struct EpiLinearArgs {
   const float* bias = nullptr;    // [N]
   const float* addend = nullptr;  // [M, ld_add] fp32
   long ld_add = 0;
-  const bf16* add_bf16 = nullptr;  // [M, ld_add_bf16] bf16, added like addend
-  long ld_add_bf16 = 0;
+  const bf16* add_bf16 = nullptr;  // [M, ld_add_bf16] bf16, added like addend (K-major
+  long ld_add_bf16 = 0;            // A and a bf16 output only, with nothing else)
   // SiLU: the value after bias / addends is stored to pre_bf16 (if given),
   // then out = SiLU(value); dsilu_of: out = value * SiLU'(u), u read from a
   // bf16 matrix [M, ld_dsilu].  Either one disables split-K.
@@ -79,15 +79,14 @@ size_t splitk_scratch_bytes(int M, int N, int K);
 struct EpiInjectArgs {
   const float* bias;  // b_d1 [k1*d]
   bf16* D_save;       // [M, k1*d] or null
-  const bf16* Xsrc;   // X as [B*m*k2, k1*d] (zero-padded to whole blocks if L % P != 0)
-  bf16* X_out;
+  const bf16* X;      // [B, L, d]
+  bf16* X_out;        // [B, L, d], all of it written (shift = 1: block 0 from X)
   const float *w_x, *w_dlt, *b_g;  // gate vectors (gated) or null (add)
   int d, k1, k2, m, L, shift, gated;
 };
 
 struct EpiDXArgs {
-  const bf16* dXd;  // direct gradient as [B*m*k2, k1*d] (padded like Xsrc)
-  bf16* dX;
+  bf16* dX;  // [B, L, d]: holds the direct gradient, the product is added
   int d, k1, k2, m, L;
 };
 
@@ -104,7 +103,7 @@ struct EpiAffine2DArgs {
   bf16* S_save;        // s in patch order [B*m, P*d]
   bf16* X_out;         // [B, gh*gw, d]
   const float* stats;  // [B*gh*gw, 2] mean, 1/std of X per token
-  const bf16* Xp;      // X in patch order [B*m, P*d]
+  const bf16* X;       // [B, gh*gw, d]
   int d, patch, gh, gw, m;
 };
 cudaError_t gemm_affine2d(int M, int N, int K, Operand A, Operand B, const EpiAffine2DArgs& e,
@@ -270,10 +269,6 @@ cudaError_t attn_bwd(const bf16* qkv, const bf16* O, const bf16* dO, const float
                      bf16* dqkv, int B, int m, int d, int nh, bool causal, cudaStream_t st);
 
 // ----------------------------------------------------------- elementwise
-// Copy the first `rows` rows (width d) of each sequence of src [B, Ls, d] to
-// dst [B, Ld, d] (block 0 of the causal routing: X_out = X, dX = dX_out).
-cudaError_t copy_block0(const bf16* src, long Ls, bf16* dst, long Ld, int B, int d, int rows,
-                        cudaStream_t st);
 // dst [B, Lp, d] = src [B, L, d] padded with zero rows (Lp >= L).
 cudaError_t pad_rows(const bf16* src, bf16* dst, int B, long L, long Lp, int d, cudaStream_t st);
 
@@ -287,8 +282,7 @@ struct InjBwdArgs {
   const bf16* X;
   const bf16* D;
   bf16* dD;
-  bf16* dX;     // direct gradient, [B, Ldx, d]
-  long Ldx;     // rows per sequence of dX (L, or m*P when padded)
+  bf16* dX;     // direct gradient, [B, L, d] (shift = 1: block 0 from G)
   const float *w_x, *w_dlt, *b_g;
   int d, k1, k2, m, L, B, shift, gated;
 };
