@@ -18,105 +18,124 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-// One pass over the tokens of the 2D layer, one warp per token t = (b, y, x):
-// the patch copy Xp[r, (py*p + px)*d + ch] = X[t, ch] for patch r = (b, by, bx)
-// (Eq. partition, the compression GEMM's operand) and the token's LayerNorm
-// statistics stats[t] = (mean, 1/sqrt(var + 1e-6)) (Eq. inj-affine), from
-// registers (two passes over the row held by the warp).  d <= 512.
+// One pass over the tokens of the 2D layer, PG_T consecutive tokens t = (b, y, x)
+// per warp, their rows loaded together (one at a time left too little in flight:
+// 376 us for four 512 x 512 images at d = 512, 334 so, 6.5 TB/s): the patch copy Xp[r, (py*p + px)*d + ch] = X[t, ch] for
+// patch r = (b, by, bx) (Eq. partition, the compression GEMM's operand) and the
+// token's LayerNorm statistics stats[t] = (mean, 1/sqrt(var + 1e-6)) (Eq.
+// inj-affine), from registers (two passes over the row).  d <= 512.
+constexpr int PG_T = 4;
 __global__ void __launch_bounds__(256) patch_gather_stats_kernel(
     const bf16* __restrict__ X, bf16* __restrict__ Xp, float* __restrict__ stats, long T, int d,
     int patch, int gh, int gw) {
   const int pz = pdl_enter();
-  const long t = ((long)blockIdx.x * blockDim.x + threadIdx.x + pz) >> 5;
+  const long t0 = (((long)blockIdx.x * blockDim.x + threadIdx.x + pz) >> 5) * PG_T;
   const int lane = threadIdx.x & 31;
-  if (t >= T) return;
   const long HW = (long)gh * gw;
-  const int b = (int)(t / HW), yx = (int)(t % HW), y = yx / gw, x = yx % gw;
   const int npw = gw / patch, m = (gh / patch) * npw;
-  const long row = (long)b * m + (y / patch) * npw + x / patch;
-  const int p = (y % patch) * patch + (x % patch);
-  const bf16* src = X + t * d;
-  bf16* dst = Xp + row * ((long)patch * patch * d) + (long)p * d;
-  uint4 u[2];
-  float s = 0.f;
+  uint4 u[PG_T][2];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int c = lane * 8 + 256 * i;
-    if (c >= d) break;
-    u[i] = __ldcs(reinterpret_cast<const uint4*>(src + c));
-    *reinterpret_cast<uint4*>(dst + c) = u[i];
-    const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
+  for (int k = 0; k < PG_T; ++k)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 f = unpack_bf16(w[j]);
-      s += f.x + f.y;
+    for (int i = 0; i < 2; ++i) {
+      const int c = lane * 8 + 256 * i;
+      u[k][i] = make_uint4(0, 0, 0, 0);
+      if (t0 + k < T && c < d)
+        u[k][i] = __ldcs(reinterpret_cast<const uint4*>(X + (t0 + k) * d + c));
     }
-  }
-  const float mu = warp_sum_f(s) / d;
-  float q = 0.f;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int c = lane * 8 + 256 * i;
-    if (c >= d) break;
-    const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
+  for (int k = 0; k < PG_T; ++k) {
+    const long t = t0 + k;
+    if (t >= T) return;
+    const int b = (int)(t / HW), yx = (int)(t % HW), y = yx / gw, x = yx % gw;
+    const long row = (long)b * m + (y / patch) * npw + x / patch;
+    const int p = (y % patch) * patch + (x % patch);
+    bf16* dst = Xp + row * ((long)patch * patch * d) + (long)p * d;
+    float s = 0.f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 f = unpack_bf16(w[j]);
-      q += (f.x - mu) * (f.x - mu) + (f.y - mu) * (f.y - mu);
+    for (int i = 0; i < 2; ++i) {
+      const int c = lane * 8 + 256 * i;
+      if (c >= d) break;
+      *reinterpret_cast<uint4*>(dst + c) = u[k][i];
+      const uint32_t w[4] = {u[k][i].x, u[k][i].y, u[k][i].z, u[k][i].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 f = unpack_bf16(w[j]);
+        s += f.x + f.y;
+      }
     }
-  }
-  const float var = warp_sum_f(q) / d;
-  if (lane == 0) {
-    stats[2 * t] = mu;
-    stats[2 * t + 1] = rsqrtf(var + 1e-6f);
+    const float mu = warp_sum_f(s) / d;
+    float q = 0.f;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int c = lane * 8 + 256 * i;
+      if (c >= d) break;
+      const uint32_t w[4] = {u[k][i].x, u[k][i].y, u[k][i].z, u[k][i].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 f = unpack_bf16(w[j]);
+        q += (f.x - mu) * (f.x - mu) + (f.y - mu) * (f.y - mu);
+      }
+    }
+    const float var = warp_sum_f(q) / d;
+    if (lane == 0)
+      *reinterpret_cast<float2*>(stats + 2 * t) = make_float2(mu, rsqrtf(var + 1e-6f));
   }
 }
 
-// Timestep conditioning of one image: e = [cos(1000 t w_k), sin(1000 t w_k)],
-// w_k = 10000^(-k/128); a1 = W_t1 e + b_t1; u = SiLU(a1); gb = W_t2 u + b_t2
-// = [gamma | beta].  One CTA per image, one warp per output.
-__global__ void __launch_bounds__(256) temb_fwd_kernel(const float* __restrict__ t, int d,
-                                                       const bf16* __restrict__ W_t1,
-                                                       const float* __restrict__ b_t1,
-                                                       const bf16* __restrict__ W_t2,
-                                                       const float* __restrict__ b_t2,
-                                                       float* __restrict__ e_out,
-                                                       float* __restrict__ a1_out,
-                                                       float* __restrict__ u_out,
-                                                       float* __restrict__ gb_out) {
+// Timestep conditioning of image b = blockIdx.y: e = [cos(1000 t w_k), sin(1000 t
+// w_k)], w_k = 10000^(-k/128); a1 = W_t1 e + b_t1; u = SiLU(a1); gb = W_t2 u +
+// b_t2 = [gamma | beta].  One warp per output, 8 outputs a CTA, one kernel per
+// layer of the MLP (a single CTA per image, 3/2 d dot products one after another
+// in each of its warps, took 313 us at d = 512; the two take 8).
+constexpr int TE_WARPS = 8;
+__global__ void __launch_bounds__(32 * TE_WARPS)
+    temb_hidden_kernel(const float* __restrict__ t, int d, const bf16* __restrict__ W_t1,
+                       const float* __restrict__ b_t1, float* __restrict__ e_out,
+                       float* __restrict__ a1_out, float* __restrict__ u_out) {
   const int pz = pdl_enter();
-  extern __shared__ float sm[];  // e [256], u [d]
-  float* e = sm;
-  float* u = sm + 256;
-  const int b = blockIdx.x + pz, tid = threadIdx.x + pz, lane = tid & 31, warp = tid >> 5;
-  const float tb = 1000.f * t[b];
+  __shared__ float e[256];
+  const int b = blockIdx.y + pz, tid = threadIdx.x, lane = tid & 31;
   if (tid < 128) {
     const float w = expf(-(float)tid * (9.210340371976184f / 128.f));  // ln(10000)/128
-    const float a = tb * w;
+    const float a = 1000.f * t[b] * w;
     e[tid] = cosf(a);
     e[tid + 128] = sinf(a);
   }
   __syncthreads();
-  if (tid < 256) e_out[b * 256 + tid] = e[tid];
-  for (int o = warp; o < d; o += 8) {
-    float acc = 0.f;
-    for (int k = lane; k < 256; k += 32) acc = fmaf(__bfloat162float(W_t1[(long)o * 256 + k]), e[k], acc);
-    acc = warp_sum_f(acc);
-    if (lane == 0) {
-      const float a = acc + b_t1[o];
-      a1_out[(long)b * d + o] = a;
-      const float uu = a * sigmoidf_(a);
-      u[o] = uu;
-      u_out[(long)b * d + o] = uu;
-    }
+  if (blockIdx.x == 0) e_out[b * 256 + tid] = e[tid];
+  const int o = blockIdx.x * TE_WARPS + (tid >> 5) + pz;
+  if (o >= d) return;
+  float w[8], acc = 0.f;
+  load8_bf16(W_t1 + (long)o * 256 + lane * 8, w);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) acc = fmaf(w[j], e[lane * 8 + j], acc);
+  acc = warp_sum_f(acc);
+  if (lane == 0) {
+    const float a = acc + b_t1[o];
+    a1_out[(long)b * d + o] = a;
+    u_out[(long)b * d + o] = a * sigmoidf_(a);
   }
-  __syncthreads();
-  for (int o = warp; o < 2 * d; o += 8) {
-    float acc = 0.f;
-    for (int k = lane; k < d; k += 32) acc = fmaf(__bfloat162float(W_t2[(long)o * d + k]), u[k], acc);
-    acc = warp_sum_f(acc);
-    if (lane == 0) gb_out[(long)b * 2 * d + o] = acc + b_t2[o];
+}
+
+__global__ void __launch_bounds__(32 * TE_WARPS)
+    temb_out_kernel(const float* __restrict__ u, int d, const bf16* __restrict__ W_t2,
+                    const float* __restrict__ b_t2, float* __restrict__ gb) {
+  const int pz = pdl_enter();
+  const int b = blockIdx.y, lane = threadIdx.x & 31;
+  const int o = blockIdx.x * TE_WARPS + (threadIdx.x >> 5) + pz;
+  if (o >= 2 * d) return;
+  float acc = 0.f;
+  for (int k = lane * 8; k < d; k += 256) {
+    float w[8], v[8];
+    load8_bf16(W_t2 + (long)o * d + k, w);
+    *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(u + (long)b * d + k + pz);
+    *reinterpret_cast<float4*>(v + 4) = *reinterpret_cast<const float4*>(u + (long)b * d + k + 4 + pz);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc = fmaf(w[j], v[j], acc);
   }
+  acc = warp_sum_f(acc);
+  if (lane == 0) gb[(long)b * 2 * d + o] = acc + b_t2[o];
 }
 
 // adaLN of the proxies (one warp per proxy row r of image b = r / m):
@@ -171,13 +190,42 @@ __global__ void __launch_bounds__(256) inj_bwd_2d_kernel(
 #pragma unroll
     for (int j = 0; j < 8; ++j) cs[i][j] = ct[i][j] = 0.f;
   const long r1 = min(R, (long)(chunk + 1) * IB2_CP);
-  for (long row = (long)chunk * IB2_CP + warp; row < r1; row += 8) {
+  // a patch's token: packed rows of G, X and S and the statistics; the next
+  // patch's are loaded while this one's are used (rows read twice, one patch at a
+  // time: 1138 us for four 512 x 512 images at d = 512, 5.7 TB/s; so 988, 6.5 TB/s)
+  struct Tok {
+    uint4 g[IB2_MAXI], x[IB2_MAXI], s[IB2_MAXI];
+    float mu, rs;
+  };
+  auto load = [&](long row, Tok& k) {
     const int b = (int)(row / m), pr = (int)(row % m), by = pr / npw, bx = pr % npw;
     const long t = ((long)b * gh + by * patch + py) * gw + bx * patch + px;
-    const float mu = stats[2 * t], rs = stats[2 * t + 1];
-    const bf16* g = G + t * d;
-    const bf16* xr = X + t * d;
-    const bf16* sr = S + row * ((long)P * d) + (long)p * d;
+    k.mu = stats[2 * t];
+    k.rs = stats[2 * t + 1];
+#pragma unroll
+    for (int i = 0; i < IB2_MAXI; ++i) {
+      const int c = lane * 8 + 256 * i;
+      if (c >= d) break;
+      k.g[i] = __ldcs(reinterpret_cast<const uint4*>(G + t * d + c));
+      k.x[i] = __ldcs(reinterpret_cast<const uint4*>(X + t * d + c));
+      k.s[i] = __ldcs(reinterpret_cast<const uint4*>(S + row * ((long)P * d) + (long)p * d + c));
+    }
+  };
+  auto unpack8 = [](const uint4& u, float* v) {
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 f = unpack_bf16(w[q]);
+      v[2 * q] = f.x;
+      v[2 * q + 1] = f.y;
+    }
+  };
+  Tok cur, nxt;
+  long row = (long)chunk * IB2_CP + warp;
+  if (row < r1) load(row, cur);
+  for (; row < r1; row += 8) {
+    if (row + 8 < r1) load(row + 8, nxt);
+    const float mu = cur.mu, rs = cur.rs;
     bf16* dds = dD + row * (2L * P * d) + (long)p * 2 * d;
     bf16* ddt = dds + d;
     bf16* dxo = dXd + row * ((long)P * d) + (long)p * d;
@@ -187,9 +235,9 @@ __global__ void __launch_bounds__(256) inj_bwd_2d_kernel(
       const int c = lane * 8 + 256 * i;
       if (c >= d) break;
       float gv[8], xv[8], sv[8], o[8];
-      load8_bf16(g + c, gv);
-      load8_bf16(xr + c, xv);
-      load8_bf16(sr + c, sv);
+      unpack8(cur.g[i], gv);
+      unpack8(cur.x[i], xv);
+      unpack8(cur.s[i], sv);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const float n = (xv[j] - mu) * rs, dn = gv[j] * (1.f + sv[j]);
@@ -200,7 +248,7 @@ __global__ void __launch_bounds__(256) inj_bwd_2d_kernel(
         ct[i][j] += gv[j];
       }
       store8_bf16(dds + c, o);
-      *reinterpret_cast<uint4*>(ddt + c) = *reinterpret_cast<const uint4*>(g + c);
+      *reinterpret_cast<uint4*>(ddt + c) = cur.g[i];
     }
     const float m1 = warp_sum_f(s1) / d, m2 = warp_sum_f(s2) / d;
 #pragma unroll
@@ -208,9 +256,9 @@ __global__ void __launch_bounds__(256) inj_bwd_2d_kernel(
       const int c = lane * 8 + 256 * i;
       if (c >= d) break;
       float gv[8], xv[8], sv[8], o[8];
-      load8_bf16(g + c, gv);
-      load8_bf16(xr + c, xv);
-      load8_bf16(sr + c, sv);
+      unpack8(cur.g[i], gv);
+      unpack8(cur.x[i], xv);
+      unpack8(cur.s[i], sv);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const float n = (xv[j] - mu) * rs, dn = gv[j] * (1.f + sv[j]);
@@ -218,6 +266,7 @@ __global__ void __launch_bounds__(256) inj_bwd_2d_kernel(
       }
       store8_bf16(dxo + c, o);
     }
+    cur = nxt;
   }
   // the block's sums over its patches, in a fixed order (deterministic)
 #pragma unroll
@@ -291,7 +340,21 @@ __global__ void adaln_param_part_kernel(const float* __restrict__ dHq, const flo
   const int rows = (m + chunks - 1) / chunks;
   const long r0 = (long)b * m + (long)ck * rows, r1 = (long)b * m + min(m, (ck + 1) * rows);
   float g = 0.f, be = 0.f;
-  for (long r = r0; r < r1; ++r) {
+  long r = r0;
+  for (; r + 7 < r1; r += 8) {  // eight rows' loads in flight
+    float v[8], n[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      v[k] = dHq[(r + k) * d + c];
+      n[k] = nH[(r + k) * d + c];
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      g = fmaf(v[k], n[k], g);
+      be += v[k];
+    }
+  }
+  for (; r < r1; ++r) {
     const float v = dHq[r * d + c];
     g = fmaf(v, nH[r * d + c], g);
     be += v;
@@ -312,16 +375,35 @@ __global__ void adaln_param_final_kernel(const float* __restrict__ part, float* 
   dgb[i] = s;
 }
 
-// du = W_t2^T dgb, da1 = du * SiLU'(a1), per image (thread per column i).
-__global__ void temb_bwd_du_kernel(const float* __restrict__ dgb, const bf16* __restrict__ W_t2,
-                                   const float* __restrict__ a1, float* __restrict__ da1, int d) {
+// du = W_t2^T dgb, da1 = du * SiLU'(a1), per image.  A CTA takes 64 columns (two a
+// lane) and adds rows w, w + 32, ... in warp w, the warps' sums then in warp order
+// (a thread per column walking all 2d rows took 110 us at d = 512).
+constexpr int TD_WARPS = 32;
+__global__ void __launch_bounds__(32 * TD_WARPS)
+    temb_bwd_du_kernel(const float* __restrict__ dgb, const bf16* __restrict__ W_t2,
+                       const float* __restrict__ a1, float* __restrict__ da1, int d) {
   const int pz = pdl_enter();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x + pz, b = blockIdx.y;
-  if (i >= d) return;
+  __shared__ float red[TD_WARPS][64];
+  const int b = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int c0 = blockIdx.x * 64 + pz;
+  float2 s = make_float2(0.f, 0.f);
+#pragma unroll 8
+  for (int o = w; o < 2 * d; o += TD_WARPS) {
+    const float2 f = unpack_bf16(*reinterpret_cast<const uint32_t*>(W_t2 + (long)o * d + c0 + 2 * lane));
+    const float g = dgb[(long)b * 2 * d + o + pz];
+    s.x = fmaf(f.x, g, s.x);
+    s.y = fmaf(f.y, g, s.y);
+  }
+  red[w][2 * lane] = s.x;
+  red[w][2 * lane + 1] = s.y;
+  __syncthreads();
+  if (threadIdx.x >= 64) return;
   float du = 0.f;
-  for (int o = 0; o < 2 * d; ++o) du = fmaf(__bfloat162float(W_t2[(long)o * d + i]), dgb[(long)b * 2 * d + o], du);
-  const float z = a1[(long)b * d + i], sg = sigmoidf_(z);
-  da1[(long)b * d + i] = du * sg * (1.f + z * (1.f - sg));
+#pragma unroll
+  for (int k = 0; k < TD_WARPS; ++k) du += red[k][threadIdx.x];
+  const long i = (long)b * d + c0 + threadIdx.x;
+  const float z = a1[i], sg = sigmoidf_(z);
+  da1[i] = du * sg * (1.f + z * (1.f - sg));
 }
 
 // Weight gradients of the timestep MLP (sums over the B images):
@@ -361,7 +443,7 @@ cudaError_t patch_gather_stats(const bf16* X, bf16* Xp, float* stats, int B, int
   if (d > 512 || d % 8 != 0) return cudaErrorInvalidValue;
   const long T = (long)B * gh * gw;
   LaunchTimer lt("patch_gather_stats", st, 0.0, 4.0 * T * d + 8.0 * T);
-  return launch_kernel(patch_gather_stats_kernel, (unsigned)((T * 32 + 255) / 256), 256, 0, st, X,
+  return launch_kernel(patch_gather_stats_kernel, (unsigned)((T + 8 * PG_T - 1) / (8 * PG_T)), 256, 0, st, X,
                        Xp, stats, T, d, patch, gh, gw);
 }
 
@@ -369,8 +451,12 @@ cudaError_t temb_fwd(const float* t, int B, int d, const bf16* W_t1, const float
                      const bf16* W_t2, const float* b_t2, float* e, float* a1, float* u, float* gb,
                      cudaStream_t st) {
   LaunchTimer lt("temb_fwd", st, 2.0 * B * (256.0 * d + 2.0 * d * d), 2.0 * (256.0 * d + 2.0 * d * d));
-  return launch_kernel(temb_fwd_kernel, B, 256, (256 + d) * sizeof(float), st, t, d, W_t1, b_t1,
-                       W_t2, b_t2, e, a1, u, gb);
+  const cudaError_t err =
+      launch_kernel(temb_hidden_kernel, dim3((d + TE_WARPS - 1) / TE_WARPS, B), 32 * TE_WARPS, 0, st,
+                    t, d, W_t1, b_t1, e, a1, u);
+  if (err != cudaSuccess) return err;
+  return launch_kernel(temb_out_kernel, dim3((2 * d + TE_WARPS - 1) / TE_WARPS, B), 32 * TE_WARPS, 0,
+                       st, u, d, W_t2, b_t2, gb);
 }
 
 cudaError_t adaln_fwd(const float* H, const float* gb, float* nH, float* rstd, bf16* Hq, long R,
@@ -431,8 +517,8 @@ cudaError_t temb_bwd(const float* dgb, const bf16* W_t2, const float* a1, const 
                      const float* e, float* da1, const TembGrads& g, int B, int d,
                      cudaStream_t st) {
   LaunchTimer lt("temb_bwd", st, 0.0, 8.0 * d * d);
-  dim3 g1((d + 255) / 256, B);
-  const cudaError_t err = launch_kernel(temb_bwd_du_kernel, g1, 256, 0, st, dgb, W_t2, a1, da1, d);
+  const cudaError_t err = launch_kernel(temb_bwd_du_kernel, dim3(d / 64, B), 32 * TD_WARPS, 0, st,
+                                        dgb, W_t2, a1, da1, d);
   if (err != cudaSuccess) return err;
   const long total = 2L * d * d + 2L * d + (long)d * 256 + d;
   return launch_kernel(temb_wgrad_kernel, (unsigned)((total + 255) / 256), 256, 0, st, dgb, u, da1,
