@@ -83,7 +83,8 @@ Dims dims_of(const pf_layer_desc& s) {
 
 // Largest split-K scratch needed by the layer's linear GEMMs (forward or
 // backward); the GEMM shapes below mirror the launch sequence.
-size_t splitk_need(const pf_layer_desc& s, const Dims& g, bool bwd) {
+size_t splitk_need(const pf_layer_desc& s, const Dims& g, bool bwd,
+                   size_t (*bytes)(int, int, int) = splitk_scratch_bytes) {
   const int d = (int)g.d, R = (int)g.R, r1 = (int)g.rows1, N1 = (int)g.N1, n2 = (int)(g.k2 * d);
   struct S3 {
     int M, N, K;
@@ -112,8 +113,18 @@ size_t splitk_need(const pf_layer_desc& s, const Dims& g, bool bwd) {
                             {T, d, q}});
   }
   size_t m = 0;
-  for (const S3& x : v) m = std::max(m, splitk_scratch_bytes(x.M, x.N, x.K));
+  for (const S3& x : v) m = std::max(m, bytes(x.M, x.N, x.K));
   return m;
+}
+
+// Split-K scratch of a backward whose other buffers take `off` bytes: what its
+// GEMMs want, except that it takes no layer past the allocation-free entry's
+// fixed scratch that fits it with the least.
+size_t splitk_bwd(const pf_layer_desc& s, const Dims& g, size_t off) {
+  const size_t want = splitk_need(s, g, true), least = splitk_need(s, g, true, splitk_scratch_least);
+  const size_t used = ((off + 255) & ~size_t(255)) + 256, all = PF_NOALLOC_SCRATCH_BYTES;
+  const size_t room = used < all ? all - used : 0;  // a multiple of 256
+  return want <= room || least > room ? want : std::min(want, room);
 }
 
 EpiLinearArgs with_sk(EpiLinearArgs e, float* sk, size_t skb) {
@@ -243,7 +254,7 @@ BwdWs carve_bwd(Carve& c, const pf_layer_desc& s, const Dims& g) {
   if (g.f == PF_F_MLP) pe = std::max(pe, colsum_part_elems(g.R, (int)(4 * g.d)));
   w.part_elems = pe;
   w.part = c.take<float>(pe);
-  w.skb = splitk_need(s, g, true);
+  w.skb = splitk_bwd(s, g, c.off);
   w.sk = c.take<float>(w.skb / sizeof(float));
   return w;
 }
@@ -297,7 +308,7 @@ Bwd2DWs carve_bwd_2d(Carve& c, const pf_layer_desc& s, const Dims& g) {
   w.part = c.take<float>(pe);
   w.dgb = c.take<float>(g.B * 2 * g.d);
   w.da1 = c.take<float>(g.B * g.d);
-  w.skb = splitk_need(s, g, true);
+  w.skb = splitk_bwd(s, g, c.off);
   w.sk = c.take<float>(w.skb / sizeof(float));
   return w;
 }

@@ -99,22 +99,75 @@ int max_pairs(Kern kern, int threads, int smem) {
   return std::min(n, num_sms() / 2);
 }
 
+// How an M x N x K product is tiled: 128- or 256-wide tiles, on CTA pairs or
+// not, K in S slices.
+struct Plan {
+  int bn = 128, S = 1;
+  bool pair = false;
+};
+
+// Cycles of a plan, from measured rates: one 64-deep K block of a 128 x 128 tile
+// takes a CTA 552 cycles, of a 128 x 256 tile 770, of a pair's 256 x 256 tile 656
+// (the pair reads half as much shared memory per MMA and its ring is deeper); a
+// wave of tiles costs about 1200 more to fill and hand over, and slices a pass of
+// S + 1 fp32 matrices at 3300 bytes a cycle after another launch.  The split
+// products of the 65536-token layer (M = N = 1024, K = 65536) take 124 + 10 us
+// on 7 slices of 128-wide tiles, 90 + 11 on 9 of a pair's; M 4096, N 1024, K 8192
+// takes 57 us on 128 single CTAs, 50 on 64 pairs.
+constexpr int kPlanSms = 152;  // planning target (GB300); fixed so sizes are device-independent
+double plan_cost(int M, int N, int K, int bn, bool pair, int S) {
+  const long tm = pair ? 2 * GEMM_BM : GEMM_BM;
+  const long tiles = ((N + bn - 1) / bn) * ((M + tm - 1) / tm) * S;
+  const long units = pair ? kPlanSms / 2 : kPlanSms, waves = (tiles + units - 1) / units;
+  const long nk = (K + GEMM_BK - 1) / GEMM_BK, kb = (nk + S - 1) / S;
+  const double c = bn == 128 ? 552. : pair ? 656. : 770.;
+  const double red = S > 1 ? 5000. + 4.0 * M * (double)N * (S + 1) / 3300. : 0.;
+  return waves * (kb * c + 1200.) + red;
+}
+
+// The cheapest plan whose slices' partial sums fit `bytes`: slices are at least
+// 16 K blocks deep and must promise a tenth, since a last wave that is partly
+// empty costs less than the model says (weight gradients of the 262144-token
+// layer, 128 pair tiles in two waves: 320 us, on four slices 321 + 33).
+Plan gemm_plan(int M, int N, int K, size_t bytes) {
+  Plan best;
+  const long nk = (K + GEMM_BK - 1) / GEMM_BK;
+  double cost = 1e300;
+  for (int v = 0; v < 3; ++v) {
+    const int bn = v == 0 ? 128 : 256;
+    const bool pair = v == 2;
+    if (v > 0 && N < 256) continue;
+    for (int S = 1; S <= 32 && (S == 1 || (nk / S >= 16 && v != 1)); ++S) {
+      if (S > 1 && (N % 4 != 0 || (size_t)S * M * N * sizeof(float) > bytes)) break;
+      const double c = plan_cost(M, N, K, bn, pair, S) * (S > 1 ? 1.0 / 0.9 : 1.0);
+      if (c < cost) {
+        cost = c;
+        best.bn = bn;
+        best.pair = pair;
+        best.S = S;
+      }
+    }
+  }
+  return best;
+}
+
 template <int BN, bool AMN, bool BMN, class Epi>
 cudaError_t launch(int M, int N, int K, const CUtensorMap& ta, const CUtensorMap& tb,
-                   const Epi& epi, cudaStream_t st, int splits) {
-  if constexpr (BN == 256) {
-    // CTA pairs (256 x 256 tiles, half of B per CTA, a deeper stage ring)
-    // when every co-resident pair gets a tile
+                   const Epi& epi, cudaStream_t st, const Plan& plan) {
+  const int splits = plan.S;
+  if constexpr (BN == 256) {  // CTA pairs: 256 x 256 tiles, half of B per CTA
     auto kern2 = gemm_tc_kernel<BN, AMN, BMN, Epi, true>;
     constexpr int smem2 = GemmCfg<BN, true, gemm_stage_bytes<Epi>(true)>::SMEM_BYTES;
-    cudaError_t e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
-    if (e != cudaSuccess) return e;
-    static const int pairs = max_pairs(kern2, GEMM_THREADS, smem2);
-    const long pair_tiles =
-        (long)((N + BN - 1) / BN) * ((M + 2 * GEMM_BM - 1) / (2 * GEMM_BM)) * splits;
-    if (pairs > 0 && pair_tiles >= pairs)
-      return launch_clusters(2, kern2, 2 * (unsigned)std::min<long>(pair_tiles, pairs),
-                             GEMM_THREADS, smem2, st, ta, tb, M, N, K, splits, epi);
+    if (plan.pair) {
+      cudaError_t e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
+      if (e != cudaSuccess) return e;
+      static const int pairs = max_pairs(kern2, GEMM_THREADS, smem2);
+      const long pair_tiles =
+          (long)((N + BN - 1) / BN) * ((M + 2 * GEMM_BM - 1) / (2 * GEMM_BM)) * splits;
+      if (pairs > 0)
+        return launch_clusters(2, kern2, 2 * (unsigned)std::min<long>(pair_tiles, pairs),
+                               GEMM_THREADS, smem2, st, ta, tb, M, N, K, splits, epi);
+    }
   }
   auto kern = gemm_tc_kernel<BN, AMN, BMN, Epi>;
   constexpr int smem = GemmCfg<BN, false, gemm_stage_bytes<Epi>(false)>::SMEM_BYTES;
@@ -126,17 +179,17 @@ cudaError_t launch(int M, int N, int K, const CUtensorMap& ta, const CUtensorMap
 }
 
 // Operand majors that the epilogue's callers use: all four for the linear
-// ones, K-major A (and one major of B) for the fused ones.
+// ones, K-major A (and for a direct one K-major B) for the fused ones.
 template <int BN, class Epi>
 cudaError_t launch_majors(int M, int N, int K, const Operand& A, const Operand& B,
                           const CUtensorMap& ta, const CUtensorMap& tb, const Epi& epi,
-                          cudaStream_t st, int splits = 1) {
-  if (!A.mn && !B.mn) return launch<BN, false, false>(M, N, K, ta, tb, epi, st, splits);
+                          cudaStream_t st, const Plan& plan) {
+  if (!A.mn && !B.mn) return launch<BN, false, false>(M, N, K, ta, tb, epi, st, plan);
   if constexpr (!Epi::kDirect)
-    if (!A.mn && B.mn) return launch<BN, false, true>(M, N, K, ta, tb, epi, st, splits);
+    if (!A.mn && B.mn) return launch<BN, false, true>(M, N, K, ta, tb, epi, st, plan);
   if constexpr (!Epi::kRows) {
-    if (A.mn && B.mn) return launch<BN, true, true>(M, N, K, ta, tb, epi, st, splits);
-    return launch<BN, true, false>(M, N, K, ta, tb, epi, st, splits);
+    if (A.mn && B.mn) return launch<BN, true, true>(M, N, K, ta, tb, epi, st, plan);
+    return launch<BN, true, false>(M, N, K, ta, tb, epi, st, plan);
   }
   return cudaErrorInvalidValue;
 }
@@ -155,18 +208,16 @@ cudaError_t gemm_dispatch(int M, int N, int K, Operand A, Operand B, const Epi& 
   if (!make_operand_map(&ta, A, M, K) ||
       !(Epi::kDirect ? make_segment_map(&tb, B, N, K) : make_operand_map(&tb, B, N, K)))
     return cudaErrorInvalidValue;
-  const long tiles256 = (long)((N + 255) / 256) * ((M + GEMM_BM - 1) / GEMM_BM);
   LaunchTimer lt(gemm_tag_label(), st, 2.0 * M * N * (double)K,
                  2.0 * ((double)M * K + (double)N * K) + gemm_tag_bytes());
-  // 128 x 256 tiles move about 2/3 of the shared-memory bytes per FLOP of
-  // 128 x 128 tiles (the mainloop's bound); take them unless they need more
-  // than 1.5x the waves
-  const long tiles128 = (long)((N + 127) / 128) * ((M + GEMM_BM - 1) / GEMM_BM);
-  const long sms = num_sms(), w256 = (tiles256 + sms - 1) / sms, w128 = (tiles128 + sms - 1) / sms;
-  if (Epi::kPaired || (N >= 256 && 3 * w256 <= 2 * w128))
-    return launch_majors<256>(M, N, K, A, B, ta, tb, epi, st);
-  if constexpr (!Epi::kPaired) return launch_majors<128>(M, N, K, A, B, ta, tb, epi, st);
-  return cudaErrorInvalidValue;
+  Plan plan = gemm_plan(M, N, K, 0);
+  if constexpr (Epi::kPaired) {
+    plan.bn = 256;
+    plan.pair = plan_cost(M, N, K, 256, true, 1) <= plan_cost(M, N, K, 256, false, 1);
+  } else if (plan.bn == 128) {
+    return launch_majors<128>(M, N, K, A, B, ta, tb, epi, st, plan);
+  }
+  return launch_majors<256>(M, N, K, A, B, ta, tb, epi, st, plan);
 }
 
 // out = sum_s part[s] (+ bias) (+ addend) -> fp32 and/or bf16, 4 columns per thread.
@@ -208,34 +259,35 @@ bool tmap_bf16_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t out
   return make_map(m, base, inner, outer, ld, box_inner, box_outer);
 }
 
-int splitk_factor(int M, int N, int K) {
-  constexpr int kSms = 152;  // planning target (GB300); fixed so sizes are device-independent
+size_t splitk_scratch_bytes(int M, int N, int K) {
+  const int S = gemm_plan(M, N, K, ~size_t(0)).S;
+  return S > 1 ? (size_t)S * M * N * sizeof(float) : 0;
+}
+
+size_t splitk_scratch_least(int M, int N, int K) {
   const long tiles = (long)((N + 127) / 128) * ((M + GEMM_BM - 1) / GEMM_BM);
   const int num_k = (K + GEMM_BK - 1) / GEMM_BK;
-  if (tiles >= kSms || num_k < 32) return 1;
+  if (tiles >= kPlanSms || num_k < 32) return 0;
   int best = 1;
-  double best_eff = (double)tiles / kSms;
+  double best_eff = (double)tiles / kPlanSms;
   for (int S = 2; S <= 16 && num_k / S >= 16; ++S) {
     const long t = tiles * S;
-    const double eff = (double)t / (((t + kSms - 1) / kSms) * kSms);
+    const double eff = (double)t / (((t + kPlanSms - 1) / kPlanSms) * kPlanSms);
     if (eff > best_eff + 1e-9) {
       best = S;
       best_eff = eff;
     }
   }
-  return best;
-}
-
-size_t splitk_scratch_bytes(int M, int N, int K) {
-  const int S = splitk_factor(M, N, K);
-  return S > 1 ? (size_t)S * M * N * sizeof(float) : 0;
+  return best > 1 ? (size_t)best * M * N * sizeof(float) : 0;
 }
 
 cudaError_t gemm_linear(int M, int N, int K, Operand A, Operand B, const EpiLinearArgs& e,
                         cudaStream_t st) {
-  const int S = splitk_factor(M, N, K);
-  if (S > 1 && e.splitk_scratch && (size_t)S * M * N * sizeof(float) <= e.splitk_bytes &&
-      N % 4 == 0 && !e.act_silu && !e.pre_bf16 && !e.dsilu_of) {
+  Plan plan;
+  if (e.splitk_scratch && !e.act_silu && !e.pre_bf16 && !e.dsilu_of)
+    plan = gemm_plan(M, N, K, e.splitk_bytes);
+  const int S = plan.S;
+  if (S > 1) {
     // deterministic split-K: raw partials, then one reduce applying the epilogue
     if (M <= 0 || N % 32 != 0 || !operand_ok(A) || !operand_ok(B)) return cudaErrorInvalidValue;
     CUtensorMap ta, tb;
@@ -245,7 +297,9 @@ cudaError_t gemm_linear(int M, int N, int K, Operand A, Operand B, const EpiLine
     {
       LaunchTimer lt(gemm_tag_label(), st, 2.0 * M * N * (double)K,
                      2.0 * ((double)M * K + (double)N * K) + 4.0 * S * M * N);
-      cudaError_t err = launch_majors<128>(M, N, K, A, B, ta, tb, epi, st, S);
+      const cudaError_t err =
+          plan.bn == 256 ? launch_majors<256>(M, N, K, A, B, ta, tb, epi, st, plan)
+                         : launch_majors<128>(M, N, K, A, B, ta, tb, epi, st, plan);
       if (err != cudaSuccess) return err;
     }
     LaunchTimer lt("splitk_reduce", st, (double)S * M * N, 4.0 * (S + 1.0) * M * N);

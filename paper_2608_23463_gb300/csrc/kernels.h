@@ -71,10 +71,11 @@ struct EpiLinearArgs {
   float* splitk_scratch = nullptr;
   size_t splitk_bytes = 0;
 };
-// Split-K factor chosen for an M x N x K linear GEMM (1: none) and the fp32
-// scratch it needs; independent of the device.
-int splitk_factor(int M, int N, int K);
+// fp32 scratch of an M x N x K linear GEMM's split-K (0: it is not split) at the
+// tiling it takes when given enough, and the least that a caller short of memory
+// should give (it splits as far as that goes); independent of the device.
 size_t splitk_scratch_bytes(int M, int N, int K);
+size_t splitk_scratch_least(int M, int N, int K);
 
 struct EpiInjectArgs {
   const float* bias;  // b_d1 [k1*d]

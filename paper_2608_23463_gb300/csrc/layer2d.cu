@@ -20,10 +20,11 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 
 // One pass over the tokens of the 2D layer, PG_T consecutive tokens t = (b, y, x)
 // per warp, their rows loaded together (one at a time left too little in flight:
-// 376 us for four 512 x 512 images at d = 512, 334 so, 6.5 TB/s): the patch copy Xp[r, (py*p + px)*d + ch] = X[t, ch] for
-// patch r = (b, by, bx) (Eq. partition, the compression GEMM's operand) and the
-// token's LayerNorm statistics stats[t] = (mean, 1/sqrt(var + 1e-6)) (Eq.
-// inj-affine), from registers (two passes over the row).  d <= 512.
+// 376 us for four 512 x 512 images at d = 512, 334 so, 6.5 TB/s): the patch copy
+// Xp[r, (py*p + px)*d + ch] = X[t, ch] for patch r = (b, by, bx) (Eq. partition,
+// the compression GEMM's operand) and the token's LayerNorm statistics stats[t]
+// = (mean, 1/sqrt(var + 1e-6)) (Eq. inj-affine), from registers (two passes over
+// the row).  d <= 512.
 constexpr int PG_T = 4;
 __global__ void __launch_bounds__(256) patch_gather_stats_kernel(
     const bf16* __restrict__ X, bf16* __restrict__ Xp, float* __restrict__ stats, long T, int d,

@@ -1,0 +1,64 @@
+"""Split contractions: weight gradients and compressions whose output is a few
+tiles and whose K is long run in K slices on CTA pairs or single CTAs, with as
+many slices as the scratch that the caller gives allows.  A layer's weight
+gradients and proxies must not depend on that beyond the order of fp32 sums."""
+import pytest
+import torch
+
+import paper_2608_23463_gb300 as pf
+import pf_synth as S
+from oracle import layer as OL
+from paper_2608_23463_gb300.layer import ProxyLayer, to_device
+from tests._util import assert_close, assert_grad_close
+
+pytestmark = pytest.mark.gpu
+
+# K = P d for the compression (M = L / P rows), K = L / k1 for the weight gradients
+SPECS = {
+    # M = 47 rows x N = 192: single CTAs, ragged N tile; K = 24576
+    "few_rows": S.LayerSpec(batch=1, L=47 * 128, d=192, n_heads=3, P=128),
+    # pairs with a ragged M tile (300 rows), K = 32768 for the compression
+    "pairs_ragged_m": S.LayerSpec(batch=1, L=300 * 64, d=512, n_heads=8, P=64),
+    # long K (rows) for the weight gradients, the last K block partly filled
+    "long_k": S.LayerSpec(batch=3, L=8191, d=256, n_heads=4, P=4, levels=2, k1=2, k2=2),
+}
+
+
+@pytest.mark.parametrize("name", list(SPECS))
+def test_split_contractions(name):
+    spec = SPECS[name]
+    inp = S.make_layer_inputs(spec, 90 + len(name))
+    lay = ProxyLayer(spec, inp)
+    X, G = to_device(inp["X"], torch.bfloat16), to_device(inp["G"], torch.bfloat16)
+    H = lay.empty_proxy()
+    Xo = lay.forward(X, H_out=H)
+    dX = lay.backward(X, G)
+    pf.pf_sync_check(torch.cuda.current_stream().cuda_stream)
+    ref, rH = OL.layer_fwd(spec, inp, inp["X"])
+    rdX, _, rg = OL.layer_bwd(spec, inp, inp["X"], inp["G"])
+    assert_close("H_out", H.cpu().numpy(), rH)
+    assert_grad_close("X_out", Xo.float().cpu().numpy(), ref)
+    assert_grad_close("dX", dX.float().cpu().numpy(), rdX)
+    for k, v in rg.items():
+        assert_grad_close("grad " + k, lay.grads[k].cpu().numpy(), v)
+
+
+@pytest.mark.parametrize("L,P,d", [(1000, 16, 128), (4000, 16, 64), (900, 8, 192), (300, 64, 256)])
+def test_small_layers_still_fit_the_fixed_scratch(L, P, d):
+    """The split scratch of a backward gives way to the allocation-free entry's limit."""
+    spec = S.LayerSpec(batch=2, L=L, d=d, n_heads=d // 64, P=P)
+    need = pf.proxy_layer_workspace_size(pf.layer_desc(spec), 1)
+    assert need <= pf.PF_NOALLOC_SCRATCH_BYTES
+    inp = S.make_layer_inputs(spec, 5)
+    lay = ProxyLayer(spec, inp)
+    X, G = to_device(inp["X"], torch.bfloat16), to_device(inp["G"], torch.bfloat16)
+    st = torch.cuda.current_stream().cuda_stream
+    lay.forward(X)
+    dX = lay.backward(X, G)
+    ref = {k: v.clone() for k, v in lay.grads.items()}
+    dX2 = torch.empty_like(dX)
+    pf.proxy_layer_bwd_noalloc(lay.desc, lay.p_struct, X, None, None, lay.saved, G, None, dX2, None,
+                               lay.g_struct, st)
+    pf.pf_sync_check(st)
+    assert torch.equal(dX, dX2)
+    assert all(torch.equal(ref[k], lay.grads[k]) for k in ref)
