@@ -5,21 +5,30 @@
 //   dQ = dS K / 8.
 // Two kernels share one skeleton (no atomics, deterministic):
 //   DKDV: item = (128-key tile, head, sequence); stationary X1 = K, X2 = V;
-//         streamed 64-query tiles Y1 = Q_j, Y2 = dO_j.
-//           T1 = X1 Y1^T = S^T,  T2 = X2 Y2^T = dP^T     (TMEM, M=128 N=64)
+//         streamed 128-query tiles Y1 = Q_j, Y2 = dO_j.
+//           T1 = X1 Y1^T = S^T,  T2 = X2 Y2^T = dP^T     (TMEM, M=128 N=128)
 //           E1 = P^T, E2 = dS^T  (bf16, written to TMEM by the row warps)
 //           dV += E1 Y2,  dK += E2 Y1    (A from TMEM; TMEM accumulators)
 //   DQ:   item = (128-query tile, head, sequence); stationary X1 = Q, X2 = dO;
-//         streamed 64-key tiles Y1 = K_j, Y2 = V_j.
+//         streamed 128-key tiles Y1 = K_j, Y2 = V_j.
 //           T1 = S,  T2 = dP,  E2 = dS,  dQ += E2 Y1
 // Roles: warp 0 TMA producer (DKDV: it also stages each step's (LSE, Di)
 // pairs of the streamed queries in shared memory), warp 1 MMA issuer, warps
-// 2-9 the row warps: two per TMEM lane quarter, each thread one row (TMEM
-// lane) and one half of the 64 streamed columns.  T1/T2 and E are double-buffered so the MMAs of step
-// j+1 overlap the row work of step j.  E stays in TMEM as the A operand of the
-// accumulating MMAs, so those read only their B tile from shared memory
-// (shared-memory bandwidth, not the tensor pipe, bounds M=128 N=64 MMAs whose
-// operands both come from shared memory).  Every wait is bounded.
+// 2-17 the row warps: four per TMEM lane quarter, each thread one row (TMEM
+// lane) and one quarter of the 128 streamed columns.  A thread takes its 32
+// scores and 32 dP into registers first and frees T1/T2, so the score MMAs of
+// step j+1 and the accumulating MMAs of step j-1 run while it works on step j:
+// the tensor pipe always has one or the other.  E stays in TMEM as the A operand
+// of the accumulating MMAs, so those read only their B tile from shared memory.
+// Every wait is bounded.
+// What bounds it and why 128 streamed columns a step: an M=128 K=16 MMA takes
+// ~107 cycles at N=128 and hardly less at N=64, and the hand-offs of a step
+// (barriers, TMEM round trips) cost the same.  Steps of 64 with T and E double-
+// buffered took 1620 (DKDV) and 1475 (DQ) cycles each, steps of 128 take 2550 and
+// 1690, about the time of their 24 and 16 MMAs.  16384 proxies of 8 heads, causal:
+// 706 -> 555 and 642 -> 367 us; 131072 tokens against 2048 proxies, 16 heads: 1676
+// -> 1341 and 1380 -> 896.  With eight row warps (64 columns a thread) DKDV takes
+// 572 and DQ 367; scalar instead of packed arithmetic there 556 and 408.
 //
 // The cross-attention of the injection (Eq. inj-cross) runs on the same
 // kernels: queries are tokens, keys / values proxies (separate matrices, Lq
@@ -36,20 +45,19 @@ namespace pf {
 namespace {
 
 constexpr int BW_M = 128;  // stationary rows (TMEM lanes)
-constexpr int BW_N = 64;   // streamed rows per step
+constexpr int BW_N = 128;  // streamed rows per step
 constexpr int BW_D = 64;   // head width
 constexpr int BW_STAGES = 4;
-constexpr int BW_ROW_THREADS = 256;  // warps 2-9
+constexpr int BW_ROW_THREADS = 512;  // warps 2-17
 constexpr int BW_THREADS = 64 + BW_ROW_THREADS;
 constexpr uint32_t BW_X_BYTES = BW_M * BW_D * 2;  // 16 KB per stationary tile
-constexpr uint32_t BW_Y_BYTES = BW_N * BW_D * 2;  // 8 KB per streamed tile
+constexpr uint32_t BW_Y_BYTES = BW_N * BW_D * 2;  // 16 KB per streamed tile
 constexpr uint32_t BW_OFF_Y = 2 * 2 * BW_X_BYTES;                       // X: [2 bufs][X1, X2]
 constexpr uint32_t BW_OFF_LD = BW_OFF_Y + BW_STAGES * 2 * BW_Y_BYTES;  // Y: [stage][Y1, Y2]
-constexpr uint32_t BW_OFF_BAR = BW_OFF_LD + BW_STAGES * BW_N * 8;      // (lse, Di) [stage][64]
+constexpr uint32_t BW_OFF_BAR = BW_OFF_LD + BW_STAGES * BW_N * 8;      // (lse, Di) [stage][128]
 constexpr uint32_t BW_SMEM = BW_OFF_BAR + 256 + 1024;
-// TMEM columns: T1 at 0 / 64, T2 at 128 / 192 (fp32, per buffer), accumulators
-// at 256 (dV or dQ) and 320 (dK), E at 384 / 448 (per buffer: E1 at +0, E2 at
-// +32, bf16 pairs: streamed column c in 32-bit column c / 2)
+// TMEM columns: T1 at 0, T2 at 128 (fp32), accumulators at 256 (dV or dQ) and 320
+// (dK), E1 at 384, E2 at 448 (bf16 pairs: streamed column c in 32-bit column c / 2)
 constexpr uint32_t BW_TMEM_COLS = 512;
 constexpr uint32_t BW_TM_E = 384;
 
@@ -119,12 +127,12 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   const uint32_t b0 = smem_u32(smem + BW_OFF_BAR);
-  // x_full[2] x_empty[2] y_full[S] y_empty[S] t_full[2] t_free[2] e_full[2] e_free[2]
-  // acc_full acc_free done
+  // x_full[2] x_empty[2] y_full[S] y_empty[S] t_full t_free e_full e_free acc_full
+  // acc_free done
   const uint32_t x_full = b0, x_empty = b0 + 16, y_full = b0 + 32,
                  y_empty = y_full + 8 * BW_STAGES, t_full = y_empty + 8 * BW_STAGES,
-                 t_free = t_full + 16, e_full = t_free + 16, e_free = e_full + 16,
-                 acc_full = e_free + 16, acc_free = acc_full + 8, done = acc_free + 8;
+                 t_free = t_full + 8, e_full = t_free + 8, e_free = e_full + 8,
+                 acc_full = e_free + 8, acc_free = acc_full + 8, done = acc_free + 8;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + BW_OFF_BAR + 240);
   const uint32_t sbase = smem_u32(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -133,11 +141,11 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
     for (int i = 0; i < 2; ++i) {
       mbar_init(x_full + 8 * i, 1);
       mbar_init(x_empty + 8 * i, 1);
-      mbar_init(t_full + 8 * i, 1);
-      mbar_init(t_free + 8 * i, BW_ROW_THREADS / 32);  // one arrival per row warp
-      mbar_init(e_full + 8 * i, BW_ROW_THREADS / 32);
-      mbar_init(e_free + 8 * i, 1);
     }
+    mbar_init(t_full, 1);
+    mbar_init(t_free, BW_ROW_THREADS / 32);  // one arrival per row warp
+    mbar_init(e_full, BW_ROW_THREADS / 32);
+    mbar_init(e_free, 1);
     for (int i = 0; i < BW_STAGES; ++i) {
       mbar_init(y_full + 8 * i, 1);
       mbar_init(y_empty + 8 * i, 1);
@@ -161,10 +169,10 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     // Lane 0 issues the copies.  DKDV: the whole warp also stages the (lse,
-    // Di) pairs of each step's 64 streamed queries in the stage's slot before
+    // Di) pairs of each step's 128 streamed queries in the stage's slot before
     // lane 0 arms the stage's full barrier, so that the row warps read them
     // after that barrier (the values for the next step are loaded one step
-    // ahead, two queries per lane).
+    // ahead, four queries per lane).
     if (lane == 0) {
       prefetch_tmap(&tmX1);
       prefetch_tmap(&tmX2);
@@ -178,13 +186,16 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
       const long o = ((long)b * a.nh + h) * a.Lq + qq;
       return make_float2(a.lse[o], a.Di[o]);
     };
-    float2 ld0 = make_float2(0.f, 0.f), ld1 = ld0;  // next step's pairs of queries lane, lane + 32
+    float2 ldp[BW_N / 32];  // next step's pairs of queries lane + 32 i
+    auto fetch_step = [&](int b, int h, int q0) {
+#pragma unroll
+      for (int i = 0; i < BW_N / 32; ++i) ldp[i] = fetch_ld(b, h, q0, lane + 32 * i);
+    };
     int k = bw_rank(blockIdx.x, 0);
     if (DKDV && k < a.n_items) {
       int t, h, b, j0, n;
       bw_item<DKDV>(a, k, t, h, b, j0, n);
-      ld0 = fetch_ld(b, h, j0 * BW_N, lane);
-      ld1 = fetch_ld(b, h, j0 * BW_N, lane + 32);
+      fetch_step(b, h, j0 * BW_N);
     }
     bool ok = true;
     uint32_t it = 0;
@@ -208,8 +219,8 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
           break;
         }
         if (DKDV) {
-          ld_ring[st * BW_N + lane] = ld0;
-          ld_ring[st * BW_N + 32 + lane] = ld1;
+#pragma unroll
+          for (int i = 0; i < BW_N / 32; ++i) ld_ring[st * BW_N + 32 * i + lane] = ldp[i];
           __syncwarp();
         }
         if (lane == 0) {
@@ -222,15 +233,13 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
         y_issued = G + 1;
         if (DKDV) {  // the pairs of the next step (this item's or the next item's first)
           if (j + 1 < n) {
-            ld0 = fetch_ld(b, h, (j0 + j + 1) * BW_N, lane);
-            ld1 = fetch_ld(b, h, (j0 + j + 1) * BW_N, lane + 32);
+            fetch_step(b, h, (j0 + j + 1) * BW_N);
           } else {
             const int k2 = bw_rank(blockIdx.x, rd + 1);
             if (k2 < a.n_items) {
               int t2, h2, b2, j02, n2;
               bw_item<DKDV>(a, k2, t2, h2, b2, j02, n2);
-              ld0 = fetch_ld(b2, h2, j02 * BW_N, lane);
-              ld1 = fetch_ld(b2, h2, j02 * BW_N, lane + 32);
+              fetch_step(b2, h2, j02 * BW_N);
             }
           }
         }
@@ -245,11 +254,11 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
     uint32_t it = 0, G = 0;
     // accumulate step G (local step j of its item): E_G times the step's Y tiles
     auto acc_step = [&](uint32_t G_, int j, uint32_t it_) -> bool {
-      const uint32_t eb = G_ & 1, st = G_ % BW_STAGES;
-      if (!mbar_wait_warp(e_full + 8 * eb, (G_ >> 1) & 1)) return false;
+      const uint32_t st = G_ % BW_STAGES;
+      if (!mbar_wait_warp(e_full, G_ & 1)) return false;
       if (j == 0 && !mbar_wait_warp(acc_free, (it_ & 1) ^ 1)) return false;
       tc_fence_after();
-      const uint32_t e1 = tmem + BW_TM_E + eb * 64, e2 = e1 + 32;
+      const uint32_t e1 = tmem + BW_TM_E, e2 = e1 + BW_N / 2;
       const uint32_t y1 = sbase + BW_OFF_Y + st * 2 * BW_Y_BYTES, y2 = y1 + BW_Y_BYTES;
       if (elect_one()) {
 #pragma unroll
@@ -264,7 +273,7 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
             tc_mma_f16_ts(tmem + 256, e2 + kk * 8, bd1, idesc_a, acc);  // dQ += dS K
           }
         }
-        tc_commit(e_free + 8 * eb);
+        tc_commit(e_free);
         tc_commit(y_empty + 8 * st);
       }
       __syncwarp();
@@ -279,9 +288,9 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
       tc_fence_after();
       const uint32_t x1 = sbase + xb * 2 * BW_X_BYTES, x2 = x1 + BW_X_BYTES;
       for (int j = 0; j < n; ++j) {
-        const uint32_t Gj = G + j, st = Gj % BW_STAGES, tb = Gj & 1;
+        const uint32_t Gj = G + j, st = Gj % BW_STAGES;
         if (!mbar_wait_warp(y_full + 8 * st, (Gj / BW_STAGES) & 1) ||
-            !mbar_wait_warp(t_free + 8 * tb, ((Gj >> 1) & 1) ^ 1)) {
+            !mbar_wait_warp(t_free, (Gj & 1) ^ 1)) {
           ok = false;
           break;
         }
@@ -290,12 +299,12 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < BW_D / 16; ++kk) {
-            tc_mma_f16(tmem + tb * BW_N, smem_desc_sw128(x1 + kk * 32, 16, 1024),
+            tc_mma_f16(tmem, smem_desc_sw128(x1 + kk * 32, 16, 1024),
                        smem_desc_sw128(y1 + kk * 32, 16, 1024), idesc_t, kk ? 1u : 0u);
-            tc_mma_f16(tmem + 128 + tb * BW_N, smem_desc_sw128(x2 + kk * 32, 16, 1024),
+            tc_mma_f16(tmem + BW_N, smem_desc_sw128(x2 + kk * 32, 16, 1024),
                        smem_desc_sw128(y2 + kk * 32, 16, 1024), idesc_t, kk ? 1u : 0u);
           }
-          tc_commit(t_full + 8 * tb);
+          tc_commit(t_full);
           if (j == n - 1) tc_commit(x_empty + 8 * xb);
         }
         __syncwarp();
@@ -315,9 +324,9 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
     // ------------------------------------------------------------ row warps
     const int q4 = warp & 3;
     const int r = q4 * 32 + lane;  // stationary row in the tile = TMEM lane
-    const int ch = (warp - 2) >> 2;   // half of the streamed columns: [32 ch, 32 ch + 32)
+    const int ch = (warp - 2) >> 2;   // quarter of the streamed columns: [32 ch, 32 ch + 32)
     const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16);
-    const float2* ld_ring = reinterpret_cast<const float2*>(smem + BW_OFF_LD);  // [stage][64]
+    const float2* ld_ring = reinterpret_cast<const float2*>(smem + BW_OFF_LD);  // [stage][128]
     bool ok = true;
     uint32_t G = 0, it = 0;
     for (int rd = 0, k = bw_rank(blockIdx.x, 0); k < a.n_items && ok;
@@ -332,7 +341,7 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
         di_r = a.Di[o];
       }
       for (int j = 0; j < n; ++j) {
-        const uint32_t Gj = G + j, tb = Gj & 1;
+        const uint32_t Gj = G + j;
         const int c0 = (j0 + j) * BW_N;  // first streamed index of this step
         // DKDV: the step's (lse, Di) pairs, staged by the producer before the
         // stage's full barrier (already complete: the step's scores used it;
@@ -341,113 +350,101 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
           ok = false;
           break;
         }
-        if (!mbar_wait(t_full + 8 * tb, (Gj >> 1) & 1)) {
+        if (!mbar_wait(t_full, Gj & 1)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        uint32_t s1[32], p1[32];
-        tmem_ld32_async(tl + tb * BW_N + 32 * ch, s1);
-        tmem_ld32_async(tl + 128 + tb * BW_N + 32 * ch, p1);
-        tmem_wait_ld(s1);
-        tmem_wait_ld(p1);
+        uint32_t sa[32], pa[32];  // this thread's 32 columns of T1 and T2
+        tmem_ld32_async(tl + 32 * ch, sa);
+        tmem_ld32_async(tl + BW_N + 32 * ch, pa);
+        tmem_wait_ld(sa);
+        tmem_wait_ld(pa);
         tc_fence_before();
-        mbar_arrive_warp(t_free + 8 * tb);
+        mbar_arrive_warp(t_free);
         // valid streamed columns: [lo, hi)
         int lo = 0, hi = min(BW_N, a.Ly - c0);
         if (DKDV)
           lo = max(0, bw_first_q(a, row) - c0);  // the queries that see this key
         else
           hi = min(hi, bw_vis(a, row) - c0);  // the keys this query sees
-        if (!mbar_wait(e_free + 8 * tb, ((Gj >> 1) & 1) ^ 1)) {
-          ok = false;
-          break;
-        }
         const float2* lds = ld_ring + (Gj % BW_STAGES) * BW_N;
-        uint32_t pk[16], dk[16];  // this thread's 32 columns of E1 and E2, bf16 pairs
-        // P and dS of this thread's 32 columns; columns outside [lo, hi) are
-        // masked (only the diagonal and tail steps have any)
-        auto emit = [&](auto masked) {
+        // P and dS of 32 columns from kb on, as bf16 pairs; columns outside [lo, hi)
+        // are masked (only the diagonal and tail steps have any)
+        auto emit = [&](auto masked, const uint32_t* s1, const uint32_t* p1, int kb, uint32_t* pk,
+                        uint32_t* dk) {
 #pragma unroll
           for (int g = 0; g < 4; ++g) {
-            const int kg = 4 * ch + g;  // 8-column group in the 64-wide row
             const uint32_t* sv = s1 + g * 8;
             const uint32_t* dv = p1 + g * 8;
-            float pe[8], de[8];
-            // DKDV: the group's (lse, Di) with 128-bit shared loads, two columns
-            // each (the compiler cannot prove the alignment of the float2 array)
-            float l8[8], d8[8];
-            if (DKDV) {
-              const float4* l4 = reinterpret_cast<const float4*>(lds) + kg * 4;
-#pragma unroll
-              for (int e2 = 0; e2 < 4; ++e2) {
-                const float4 v = l4[e2];
-                l8[2 * e2] = v.x;
-                d8[2 * e2] = v.y;
-                l8[2 * e2 + 1] = v.z;
-                d8[2 * e2 + 1] = v.w;
-              }
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int c = kg * 8 + e;
-              const float l2 = DKDV ? l8[e] : lse_r, dd = DKDV ? d8[e] : di_r;
-              float p = ex2_approx(fmaf(__uint_as_float(sv[e]), a.sl2, -l2));
-              if (decltype(masked)::value && (c < lo || c >= hi)) p = 0.f;
-              pe[e] = p;
-              de[e] = p * (__uint_as_float(dv[e]) - dd);
-            }
+            // (lse, Di) of two columns per 128-bit shared load (DKDV); packed fp32x2
+            // arithmetic on column pairs (each lane an IEEE fp32 operation)
+            const float4* l4 = reinterpret_cast<const float4*>(lds + kb) + g * 4;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              pk[4 * g + e] = pack_bf16(pe[2 * e], pe[2 * e + 1]);
-              dk[4 * g + e] = pack_bf16(de[2 * e], de[2 * e + 1]);
+              const int c = kb + g * 8 + 2 * e;
+              float2 nl = make_float2(-lse_r, -lse_r), nd = make_float2(-di_r, -di_r);
+              if (DKDV) {
+                const float4 v = l4[e];
+                nl = make_float2(-v.x, -v.z);
+                nd = make_float2(-v.y, -v.w);
+              }
+              const float2 z = __ffma2_rn(
+                  make_float2(__uint_as_float(sv[2 * e]), __uint_as_float(sv[2 * e + 1])),
+                  make_float2(a.sl2, a.sl2), nl);
+              float2 p = make_float2(ex2_approx(z.x), ex2_approx(z.y));
+              if (decltype(masked)::value) {
+                if (c < lo || c >= hi) p.x = 0.f;
+                if (c + 1 < lo || c + 1 >= hi) p.y = 0.f;
+              }
+              const float2 ds = __fmul2_rn(
+                  p, __fadd2_rn(make_float2(__uint_as_float(dv[2 * e]), __uint_as_float(dv[2 * e + 1])),
+                                nd));
+              pk[4 * g + e] = pack_bf16(p.x, p.y);
+              dk[4 * g + e] = pack_bf16(ds.x, ds.y);
             }
           }
         };
+        uint32_t pk[16], dk[16];  // this thread's 32 columns of E1 and E2
         if (lo <= 32 * ch && hi >= 32 * ch + 32)
-          emit(std::false_type{});
+          emit(std::false_type{}, sa, pa, 32 * ch, pk, dk);
         else
-          emit(std::true_type{});
-        const uint32_t te = tl + BW_TM_E + tb * 64 + 16 * ch;
+          emit(std::true_type{}, sa, pa, 32 * ch, pk, dk);
+        if (!mbar_wait(e_free, (Gj & 1) ^ 1)) {  // the previous step's E has been read
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t te = tl + BW_TM_E + 16 * ch;
         if (DKDV) tmem_st16(te, pk);
-        tmem_st16(te + 32, dk);
+        tmem_st16(te + BW_N / 2, dk);
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive_warp(e_full + 8 * tb);
+        mbar_arrive_warp(e_full);
       }
       if (!ok) break;
       G += n;
       // accumulators -> dK, dV (DKDV) or dQ (DQ) rows
       if (!mbar_wait(acc_full, it & 1)) break;
       tc_fence_after();
-      uint32_t u0[32], w0[32];  // this thread's 32 columns of dV / dQ and of dK
-      tmem_ld32_async(tl + 256 + 32 * ch, u0);
-      if (DKDV) tmem_ld32_async(tl + 320 + 32 * ch, w0);
-      tmem_wait_ld(u0);
-      if (DKDV) tmem_wait_ld(w0);
+      uint32_t u0[16], w0[16];  // this thread's 16 columns of dV / dQ and of dK
+      tmem_ld16(tl + 256 + 16 * ch, u0);
+      if (DKDV) tmem_ld16(tl + 320 + 16 * ch, w0);
       tc_fence_before();
       mbar_arrive_warp(acc_free);
       if (row < a.Lx) {
         const long srow = (long)b * a.Lx + row;
-        bf16* pu = a.out_u + srow * a.ld_u + a.col_u + h * BW_D + 32 * ch;
-        const float su = DKDV ? 1.f : a.scale;
+        auto store = [&](bf16* o, const uint32_t* v, float sc) {
 #pragma unroll
-        for (int i = 0; i < 32; i += 8)
-          *reinterpret_cast<uint4*>(pu + i) = make_uint4(
-              pack_bf16(__uint_as_float(u0[i]) * su, __uint_as_float(u0[i + 1]) * su),
-              pack_bf16(__uint_as_float(u0[i + 2]) * su, __uint_as_float(u0[i + 3]) * su),
-              pack_bf16(__uint_as_float(u0[i + 4]) * su, __uint_as_float(u0[i + 5]) * su),
-              pack_bf16(__uint_as_float(u0[i + 6]) * su, __uint_as_float(u0[i + 7]) * su));
-        if (DKDV) {
-          bf16* pw = a.out_w + srow * a.ld_w + a.col_w + h * BW_D + 32 * ch;
-#pragma unroll
-          for (int i = 0; i < 32; i += 8)
-            *reinterpret_cast<uint4*>(pw + i) = make_uint4(
-                pack_bf16(__uint_as_float(w0[i]) * a.scale, __uint_as_float(w0[i + 1]) * a.scale),
-                pack_bf16(__uint_as_float(w0[i + 2]) * a.scale, __uint_as_float(w0[i + 3]) * a.scale),
-                pack_bf16(__uint_as_float(w0[i + 4]) * a.scale, __uint_as_float(w0[i + 5]) * a.scale),
-                pack_bf16(__uint_as_float(w0[i + 6]) * a.scale, __uint_as_float(w0[i + 7]) * a.scale));
-        }
+          for (int i = 0; i < 16; i += 8)
+            *reinterpret_cast<uint4*>(o + i) = make_uint4(
+                pack_bf16(__uint_as_float(v[i]) * sc, __uint_as_float(v[i + 1]) * sc),
+                pack_bf16(__uint_as_float(v[i + 2]) * sc, __uint_as_float(v[i + 3]) * sc),
+                pack_bf16(__uint_as_float(v[i + 4]) * sc, __uint_as_float(v[i + 5]) * sc),
+                pack_bf16(__uint_as_float(v[i + 6]) * sc, __uint_as_float(v[i + 7]) * sc));
+        };
+        store(a.out_u + srow * a.ld_u + a.col_u + h * BW_D + 16 * ch, u0, DKDV ? 1.f : a.scale);
+        if (DKDV) store(a.out_w + srow * a.ld_w + a.col_w + h * BW_D + 16 * ch, w0, a.scale);
       }
     }
   }
@@ -527,11 +524,10 @@ cudaError_t attn_bwd_tc(const bf16* qkv, const bf16* dO, const float* lse, const
   if (d != nh * BW_D || ((uintptr_t)qkv & 15) || ((uintptr_t)dO & 15) || ((uintptr_t)dqkv & 15))
     return cudaErrorInvalidValue;
   const uint64_t rows = (uint64_t)B * m;
-  CUtensorMap qkv128, qkv64, do128, do64;
-  if (!tmap_bf16_2d(&qkv128, qkv, 3ull * d, rows, 3ull * d, 64, BW_M) ||
-      !tmap_bf16_2d(&qkv64, qkv, 3ull * d, rows, 3ull * d, 64, BW_N) ||
-      !tmap_bf16_2d(&do128, dO, (uint64_t)d, rows, (uint64_t)d, 64, BW_M) ||
-      !tmap_bf16_2d(&do64, dO, (uint64_t)d, rows, (uint64_t)d, 64, BW_N))
+  static_assert(BW_M == BW_N, "one tensor map serves stationary and streamed tiles");
+  CUtensorMap tqkv, tdo;
+  if (!tmap_bf16_2d(&tqkv, qkv, 3ull * d, rows, 3ull * d, 64, BW_M) ||
+      !tmap_bf16_2d(&tdo, dO, (uint64_t)d, rows, (uint64_t)d, 64, BW_M))
     return cudaErrorInvalidValue;
   BwArgs a{};
   a.lse = lse;
@@ -546,15 +542,15 @@ cudaError_t attn_bwd_tc(const bf16* qkv, const bf16* dO, const float* lse, const
   a.ld_u = a.ld_w = 3L * d;
   const double pairs = (double)B * nh * (causal ? 0.5 * m * (m + 1.0) : (double)m * m);
   cudaError_t e;
-  // DKDV: X1 = K, X2 = V (128 rows); Y1 = Q, Y2 = dO (64 rows); u = dV, w = dK
+  // DKDV: X1 = K, X2 = V; Y1 = Q, Y2 = dO; u = dV, w = dK
   a.col_u = 2 * d;
   a.col_w = d;
-  if ((e = bw_launch<true>(qkv128, qkv128, qkv64, do64, d, 2 * d, 0, 0, a, "attn_bwd_dkdv",
+  if ((e = bw_launch<true>(tqkv, tqkv, tqkv, tdo, d, 2 * d, 0, 0, a, "attn_bwd_dkdv",
                            8.0 * BW_D * pairs, 2.0 * B * m * (5.0 * d), st)) != cudaSuccess)
     return e;
-  // DQ: X1 = Q, X2 = dO (128 rows); Y1 = K, Y2 = V (64 rows); u = dQ
+  // DQ: X1 = Q, X2 = dO; Y1 = K, Y2 = V; u = dQ
   a.col_u = 0;
-  return bw_launch<false>(qkv128, do128, qkv64, qkv64, 0, 0, d, 2 * d, a, "attn_bwd_dq",
+  return bw_launch<false>(tqkv, tdo, tqkv, tqkv, 0, 0, d, 2 * d, a, "attn_bwd_dq",
                           6.0 * BW_D * pairs, 2.0 * B * m * (4.0 * d), st);
 }
 
@@ -565,13 +561,10 @@ cudaError_t attn_cross_bwd(const bf16* qa, long ldq, const bf16* kv, const bf16*
       ((uintptr_t)dO & 15) || ((uintptr_t)dqa & 15) || ((uintptr_t)dkv & 15) || (ldq * 2) % 16)
     return cudaErrorInvalidValue;
   const uint64_t rq = (uint64_t)B * Lq, rk = (uint64_t)B * Lk;
-  CUtensorMap qa128, qa64, kv128, kv64, do128, do64;
-  if (!tmap_bf16_2d(&qa128, qa, (uint64_t)ldq, rq, (uint64_t)ldq, 64, BW_M) ||
-      !tmap_bf16_2d(&qa64, qa, (uint64_t)ldq, rq, (uint64_t)ldq, 64, BW_N) ||
-      !tmap_bf16_2d(&kv128, kv, 2ull * d, rk, 2ull * d, 64, BW_M) ||
-      !tmap_bf16_2d(&kv64, kv, 2ull * d, rk, 2ull * d, 64, BW_N) ||
-      !tmap_bf16_2d(&do128, dO, (uint64_t)d, rq, (uint64_t)d, 64, BW_M) ||
-      !tmap_bf16_2d(&do64, dO, (uint64_t)d, rq, (uint64_t)d, 64, BW_N))
+  CUtensorMap tqa, tkv, tdo;
+  if (!tmap_bf16_2d(&tqa, qa, (uint64_t)ldq, rq, (uint64_t)ldq, 64, BW_M) ||
+      !tmap_bf16_2d(&tkv, kv, 2ull * d, rk, 2ull * d, 64, BW_M) ||
+      !tmap_bf16_2d(&tdo, dO, (uint64_t)d, rq, (uint64_t)d, 64, BW_M))
     return cudaErrorInvalidValue;
   BwArgs a{};
   a.lse = lse;
@@ -591,22 +584,22 @@ cudaError_t attn_cross_bwd(const bf16* qa, long ldq, const bf16* kv, const bf16*
   }
   pairs *= (double)B * nh;
   cudaError_t e;
-  // DKDV: X1 = K, X2 = V (proxies, 128 rows); Y1 = Q, Y2 = dO (tokens, 64 rows);
+  // DKDV: X1 = K, X2 = V (proxies); Y1 = Q, Y2 = dO (tokens);
   // u = dV (dkv columns [d, 2d)), w = dK (columns [0, d))
   a.out_u = a.out_w = dkv;
   a.ld_u = a.ld_w = 2L * d;
   a.col_u = d;
   a.col_w = 0;
-  if ((e = bw_launch<true>(kv128, kv128, qa64, do64, 0, d, 0, 0, a, "attn_cross_bwd_dkdv",
+  if ((e = bw_launch<true>(tkv, tkv, tqa, tdo, 0, d, 0, 0, a, "attn_cross_bwd_dkdv",
                            8.0 * BW_D * pairs, 2.0 * B * (Lk * 4.0 * d + Lq * 2.0 * d), st)) !=
       cudaSuccess)
     return e;
-  // DQ: X1 = Q, X2 = dO (tokens, 128 rows); Y1 = K, Y2 = V (proxies, 64 rows);
+  // DQ: X1 = Q, X2 = dO (tokens); Y1 = K, Y2 = V (proxies);
   // u = dQ (dqa columns [0, d))
   a.out_u = dqa;
   a.ld_u = ldq;
   a.col_u = 0;
-  return bw_launch<false>(qa128, do128, kv64, kv64, 0, 0, 0, d, a, "attn_cross_bwd_dq",
+  return bw_launch<false>(tqa, tdo, tkv, tkv, 0, 0, 0, d, a, "attn_cross_bwd_dq",
                           6.0 * BW_D * pairs, 2.0 * B * (Lq * 3.0 * d + Lk * 2.0 * d), st);
 }
 

@@ -1,0 +1,47 @@
+"""Attention backward at proxy and token counts around its 128-row tiles and
+128-column steps: one row, one short of, at and past a tile, several tiles; causal
+and bidirectional proxies, and tokens against proxies (cross injection) where
+block boundaries fall inside tiles and steps."""
+import pytest
+import torch
+
+import paper_2608_23463_gb300 as pf
+import pf_synth as S
+from oracle import layer as OL
+from paper_2608_23463_gb300.layer import ProxyLayer, to_device
+from tests._util import CROSS_MAX_TOL, CROSS_TOL, assert_grad_close
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(spec, seed, tol, max_tol):
+    inp = S.make_layer_inputs(spec, seed, with_h_in=True)
+    lay = ProxyLayer(spec, inp)
+    X, G = to_device(inp["X"], torch.bfloat16), to_device(inp["G"], torch.bfloat16)
+    H_in = to_device(inp["H_in"], torch.float32)
+    dH = lay.empty_proxy()
+    lay.forward(X, H_in)
+    dX = lay.backward(X, G, H_in, dH_in=dH)
+    pf.pf_sync_check(torch.cuda.current_stream().cuda_stream)
+    rdX, rdH, rg = OL.layer_bwd(spec, inp, inp["X"], inp["G"], inp["H_in"])
+    assert_grad_close("dX", dX.float().cpu().numpy(), rdX, tol, max_tol)
+    assert_grad_close("dH_in", dH.cpu().numpy(), rdH, tol, max_tol)
+    for k in ("W_qkv",) + (("W_qa", "W_kvx") if spec.inject == S.INJ_CROSS else ()):
+        assert_grad_close("grad " + k, lay.grads[k].cpu().numpy(), rg[k], tol, max_tol)
+
+
+@pytest.mark.parametrize("mode", [S.CAUSAL_1D, S.BIDIR_1D])
+@pytest.mark.parametrize("m", [2, 127, 128, 129, 300])
+def test_proxy_attention_backward_edges(m, mode):
+    # four-token blocks: the gradients are held to the cross injection's bar, whose bf16
+    # floor is as high
+    spec = S.LayerSpec(batch=2, L=4 * m - 1, d=128, n_heads=2, P=4, mode=mode)
+    _check(spec, m, CROSS_TOL, CROSS_MAX_TOL)
+
+
+@pytest.mark.parametrize("L,P,mode", [(129, 1, S.CAUSAL_1D), (257, 3, S.CAUSAL_1D),
+                                      (1000, 7, S.CAUSAL_1D), (520, 130, S.CAUSAL_1D),
+                                      (385, 3, S.BIDIR_1D)])
+def test_cross_attention_backward_edges(L, P, mode):
+    spec = S.LayerSpec(batch=2, L=L, d=128, n_heads=2, P=P, mode=mode, inject=S.INJ_CROSS)
+    _check(spec, L, CROSS_TOL, CROSS_MAX_TOL)
