@@ -347,44 +347,67 @@ __global__ void __launch_bounds__(256, 2) inj_bwd_stream_kernel(InjBwdArgs a,
   }
 }
 
-// Deterministic warp sum: lane j adds summands j, j+32, ... in order, then a
-// fixed xor-shuffle tree.
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-  return v;
+// Column sums of `rows` rows, taken by a CTA of FS_WARPS warps, W (a power of two)
+// of them to 32 columns: warp w of a column group adds rows w, w + W, ... of its
+// lane's column (one 128-byte segment per load), then the W totals are added in
+// warp order.  The caller's columns start at c0 + 32 * (warp / W); returns the
+// total and the column, which is negative in threads that hold none.
+constexpr int FS_WARPS = 16;
+__device__ __forceinline__ float col_total(const float* __restrict__ p, int c0, int C, int rows,
+                                           long stride, int W, int& col) {
+  __shared__ float s_w[FS_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = warp & (W - 1);
+  col = c0 + (warp - w) / W * 32 + lane;
+  float a = 0.f;
+  if (col < C) {
+#pragma unroll 8
+    for (int r = w; r < rows; r += W) a += p[(long)r * stride + col];
+  }
+  s_w[warp][lane] = a;
+  __syncthreads();
+  if (w != 0 || col >= C) {
+    col = -1;
+    return 0.f;
+  }
+  float t = 0.f;
+  for (int k = 0; k < W; ++k) t += s_w[warp + k][lane];
+  return t;
 }
 
-// Column totals of the partials, one thread per (quantity q, column), chunks
-// added in order (coalesced across threads): q = 0 gives db_d1; the totals of
-// q = 1..3 are left in chunk 0's slots of part for the gate reduction below.
-__global__ void inj_bwd_colsum_kernel(float* __restrict__ part, int n_chunks, int N,
-                                      float* __restrict__ db_d1, int gates) {
+// Warps per column group: more than 16 rows are shared out.  One thread per column
+// adding all its rows took 52 us for 4096 columns of 512 chunks (with the gate
+// reduction; 15.5 so, 33 MB from L2 in two launches); 16 warps always, 20 us for
+// 65536 columns of 32 chunks (16.4 so: a CTA for every 32 columns is too little).
+int col_warps(int rows) {
+  int W = 1;
+  while (W < FS_WARPS && rows > 16 * W) W *= 2;
+  return W;
+}
+
+// Column totals of the partials over the chunks: q = blockIdx.y = 0 gives db_d1;
+// the totals of q = 1..3 go to `tot` (chunk 0's slots of part: only the threads
+// that write a column read it) for the gate reduction below.
+__global__ void __launch_bounds__(32 * FS_WARPS)
+    inj_bwd_colsum_kernel(const float* part, float* tot, int n_chunks, int N, int W,
+                          float* __restrict__ db_d1) {
   const int pz = pdl_enter();
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
-  const int nq = gates ? 4 : 1;
-  if (i >= (long)nq * N) return;
-  const int q = (int)(i / N), col = (int)(i % N);
-  float s = 0.f;
-#pragma unroll 8
-  for (int c = 0; c < n_chunks; ++c) s += part[((long)c * 4 + q) * N + col];
-  if (q == 0)
-    db_d1[col] = s;
-  else
-    part[(long)q * N + col] = s;
+  const int q = blockIdx.y;
+  int col;
+  const float t = col_total(part + (long)q * N, blockIdx.x * (FS_WARPS / W * 32) + pz, N, n_chunks,
+                            4L * N, W, col);
+  if (col >= 0) (q == 0 ? db_d1 : tot + (long)q * N)[col] = t;
 }
 
 // Gate gradients: g_q[ch] = sum over the k1 token positions t of the column
 // totals of quantity q (q = 1: w_x, 2: w_dlt, 3: b_g).
-__global__ void inj_bwd_gates_kernel(const float* __restrict__ part, int N, int d, float* gw_x,
-                                     float* gw_dlt, float* gb_g) {
+__global__ void __launch_bounds__(32 * FS_WARPS)
+    inj_bwd_gates_kernel(const float* __restrict__ part, int N, int d, float* gw_x, float* gw_dlt,
+                         float* gb_g) {
   const int pz = pdl_enter();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x + pz;
-  if (i >= 3 * d) return;
-  const int q = 1 + i / d, ch = i % d, T = N / d;
-  float s = 0.f;
-  for (int t = 0; t < T; ++t) s += part[(long)q * N + (long)t * d + ch];
-  (q == 1 ? gw_x : (q == 2 ? gw_dlt : gb_g))[ch] = s;
+  const int q = 1 + blockIdx.y;
+  int col;
+  const float t = col_total(part + (long)q * N, blockIdx.x * 32 + pz, d, N / d, d, FS_WARPS, col);
+  if (col >= 0) (q == 1 ? gw_x : (q == 2 ? gw_dlt : gb_g))[col] = t;
 }
 
 template <typename T>
@@ -446,28 +469,14 @@ __global__ void __launch_bounds__(EW_THREADS) colsum_part_kernel(const T* __rest
   }
 }
 
-// Pass 2: block = 32 consecutive columns x CS_WARPS warps; warp w adds chunks
-// w, w + CS_WARPS, ... of its lane's column (a chunk row is one 128-byte
-// segment per warp), then the warp totals are added in warp order.
-constexpr int CS_WARPS = 16;
-__global__ void __launch_bounds__(32 * CS_WARPS)
+// Pass 2: a CTA per 32 consecutive columns (C a multiple of 8).
+__global__ void __launch_bounds__(32 * FS_WARPS)
     colsum_final_kernel(const float* __restrict__ part, int n_chunks, int C,
                         float* __restrict__ out) {
   const int pz = pdl_enter();
-  __shared__ float s_w[CS_WARPS][32];
-  const int lane = (threadIdx.x & 31) + pz, w = threadIdx.x >> 5;
-  const int col = blockIdx.x * 32 + lane;
-  float a = 0.f;
-  if (col < C)
-    for (int c = w; c < n_chunks; c += CS_WARPS) a += part[(long)c * C + col];
-  s_w[w][lane] = a;
-  __syncthreads();
-  if (w == 0 && col < C) {
-    float t = 0.f;
-#pragma unroll
-    for (int k = 0; k < CS_WARPS; ++k) t += s_w[k][lane];
-    out[col] = t;
-  }
+  int col;
+  const float t = col_total(part, blockIdx.x * 32 + pz, C, n_chunks, C, FS_WARPS, col);
+  if (col >= 0) out[col] = t;
 }
 
 // Row chunks of a column reduction: about 1024 CTAs in total, independent of
@@ -492,6 +501,7 @@ int colsum_groups(int C) {
 // the summation order and the workspace size are fixed.
 int colsum_chunks(long R, int C) {
   const int gx = (C + colsum_groups(C) * 8 - 1) / (colsum_groups(C) * 8);
+  if (R <= 256) return 1;  // one pass, straight to the output: a launch costs more
   long want = (1216 + gx - 1) / gx;
   want = std::min(want, (R + 63) / 64);
   return (int)std::max(want, 1L);
@@ -507,11 +517,11 @@ cudaError_t colsum_impl(const T* X, long R, int C, float* out, float* part, cuda
   {
     LaunchTimer lt("colsum", st, (double)R * C, (double)R * C * sizeof(T));
     const cudaError_t e = launch_kernel(colsum_part_kernel<T>, grid, EW_THREADS, 0, st, X, R, C, cg,
-                                        rpc, part);
-    if (e != cudaSuccess) return e;
+                                        rpc, nc == 1 ? out : part);
+    if (e != cudaSuccess || nc == 1) return e;
   }
   LaunchTimer lt("colsum_final", st, (double)nc * C, 4.0 * nc * C);
-  return launch_kernel(colsum_final_kernel, (C + 31) / 32, 32 * CS_WARPS, 0, st, part, nc, C, out);
+  return launch_kernel(colsum_final_kernel, (C + 31) / 32, 32 * FS_WARPS, 0, st, part, nc, C, out);
 }
 
 }  // namespace
@@ -524,7 +534,8 @@ cudaError_t pad_rows(const bf16* src, bf16* dst, int B, long L, long Lp, int d, 
 }
 
 // The streaming form needs whole IB_W slices and enough rows per CTA to fill
-// its ring (about two CTAs per SM of a 152-SM part, at least 128 rows each).
+// its ring (about two CTAs per SM of a 152-SM part, at least 128 rows each; with
+// 102 rows, 1024 x 65536 takes 166 us against 139 by registers).
 long ib_stream_chunks(long M, int N) {
   if (N % IB_W != 0) return 0;
   const long c = (304 + N / IB_W - 1) / (N / IB_W);
@@ -559,13 +570,14 @@ cudaError_t inj_bwd_finalize(const float* part, int n_chunks, int N, int d, floa
                              float* gw_x, float* gw_dlt, float* gb_g, cudaStream_t st) {
   LaunchTimer lt("inj_bwd_finalize", st, 0.0, 16.0 * n_chunks * N);
   const int gates = gw_x != nullptr ? 1 : 0;
-  const long n = (long)(gates ? 4 : 1) * N;
-  float* pw = const_cast<float*>(part);  // the column totals reuse chunk 0's slots
-  const cudaError_t e = launch_kernel(inj_bwd_colsum_kernel, (unsigned)((n + 255) / 256), 256, 0, st,
-                                      pw, n_chunks, N, db_d1, gates);
+  const int W = col_warps(n_chunks), cols = FS_WARPS / W * 32;
+  float* tot = const_cast<float*>(part);  // the column totals reuse chunk 0's slots
+  const cudaError_t e = launch_kernel(inj_bwd_colsum_kernel,
+                                      dim3((N + cols - 1) / cols, gates ? 4 : 1), 32 * FS_WARPS, 0,
+                                      st, part, tot, n_chunks, N, W, db_d1);
   if (e != cudaSuccess || !gates) return e;
-  return launch_kernel(inj_bwd_gates_kernel, (3 * d + 255) / 256, 256, 0, st, part, N, d, gw_x,
-                       gw_dlt, gb_g);
+  return launch_kernel(inj_bwd_gates_kernel, dim3((d + 31) / 32, 3), 32 * FS_WARPS, 0, st, part, N, d,
+                       gw_x, gw_dlt, gb_g);
 }
 
 namespace {
