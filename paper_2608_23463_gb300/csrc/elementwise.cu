@@ -479,11 +479,12 @@ __global__ void __launch_bounds__(32 * FS_WARPS)
   if (col >= 0) out[col] = t;
 }
 
-// Row chunks of a column reduction: about 1024 CTAs in total, independent of
-// the device so that results (summation order) and workspace sizes are fixed.
+// Row chunks of the injection backward by registers: at most 912 CTAs in total,
+// three waves of two per SM of a 152-SM part, independent of the device so that
+// results (summation order) and workspace sizes are fixed.
 int chunks_for(long R, int C) {
   const int gx = (C / 8 + EW_THREADS - 1) / EW_THREADS;
-  long want = (1024 + gx - 1) / gx;
+  long want = 912 / gx;
   if (want > R) want = R;
   if (want < 1) want = 1;
   return (int)want;
@@ -533,13 +534,14 @@ cudaError_t pad_rows(const bf16* src, bf16* dst, int B, long L, long Lp, int d, 
   return launch_kernel(pad_rows_kernel, grid, 256, 0, st, src, dst, L, Lp, d);
 }
 
-// The streaming form needs whole IB_W slices and enough rows per CTA to fill
-// its ring (about two CTAs per SM of a 152-SM part, at least 128 rows each; with
-// 102 rows, 1024 x 65536 takes 166 us against 139 by registers).
+// The streaming form needs whole IB_W slices and enough rows per CTA to fill its
+// ring: one wave of at most 304 CTAs (two per SM of a 152-SM part) that leaves few
+// SMs idle, at least 64 rows each.  1024 x 65536: 9 chunks, 118 us; 10 chunks, 16
+// CTAs into a second wave, 166; by registers 139.
 long ib_stream_chunks(long M, int N) {
   if (N % IB_W != 0) return 0;
-  const long c = (304 + N / IB_W - 1) / (N / IB_W);
-  return M / c >= 128 ? c : 0;
+  const long slices = N / IB_W, c = 304 / slices;
+  return c * slices >= 272 && M / c >= 64 ? c : 0;
 }
 
 int inj_bwd_chunks(long M, int N) {

@@ -16,11 +16,12 @@ pytestmark = pytest.mark.gpu
 ROWS = [1, 16, 17, 33, 256, 257, 1100]
 
 
-@pytest.mark.parametrize("rows", ROWS)
-def test_bias_gradient_is_the_exact_sum(rows):
+# 2048 columns: by registers | streamed, 64 rows to each of 304 chunks, then ragged
+@pytest.mark.parametrize("rows,P", [(r, 8) for r in ROWS] + [(19455, 32), (19456, 32), (19500, 32)])
+def test_bias_gradient_is_the_exact_sum(rows, P):
     """Add injection: the gradient of b_d1 at token t of a block is the sum of G over
     the blocks.  G holds whole numbers of at most 8, so the sum is exact."""
-    spec = S.LayerSpec(batch=1, L=8 * rows, d=64, n_heads=1, P=8, mode=S.BIDIR_1D,
+    spec = S.LayerSpec(batch=1, L=P * rows, d=64, n_heads=1, P=P, mode=S.BIDIR_1D,
                        inject=S.INJ_ADD)
     inp = S.make_layer_inputs(spec, rows)
     G = np.random.default_rng(rows).integers(-8, 9, (1, spec.L, 64)).astype(np.float32)
@@ -29,7 +30,7 @@ def test_bias_gradient_is_the_exact_sum(rows):
     lay.forward(X)
     lay.backward(X, to_device(G, torch.bfloat16))
     pf.pf_sync_check(torch.cuda.current_stream().cuda_stream)
-    want = G.reshape(rows, 8 * 64).sum(0)
+    want = G.reshape(rows, P * 64).sum(0)
     assert np.array_equal(lay.grads["b_d1"].cpu().numpy().ravel(), want)
 
 
