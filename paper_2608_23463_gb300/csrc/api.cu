@@ -181,8 +181,8 @@ Saved carve_saved(Carve& c, const pf_layer_desc& s, const Dims& g) {
   return v;
 }
 
-// The bf16 forward's workspace: padded copy of a ragged X, split-K partials,
-// and the saved activations (in `saved` when given, else here).
+// The bf16 forward's workspace: padded copy of several ragged sequences' X, split-K
+// partials, and the saved activations (in `saved` when given, else here).
 struct FwdWs {
   bf16* Xpad;
   float* sk;
@@ -192,9 +192,17 @@ struct FwdWs {
   Saved sv;
 };
 
+// L consecutive tokens of df channels as rows of N1 = k1 * df (a last block's tokens
+// past L read as zero, without a padded copy of X, which cost 262136 tokens of 1024
+// channels 156 us at each of forward and backward).
+Operand token_rows(const bf16* X, long L, long N1, int df, int mn) {
+  const long k1 = N1 / df, rem = L % k1;
+  return Operand{X, N1, mn, L / k1, (int)(rem * df)};
+}
+
 FwdWs carve_fwd(Carve& wc, const pf_layer_desc& s, const Dims& g, void* saved) {
   FwdWs f{};
-  f.Xpad = g.ragged ? wc.take<bf16>(g.B * g.Lp * g.df) : nullptr;
+  f.Xpad = g.ragged && g.B > 1 ? wc.take<bf16>(g.B * g.Lp * g.df) : nullptr;
   f.skb = splitk_need(s, g, false);
   f.sk = wc.take<float>(f.skb / sizeof(float));
   if (g.cross) f.Wqa = wc.take<bf16>(g.ldq * g.d);
@@ -220,7 +228,7 @@ struct BwdWs {
 
 BwdWs carve_bwd(Carve& c, const pf_layer_desc& s, const Dims& g) {
   BwdWs w{};
-  w.Xpad = g.ragged ? c.take<bf16>(g.B * g.Lp * g.df) : nullptr;
+  w.Xpad = g.ragged && g.B > 1 ? c.take<bf16>(g.B * g.Lp * g.df) : nullptr;
   if (g.cross) {
     w.Wqa = c.take<bf16>(g.ldq * g.d);
     w.dAg = c.take<bf16>(g.T * g.d);
@@ -694,12 +702,9 @@ pf_status proxy_layer_fwd(const pf_layer_desc* desc, const pf_layer_params* prm,
   bf16* Xo = static_cast<bf16*>(X_out);
   const int d = (int)g.d, df = (int)g.df;  // proxy and token widths
 
-  // a1: partition (a zero-copy view; the ragged tail goes through a padded copy)
-  const bf16* Xsrc = Xb;
-  if (g.ragged) {
-    PF_CUDA(pad_rows(Xb, Xpad, (int)g.B, g.L, g.Lp, df, cs));
-    Xsrc = Xpad;
-  }
+  // a1: partition, a zero-copy view (several ragged sequences go through a padded copy)
+  if (Xpad) PF_CUDA(pad_rows(Xb, Xpad, (int)g.B, g.L, g.Lp, df, cs));
+  const Operand Xop = Xpad ? Operand{Xpad, g.N1, 0} : token_rows(Xb, g.B * g.L, g.N1, df, 0);
   // a2 + a3: compression (Eq. compress-linear / factor-cascade), H = H_in + C
   {
     EpiLinearArgs e;
@@ -712,14 +717,14 @@ pf_status proxy_layer_fwd(const pf_layer_desc* desc, const pf_layer_params* prm,
       e.out_bf16 = sv.Hb;
       e.ld_bf16 = d;
       set_gemm_tag("compress_c1", (double)g.R * d * 6.0);
-      PF_CUDA(gemm_linear((int)g.R, d, (int)g.N1, {Xsrc, g.N1, 0},
+      PF_CUDA(gemm_linear((int)g.R, d, (int)g.N1, Xop,
                           {static_cast<const bf16*>(prm->W_c1), g.N1, 0}, with_sk(e, sk, skb), cs));
     } else {
       e.bias = prm->b_c1;
       e.out_bf16 = sv.Y;
       e.ld_bf16 = d;
       set_gemm_tag("compress_c1", (double)g.rows1 * d * 2.0);
-      PF_CUDA(gemm_linear((int)g.rows1, d, (int)g.N1, {Xsrc, g.N1, 0},
+      PF_CUDA(gemm_linear((int)g.rows1, d, (int)g.N1, Xop,
                           {static_cast<const bf16*>(prm->W_c1), g.N1, 0}, with_sk(e, sk, skb), cs));
       EpiLinearArgs e2;
       e2.bias = prm->b_c2;
@@ -870,11 +875,8 @@ pf_status proxy_layer_bwd(const pf_layer_desc* desc, const pf_layer_params* prm,
   const bf16* W_d2 = static_cast<const bf16*>(prm->W_d2);
   const bf16* W_d1 = static_cast<const bf16*>(prm->W_d1);
 
-  const bf16* Xsrc = Xb;
-  if (g.ragged) {
-    PF_CUDA(pad_rows(Xb, w.Xpad, (int)g.B, g.L, g.Lp, df, cs));
-    Xsrc = w.Xpad;
-  }
+  if (w.Xpad) PF_CUDA(pad_rows(Xb, w.Xpad, (int)g.B, g.L, g.Lp, df, cs));
+  const Operand Xop = w.Xpad ? Operand{w.Xpad, N1, 1} : token_rows(Xb, g.B * g.L, N1, df, 1);
   // the direct injection gradient goes into dX; the dX GEMM adds to it
   if (g.cross) {
     // the gated cross injection backward: output projection, gate, the
@@ -1092,7 +1094,7 @@ pf_status proxy_layer_bwd(const pf_layer_desc* desc, const pf_layer_params* prm,
     e.out_f32 = grads->W_c1;
     e.ld_f32 = N1;
     set_gemm_tag("bwd_dW_c1", (double)d * N1 * 4.0);
-    PF_CUDA(gemm_linear(d, N1, (int)g.rows1, {dYsrc, d, 1}, {Xsrc, N1, 1}, with_sk(e, w.sk, w.skb), cs));
+    PF_CUDA(gemm_linear(d, N1, (int)g.rows1, {dYsrc, d, 1}, Xop, with_sk(e, w.sk, w.skb), cs));
   }
   {
     EpiDXArgs e{dXb, df, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L};
@@ -1478,7 +1480,6 @@ namespace {
 
 struct Seg {
   long L, P, k1, k2, m, off, g0, rows1, N1;
-  bool ragged;
 };
 struct SegPlan {
   long d, nh, M;
@@ -1520,7 +1521,6 @@ pf_status seg_plan(const pf_layer_desc* desc, int32_t n, const pf_segment* segs,
     g.g0 = g0;
     g.rows1 = g.m * g.k2;
     g.N1 = g.k1 * q.d;
-    g.ragged = g.m * g.P != g.L;
     if (g.N1 > (1L << 30)) return fail(PF_ERR_UNSUPPORTED, "segment %d too large", i);
     p.s.push_back(g);
     off += a.L;
@@ -1573,7 +1573,6 @@ size_t seg_splitk(const SegPlan& p, bool bwd) {
 }
 
 struct SegFwdWs {
-  bf16* Xpad;  // the last segment, zero-padded to whole blocks (if ragged)
   float* sk;
   size_t skb;
   SegSaved sv;
@@ -1581,8 +1580,6 @@ struct SegFwdWs {
 
 SegFwdWs carve_seg_fwd(Carve& wc, const SegPlan& p, void* saved) {
   SegFwdWs f;
-  const Seg& z = p.s.back();
-  f.Xpad = z.ragged ? wc.take<bf16>(z.m * z.P * p.d) : nullptr;
   f.skb = seg_splitk(p, false);
   f.sk = wc.take<float>(f.skb / sizeof(float));
   Carve sc(saved);
@@ -1591,14 +1588,13 @@ SegFwdWs carve_seg_fwd(Carve& wc, const SegPlan& p, void* saved) {
 }
 
 struct SegBwdWs {
-  bf16 *Xpad, *dD, *dZ, *dHbar, *dA, *dQKV, *dHb, *dY;
+  bf16 *dD, *dZ, *dHbar, *dA, *dQKV, *dHb, *dY;
   float *Di, *dHf, *part, *sk, *gtmp, *gsum;
   size_t skb;
 };
 
 SegBwdWs carve_seg_bwd(Carve& c, const SegPlan& p) {
   SegBwdWs w{};
-  const Seg& z = p.s.back();
   long dD = 0, dZ = 0, dY = 0, pe = 0;
   for (const Seg& g : p.s) {
     dD = std::max(dD, g.rows1 * g.N1);
@@ -1610,7 +1606,6 @@ SegBwdWs carve_seg_bwd(Carve& c, const SegPlan& p) {
     pe = std::max(pe, colsum_part_elems(g.rows1, (int)p.d));
   }
   pe = std::max(pe, colsum_part_elems((long)p.s.size(), (int)(3 * p.d)));
-  w.Xpad = z.ragged ? c.take<bf16>(z.m * z.P * p.d) : nullptr;
   w.dD = c.take<bf16>(dD);
   if (p.levels == 2) w.dZ = c.take<bf16>(dZ);
   w.dHbar = c.take<bf16>(p.M * p.d);
@@ -1694,10 +1689,7 @@ pf_status proxy_segments_fwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
   for (size_t i = 0; i < p.s.size(); ++i) {
     const Seg& g = p.s[i];
     const bf16* Xs = Xb + g.off * d;
-    if (g.ragged) {
-      PF_CUDA(pad_rows(Xs, f.Xpad, 1, g.L, g.m * g.P, d, cs));
-      Xs = f.Xpad;
-    }
+    const Operand Xop = token_rows(Xs, g.L, g.N1, d, 0);
     const bf16* W_c1 = static_cast<const bf16*>(sp[i].W_c1);
     EpiLinearArgs e;
     e.bias = sp[i].b_c1;
@@ -1705,13 +1697,13 @@ pf_status proxy_segments_fwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
     if (p.levels == 1) {
       e.out_bf16 = sv.Hb + g.g0 * d;
       set_gemm_tag("seg_compress_c1", (double)g.m * d * 2.0);
-      PF_CUDA(gemm_linear((int)g.m, d, (int)g.N1, {Xs, g.N1, 0}, {W_c1, g.N1, 0},
+      PF_CUDA(gemm_linear((int)g.m, d, (int)g.N1, Xop, {W_c1, g.N1, 0},
                           with_sk(e, f.sk, f.skb), cs));
     } else {
       const int n2 = (int)(g.k2 * d);
       e.out_bf16 = sv.Y[i];
       set_gemm_tag("seg_compress_c1", (double)g.rows1 * d * 2.0);
-      PF_CUDA(gemm_linear((int)g.rows1, d, (int)g.N1, {Xs, g.N1, 0}, {W_c1, g.N1, 0},
+      PF_CUDA(gemm_linear((int)g.rows1, d, (int)g.N1, Xop, {W_c1, g.N1, 0},
                           with_sk(e, f.sk, f.skb), cs));
       EpiLinearArgs e2;
       e2.bias = sp[i].b_c2;
@@ -1795,18 +1787,12 @@ pf_status proxy_segments_bwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
   // the last proxy feeds no block
   PF_CUDA(cudaMemsetAsync(w.dHbar + (p.M - 1) * d, 0, d * sizeof(bf16), cs));
   if (p.gated) PF_CUDA(cudaMemsetAsync(w.gtmp, 0, p.s.size() * 3 * d * sizeof(float), cs));
-  std::vector<const bf16*> xs(p.s.size());
   // injection and decompression backward, segment by segment (segment 0 first:
   // its last proxy row, which feeds no block of its own, is overwritten by
   // segment 1's first source row)
   for (size_t i = 0; i < p.s.size(); ++i) {
     const Seg& g = p.s[i];
     const bf16* Xs = Xb + g.off * d;
-    xs[i] = Xs;
-    if (g.ragged) {
-      PF_CUDA(pad_rows(Xs, w.Xpad, 1, g.L, g.m * g.P, d, cs));
-      xs[i] = w.Xpad;
-    }
     const int N1 = (int)g.N1, r1 = (int)g.rows1;
     const int nch = inj_bwd_chunks(g.rows1, N1);
     InjBwdArgs a{G + g.off * d, Xs, sv.D[i], w.dD, dXb + g.off * d, prm->w_x,
@@ -1926,7 +1912,8 @@ pf_status proxy_segments_bwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
       e.out_f32 = sg[i].W_c1;
       e.ld_f32 = N1;
       set_gemm_tag("seg_bwd_dW_c1", (double)d * N1 * 4.0);
-      PF_CUDA(gemm_linear(d, N1, r1, {dYsrc, d, 1}, {xs[i], N1, 1}, with_sk(e, w.sk, w.skb), cs));
+      PF_CUDA(gemm_linear(d, N1, r1, {dYsrc, d, 1}, 
+                          token_rows(Xb + g.off * d, g.L, N1, d, 1), with_sk(e, w.sk, w.skb), cs));
     }
     EpiDXArgs e{dXb + g.off * d, d, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L};
     set_gemm_tag("seg_bwd_dX", (double)r1 * N1 * 4.0);

@@ -58,10 +58,26 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, 
 
 // rows = M (for A) or N (for B).
 bool make_operand_map(CUtensorMap* m, const Operand& op, int rows, int K) {
-  if (op.mn) return make_map(m, op.ptr, (uint64_t)rows, (uint64_t)K, (uint64_t)op.ld, 64, 64);
-  return make_map(m, op.ptr, (uint64_t)K, (uint64_t)rows, (uint64_t)op.ld, 64, 128);
+  // whole rows only; with none of them, the tail's map, which is zero past the tail
+  const bool cut = op.full >= 0, none = op.full == 0;
+  const uint64_t in = (uint64_t)(op.mn ? rows : K), out = (uint64_t)(op.mn ? K : rows);
+  return make_map(m, op.ptr, none ? (uint64_t)op.tail : in,
+                  none ? 1 : cut ? (uint64_t)op.full : out, (uint64_t)op.ld, 64, op.mn ? 64 : 128);
 }
 
+// The first `tail` columns of a matrix that ends inside a row: they have one row
+// more than the others.
+bool make_tail_map(CUtensorMap* m, const Operand& op) {
+  return make_map(m, op.ptr, (uint64_t)op.tail, (uint64_t)op.full + 1, (uint64_t)op.ld, 64,
+                  op.mn ? 64 : 128);
+}
+
+// The maps of a product: A, B, and of the one operand that ends inside a row (A if
+// both are K-major, B if both are MN-major) the columns below `tail`.
+struct Maps {
+  CUtensorMap a, b, t;
+  int tail;
+};
 // B of a direct epilogue: row n = 8 s + 2 g + e as dimensions (k, e, g, s); a box
 // holds 32 rows of one g.
 bool make_segment_map(CUtensorMap* m, const Operand& op, int rows, int K) {
@@ -75,6 +91,19 @@ bool make_segment_map(CUtensorMap* m, const Operand& op, int rows, int K) {
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(op.ptr), dims, strides, box,
             es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool make_maps(Maps* m, bool direct, int M, int N, int K, const Operand& A, const Operand& B) {
+  if ((A.full >= 0 && (A.mn || B.mn)) || (B.full >= 0 && !(A.mn && B.mn)) || A.tail % 64 != 0 ||
+      B.tail % 64 != 0 || (A.full == 0 && A.tail == 0) || (B.full == 0 && B.tail == 0))
+    return false;
+  if (!make_operand_map(&m->a, A, M, K) ||
+      !(direct ? make_segment_map(&m->b, B, N, K) : make_operand_map(&m->b, B, N, K)))
+    return false;
+  const Operand& op = A.full > 0 ? A : B;
+  m->tail = op.full > 0 ? op.tail : 0;
+  m->t = m->a;  // unused below column 0
+  return m->tail == 0 || make_tail_map(&m->t, op);
 }
 
 // Co-resident CTA pairs of the pair kernel (at most half the SMs).
@@ -152,8 +181,8 @@ Plan gemm_plan(int M, int N, int K, size_t bytes) {
 }
 
 template <int BN, bool AMN, bool BMN, class Epi>
-cudaError_t launch(int M, int N, int K, const CUtensorMap& ta, const CUtensorMap& tb,
-                   const Epi& epi, cudaStream_t st, const Plan& plan) {
+cudaError_t launch(int M, int N, int K, const Maps& tm, const Epi& epi, cudaStream_t st,
+                   const Plan& plan) {
   const int splits = plan.S;
   if constexpr (BN == 256) {  // CTA pairs: 256 x 256 tiles, half of B per CTA
     auto kern2 = gemm_tc_kernel<BN, AMN, BMN, Epi, true>;
@@ -166,7 +195,8 @@ cudaError_t launch(int M, int N, int K, const CUtensorMap& ta, const CUtensorMap
           (long)((N + BN - 1) / BN) * ((M + 2 * GEMM_BM - 1) / (2 * GEMM_BM)) * splits;
       if (pairs > 0)
         return launch_clusters(2, kern2, 2 * (unsigned)std::min<long>(pair_tiles, pairs),
-                               GEMM_THREADS, smem2, st, ta, tb, M, N, K, splits, epi);
+                               GEMM_THREADS, smem2, st, tm.a, tm.b, tm.t, tm.tail, M, N, K, splits,
+                               epi);
     }
   }
   auto kern = gemm_tc_kernel<BN, AMN, BMN, Epi>;
@@ -175,21 +205,21 @@ cudaError_t launch(int M, int N, int K, const CUtensorMap& ta, const CUtensorMap
   if (e != cudaSuccess) return e;
   const long tiles = (long)((N + BN - 1) / BN) * ((M + GEMM_BM - 1) / GEMM_BM) * splits;
   const int grid = (int)std::min<long>(tiles, num_sms());
-  return launch_kernel(kern, grid, GEMM_THREADS, smem, st, ta, tb, M, N, K, splits, epi);
+  return launch_kernel(kern, grid, GEMM_THREADS, smem, st, tm.a, tm.b, tm.t, tm.tail, M, N, K, splits,
+                       epi);
 }
 
 // Operand majors that the epilogue's callers use: all four for the linear
 // ones, K-major A (and for a direct one K-major B) for the fused ones.
 template <int BN, class Epi>
-cudaError_t launch_majors(int M, int N, int K, const Operand& A, const Operand& B,
-                          const CUtensorMap& ta, const CUtensorMap& tb, const Epi& epi,
-                          cudaStream_t st, const Plan& plan) {
-  if (!A.mn && !B.mn) return launch<BN, false, false>(M, N, K, ta, tb, epi, st, plan);
+cudaError_t launch_majors(int M, int N, int K, const Operand& A, const Operand& B, const Maps& tm,
+                          const Epi& epi, cudaStream_t st, const Plan& plan) {
+  if (!A.mn && !B.mn) return launch<BN, false, false>(M, N, K, tm, epi, st, plan);
   if constexpr (!Epi::kDirect)
-    if (!A.mn && B.mn) return launch<BN, false, true>(M, N, K, ta, tb, epi, st, plan);
+    if (!A.mn && B.mn) return launch<BN, false, true>(M, N, K, tm, epi, st, plan);
   if constexpr (!Epi::kRows) {
-    if (A.mn && B.mn) return launch<BN, true, true>(M, N, K, ta, tb, epi, st, plan);
-    return launch<BN, true, false>(M, N, K, ta, tb, epi, st, plan);
+    if (A.mn && B.mn) return launch<BN, true, true>(M, N, K, tm, epi, st, plan);
+    return launch<BN, true, false>(M, N, K, tm, epi, st, plan);
   }
   return cudaErrorInvalidValue;
 }
@@ -204,10 +234,8 @@ cudaError_t gemm_dispatch(int M, int N, int K, Operand A, Operand B, const Epi& 
                           cudaStream_t st) {
   if (M <= 0 || N <= 0 || N % 32 != 0 || K < 0 || !operand_ok(A) || !operand_ok(B))
     return cudaErrorInvalidValue;
-  CUtensorMap ta, tb;
-  if (!make_operand_map(&ta, A, M, K) ||
-      !(Epi::kDirect ? make_segment_map(&tb, B, N, K) : make_operand_map(&tb, B, N, K)))
-    return cudaErrorInvalidValue;
+  Maps tm;
+  if (!make_maps(&tm, Epi::kDirect, M, N, K, A, B)) return cudaErrorInvalidValue;
   LaunchTimer lt(gemm_tag_label(), st, 2.0 * M * N * (double)K,
                  2.0 * ((double)M * K + (double)N * K) + gemm_tag_bytes());
   Plan plan = gemm_plan(M, N, K, 0);
@@ -215,9 +243,9 @@ cudaError_t gemm_dispatch(int M, int N, int K, Operand A, Operand B, const Epi& 
     plan.bn = 256;
     plan.pair = plan_cost(M, N, K, 256, true, 1) <= plan_cost(M, N, K, 256, false, 1);
   } else if (plan.bn == 128) {
-    return launch_majors<128>(M, N, K, A, B, ta, tb, epi, st, plan);
+    return launch_majors<128>(M, N, K, A, B, tm, epi, st, plan);
   }
-  return launch_majors<256>(M, N, K, A, B, ta, tb, epi, st, plan);
+  return launch_majors<256>(M, N, K, A, B, tm, epi, st, plan);
 }
 
 // out = sum_s part[s] (+ bias) (+ addend) -> fp32 and/or bf16, 4 columns per thread.
@@ -290,16 +318,15 @@ cudaError_t gemm_linear(int M, int N, int K, Operand A, Operand B, const EpiLine
   if (S > 1) {
     // deterministic split-K: raw partials, then one reduce applying the epilogue
     if (M <= 0 || N % 32 != 0 || !operand_ok(A) || !operand_ok(B)) return cudaErrorInvalidValue;
-    CUtensorMap ta, tb;
-    if (!make_operand_map(&ta, A, M, K) || !make_operand_map(&tb, B, N, K))
-      return cudaErrorInvalidValue;
+    Maps tm;
+    if (!make_maps(&tm, false, M, N, K, A, B)) return cudaErrorInvalidValue;
     EpiPartial epi{{}, N, e.splitk_scratch};
     {
       LaunchTimer lt(gemm_tag_label(), st, 2.0 * M * N * (double)K,
                      2.0 * ((double)M * K + (double)N * K) + 4.0 * S * M * N);
       const cudaError_t err =
-          plan.bn == 256 ? launch_majors<256>(M, N, K, A, B, ta, tb, epi, st, plan)
-                         : launch_majors<128>(M, N, K, A, B, ta, tb, epi, st, plan);
+          plan.bn == 256 ? launch_majors<256>(M, N, K, A, B, tm, epi, st, plan)
+                         : launch_majors<128>(M, N, K, A, B, tm, epi, st, plan);
       if (err != cudaSuccess) return err;
     }
     LaunchTimer lt("splitk_reduce", st, (double)S * M * N, 4.0 * (S + 1.0) * M * N);

@@ -152,7 +152,8 @@ constexpr uint32_t gemm_stage_bytes(bool pair) {
 template <int BN, bool A_MN, bool B_MN, class Epi, bool PAIR = false>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   int M, int N, int K, int splits, Epi epi) {
+                   const __grid_constant__ CUtensorMap tmT, int tail, int M, int N, int K,
+                   int splits, Epi epi) {
   static_assert(!PAIR || BN == 256, "CTA pairs use 256-wide tiles");
   static_assert(!Epi::kDirect || !B_MN, "direct epilogues need a K-major B");
   constexpr uint32_t SB = gemm_stage_bytes<Epi>(PAIR);
@@ -260,8 +261,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         const uint32_t a_dst = smem_u32(smem + s * Cfg::STAGE_BYTES);
         const uint32_t b_dst = a_dst + Cfg::A_BYTES;
         const int k0 = kt * GEMM_BK;
+        // columns below `tail` of the operand that ends inside a row (A or B, by the
+        // majors) go through their own map
         if (!A_MN) {
-          ld(a_dst, &tmA, k0, m0);
+          ld(a_dst, !B_MN && !Epi::kRows && k0 < tail ? &tmT : &tmA, k0, m0);
         } else {
           ld(a_dst, &tmA, m0, k0);
           ld(a_dst + 8192, &tmA, m0 + 64, k0);
@@ -289,8 +292,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         } else {
           constexpr int JB = Cfg::B_ROWS / 64;
 #pragma unroll
-          for (int j = 0; j < JB; ++j)
-            ld(b_dst + j * 8192, &tmB, n0 + 64 * (j + (int)rank * JB), k0);
+          for (int j = 0; j < JB; ++j) {
+            const int n = n0 + 64 * (j + (int)rank * JB);
+            ld(b_dst + j * 8192, A_MN && n < tail ? &tmT : &tmB, n, k0);
+          }
         }
         issued = it + 1;
       }

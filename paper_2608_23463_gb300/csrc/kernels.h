@@ -46,6 +46,11 @@ struct Operand {
   const bf16* ptr;
   long ld;
   int mn;
+  // a matrix that ends inside a row (X of a ragged sequence): `full` whole rows of
+  // ld elements, then `tail` elements (a multiple of 64); the rest reads as zero.
+  // full < 0: the matrix has every row.
+  long full = -1;
+  int tail = 0;
 };
 
 struct EpiLinearArgs {
