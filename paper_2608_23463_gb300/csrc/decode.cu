@@ -313,11 +313,28 @@ __global__ void __launch_bounds__(512) split_kernel(
 }
 
 // Per (b, h): A_h from the split partials, A_x over the open slots 0..n_o,
-// alpha_h = sigmoid(W_a2[h] u_b + b_a2[h]), A = A_x + alpha_h A_h (fp32
+// alpha_h = sigmoid(W_a2[h] u_b + b_a2[h]), A = A_x + alpha_h A_h (bf16
 // [B, d]).  COMBINE_G groups of DH threads: thread (g, t) owns head dim t and
 // sums splits s = g, g+G, ... and open keys j = g, g+G, ...; the groups are
-// added in shared memory.  Open-key scores take one thread per key.
+// added in shared memory.  Latency bounds it (a few KB per CTA), so everything
+// that it reads is asked for at once, before the first barrier: up to COMBINE_PF
+// partials and values per thread wait in registers.  Keys' scores take DH / 8
+// lanes each; one warp makes the weights of the open keys, another those of the
+// splits.  (Sequential maxima and sums in every thread, a lane per key: 18 us for 8
+// sequences of 16 heads with an event on either side, 10.5 so; a lone small step in a
+// graph 22.5 and 20.4.)
 constexpr int COMBINE_G = 4;
+constexpr int COMBINE_PF = 16;
+__device__ __forceinline__ float warp_max(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 template <int DH>
 __global__ void __launch_bounds__(COMBINE_G * DH) combine_kernel(
     const float* __restrict__ part, int splits, const float* __restrict__ q,
@@ -326,79 +343,117 @@ __global__ void __launch_bounds__(COMBINE_G * DH) combine_kernel(
     const bf16* __restrict__ u, const bf16* __restrict__ W_a2, const float* __restrict__ b_a2,
     bf16* __restrict__ A) {
   const int pz = pdl_enter();
+  constexpr int G = COMBINE_G, NT = G * DH;
+  constexpr int LPK = DH / 8, KPP = NT / LPK;  // lanes per key, keys per pass (32)
   __shared__ float s_p[PF_DECODE_MAX_P];
   __shared__ float s_m[MAX_SPLITS], s_l[MAX_SPLITS];
-  __shared__ __align__(16) float s_q[DH];
-  __shared__ float s_red[2][COMBINE_G - 1][DH];
-  __shared__ float s_alpha;
+  __shared__ float s_red[2][G - 1][DH];
+  __shared__ float s_alpha, s_M, s_Lh, s_Lx;
   const int h = blockIdx.x + pz, b = blockIdx.y + pz, tid = threadIdx.x, lane = tid & 31;
-  const int g = tid / DH, t = tid % DH;
-  if (!valid[b]) return;  // flagged earlier; sequence untouched
-  const int n = n_open[b];  // already advanced: open slots 0..n-1 incl. the new token
-  if (tid < DH) s_q[tid] = q[(long)b * d + h * DH + tid] * sl2;
+  const int warp = tid >> 5, g = tid / DH, t = tid % DH;
+  const int ok = valid[b], n = n_open[b];  // n: already advanced, slots 0..n-1 incl. the new token
+  const int kl = tid % LPK, kg = tid / LPK;
+  float qv[8];
+  load8f(q + (long)b * d + h * DH + kl * 8, qv);
   const float* pb = part + ((long)b * splits * nh + h) * (DH + 2);
   const long pstride = (long)nh * (DH + 2);  // between splits
-  for (int s = tid; s < splits; s += blockDim.x) {
+  float pa[COMBINE_PF];
+#pragma unroll
+  for (int i = 0; i < COMBINE_PF; ++i) {
+    const int s = g + i * G;
+    pa[i] = s < splits ? pb[s * pstride + 2 + t] : 0.f;
+  }
+  for (int s = tid; s < splits; s += NT) {
     s_m[s] = pb[s * pstride];
     s_l[s] = pb[s * pstride + 1];
   }
-  // alpha (Eq. llm-gate): the last warp
-  if (tid >= blockDim.x - 32) {
+  if (!ok) return;  // flagged earlier; sequence untouched
+  const bf16* vo = V_open + (long)b * P * d + h * DH + t;
+  bf16 pv[COMBINE_PF];
+#pragma unroll
+  for (int i = 0; i < COMBINE_PF; ++i) {
+    const int j = g + i * G;
+    pv[i] = j < n ? vo[(long)j * d] : __float2bfloat16(0.f);
+  }
+  if (warp == NT / 32 - 1) {  // alpha (Eq. llm-gate)
     const int H = d / 8;
     float acc = 0.f;
-    for (int k = lane; k < H; k += 32)
-      acc = fmaf(__bfloat162float(W_a2[(long)h * H + k]), __bfloat162float(u[(long)b * H + k]),
-                 acc);
+    for (int k = lane * 8; k < H; k += 256) {
+      float wv[8], uv[8];
+      load8_bf16(W_a2 + (long)h * H + k, wv);
+      load8_bf16(u + (long)b * H + k, uv);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      for (int e = 0; e < 8; ++e) acc = fmaf(wv[e], uv[e], acc);
+    }
+    acc = warp_sum(acc);
     if (lane == 0) s_alpha = sigmoidf_(acc + b_a2[h]);
   }
+  // open-key scores
+#pragma unroll 2
+  for (int j0 = 0; j0 < n; j0 += KPP) {
+    const int j = j0 + kg;
+    float kv[8] = {}, v = 0.f;
+    if (j < n) load8_bf16(K_open + ((long)b * P + j) * d + h * DH + kl * 8, kv);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v = fmaf(qv[e] * sl2, kv[e], v);
+#pragma unroll
+    for (int o = LPK / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (kl == 0 && j < n) s_p[j] = v;
+  }
   __syncthreads();
-  // open-key scores: thread j < n computes key j's dot product (16-byte loads)
-  if (tid < n) {
-    const bf16* kr = K_open + ((long)b * P + tid) * d + h * DH;
-    float v = 0.f;
-#pragma unroll
-    for (int e = 0; e < DH; e += 8) {
-      float kv[8];
-      load8_bf16(kr + e, kv);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v = fmaf(s_q[e + i], kv[i], v);
+  if (warp == 0) {
+    float mx = -INFINITY, l = 0.f;
+    for (int j = lane; j < n; j += 32) mx = fmaxf(mx, s_p[j]);
+    mx = warp_max(mx);
+    for (int j = lane; j < n; j += 32) {
+      const float p = exp2f(s_p[j] - mx);
+      s_p[j] = p;
+      l += p;
     }
-    s_p[tid] = v;
+    l = warp_sum(l);
+    if (lane == 0) s_Lx = l;
+  } else if (warp == 1) {
+    float M = -INFINITY, l = 0.f;
+    for (int s = lane; s < splits; s += 32) M = fmaxf(M, s_m[s]);
+    M = warp_max(M);
+    for (int s = lane; s < splits; s += 32) {
+      const float w = M != -INFINITY ? exp2f(s_m[s] - M) : 0.f;
+      s_m[s] = w;
+      l = fmaf(s_l[s], w, l);
+    }
+    l = warp_sum(l);
+    if (lane == 0) {
+      s_M = M;
+      s_Lh = l;
+    }
   }
   __syncthreads();
-  float M = -INFINITY;
-  for (int s = 0; s < splits; ++s) M = fmaxf(M, s_m[s]);
-  float mx = -INFINITY;
-  for (int j = 0; j < n; ++j) mx = fmaxf(mx, s_p[j]);
   float ah = 0.f, ax = 0.f;
-  if (M != -INFINITY) {
-#pragma unroll 8
-    for (int s = g; s < splits; s += COMBINE_G)
-      ah = fmaf(pb[s * pstride + 2 + t], exp2f(s_m[s] - M), ah);
+#pragma unroll
+  for (int i = 0; i < COMBINE_PF; ++i) {
+    const int s = g + i * G;
+    if (s < splits) ah = fmaf(pa[i], s_m[s], ah);
+    if (s < n) ax = fmaf(s_p[s], __bfloat162float(pv[i]), ax);
   }
 #pragma unroll 8
-  for (int j = g; j < n; j += COMBINE_G)
-    ax = fmaf(exp2f(s_p[j] - mx), __bfloat162float(V_open[((long)b * P + j) * d + h * DH + t]),
-              ax);
+  for (int s = g + COMBINE_PF * G; s < splits; s += G)
+    ah = fmaf(pb[s * pstride + 2 + t], s_m[s], ah);
+#pragma unroll 8
+  for (int j = g + COMBINE_PF * G; j < n; j += G)
+    ax = fmaf(s_p[j], __bfloat162float(vo[(long)j * d]), ax);
   if (g > 0) {
     s_red[0][g - 1][t] = ah;
     s_red[1][g - 1][t] = ax;
   }
   __syncthreads();
   if (g > 0) return;
-  float Lh = 0.f, Lx = 0.f;
-  if (M != -INFINITY)
-    for (int s = 0; s < splits; ++s) Lh = fmaf(s_l[s], exp2f(s_m[s] - M), Lh);
-  for (int j = 0; j < n; ++j) Lx += exp2f(s_p[j] - mx);
 #pragma unroll
-  for (int i = 0; i < COMBINE_G - 1; ++i) {
+  for (int i = 0; i < G - 1; ++i) {
     ah += s_red[0][i][t];
     ax += s_red[1][i][t];
   }
-  const float Ah = (M != -INFINITY) ? ah / Lh : 0.f;
-  A[(long)b * d + h * DH + t] = __float2bfloat16(ax / Lx + s_alpha * Ah);
+  const float Ah = (s_M != -INFINITY) ? ah / s_Lh : 0.f;
+  A[(long)b * d + h * DH + t] = __float2bfloat16(ax / s_Lx + s_alpha * Ah);
 }
 
 // Append bookkeeping: a sequence is appended iff its block is full and its
