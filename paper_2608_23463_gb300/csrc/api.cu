@@ -1275,13 +1275,9 @@ pf_status proxy_kv_append(const pf_decode_desc* desc, const pf_append_params* pr
                         cs));
   }
   // the proxy's key and value rows into cache row n_proxy[b]
-  {
-    EpiAppendArgs e{static_cast<bf16*>(cache->K_proxy), static_cast<bf16*>(cache->V_proxy),
-                    cache->n_open, cache->n_proxy, d, P, s.capacity};
-    set_gemm_tag("append_kv", (double)B * 2 * d * 2.0);
-    PF_CUDA(gemm_append_kv(B, 2 * d, d, {w.Hb, d, 0}, {static_cast<const bf16*>(prm->W_kvh), d, 0},
-                           e, cs));
-  }
+  PF_CUDA(kv_rows(B, d, w.Hb, static_cast<const bf16*>(prm->W_kvh),
+                  static_cast<bf16*>(cache->K_proxy), static_cast<bf16*>(cache->V_proxy),
+                  cache->n_open, cache->n_proxy, P, s.capacity, "append_kv", cs));
   PF_CUDA(append_finish(cache->n_open, cache->n_proxy, B, P, s.capacity, cs));
   return PF_OK;
 }
@@ -1311,21 +1307,14 @@ pf_status prefill_open(const pf_decode_desc& s, const pf_decode_params* dp, cons
                        long L_hist, pf_kv_cache* cache, cudaStream_t cs) {
   const long P = s.P, d = s.d, B = s.batch;
   const long m = L_hist / P, r = L_hist - m * P;
-  for (long b = 0; b < B && r > 0; ++b) {
-    const bf16* Xr = X + (b * L_hist + m * P) * d;
-    bf16* Xo = static_cast<bf16*>(cache->X_open) + b * P * d;
-    PF_CUDA(cudaMemcpyAsync(Xo, Xr, (size_t)r * d * sizeof(bf16), cudaMemcpyDeviceToDevice, cs));
-    const bf16* Wqkv = static_cast<const bf16*>(dp->W_qkv);
-    for (int kv = 0; kv < 2; ++kv) {
-      EpiLinearArgs e;
-      e.out_bf16 = static_cast<bf16*>(kv ? cache->V_open : cache->K_open) + b * P * d;
-      e.ld_bf16 = d;
-      set_gemm_tag("prefill_open_kv", (double)r * d * 2.0);
-      PF_CUDA(gemm_linear((int)r, (int)d, (int)d, {Xr, d, 0}, {Wqkv + (1 + kv) * d * d, d, 0}, e,
-                          cs));
-    }
-  }
-  PF_CUDA(prefill_counts(cache->n_open, cache->n_proxy, (int)B, (int)m, (int)r, cs));
+  for (long b = 0; b < B && r > 0; ++b)  // W_k and W_v are rows d..3d of W_qkv
+    PF_CUDA(kv_rows((int)r, (int)d, X + (b * L_hist + m * P) * d,
+                    static_cast<const bf16*>(dp->W_qkv) + d * d,
+                    static_cast<bf16*>(cache->K_open) + b * P * d,
+                    static_cast<bf16*>(cache->V_open) + b * P * d, nullptr, nullptr, 0, 0,
+                    "prefill_open_kv", cs));
+  PF_CUDA(prefill_tail(X, static_cast<bf16*>(cache->X_open), cache->n_open, cache->n_proxy, (int)B,
+                       (int)L_hist, (int)P, (int)d, (int)m, (int)r, cs));
   return PF_OK;
 }
 

@@ -39,8 +39,12 @@ constexpr int GEMV_MAXB = 8;      // batch rows handled per launch (the MMA's N)
 constexpr int SPLIT_STAGES = 3;  // depth of the split kernel's copy ring
 constexpr int SPLIT_STAGE_BYTES = 32768;  // K + V rows of one stage
 constexpr int MAX_SPLITS = 1024;
+// Rows up to which a K/V projection runs as matrix-vector products, 8 rows to a pass
+// over the weights: 8 rows of 2048 take 11.9 us, on 128-row tiles 16.4; 56 rows of
+// 1024 take 55 in seven passes, 13.7 on tiles.
+constexpr int KV_GEMV_ROWS = 16;
 
-enum { EPI_QKV = 0, EPI_OUT = 1 };
+enum { EPI_QKV = 0, EPI_OUT = 1, EPI_KV = 2 };
 
 __device__ __forceinline__ void load8f(const float* p, float* v) {
   const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
@@ -65,6 +69,10 @@ struct GemvArgs {
   const bf16* resid;
   bf16* y;
   const int* valid;
+  // EPI_KV: K_open / V_open are the destinations of columns [0, d) and [d, 2d), row b
+  // or, given n_proxy, cache row n_proxy[b] of sequence b if its block is full
+  const int* n_proxy;
+  int cap;
 };
 
 // y[b, n] = sum_k W[n, k] x[b, k] for b < B <= 8 on the tensor cores: one
@@ -169,6 +177,14 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_kernel(GemvArgs a) {
     } else {
       a.V_open[((long)b * a.P + slot) * a.d + (n - 2 * a.d)] = __float2bfloat16(v);
     }
+  } else if (EPI == EPI_KV) {
+    long row = b;
+    if (a.n_proxy) {
+      const int np = a.n_proxy[b];
+      if (a.n_open[b] != a.P || np < 0 || np >= a.cap) return;  // flagged by append_finish
+      row = (long)b * a.cap + np;
+    }
+    (n < a.d ? a.K_open : a.V_open)[row * a.d + (n < a.d ? n : n - a.d)] = __float2bfloat16(v);
   } else {
     if (!a.valid[b]) return;  // flagged: y left untouched
     a.y[(long)b * a.N + n] = __float2bfloat16(__bfloat162float(a.resid[(long)b * a.N + n]) + v);
@@ -572,20 +588,58 @@ cudaError_t decode_step_launch(const DecodeLaunch& L, cudaStream_t st) {
   return cudaSuccess;
 }
 
-// Prefill: every sequence's cache holds m proxies and r open tokens.
-__global__ void prefill_counts_kernel(int* n_open, int* n_proxy, int B, int m, int r) {
+// Prefill: every sequence's cache holds m proxies and r open tokens, the last r of
+// its L, whose features are copied to X_open.  CTA (b, c): 16-byte pieces of
+// sequence b.
+__global__ void prefill_tail_kernel(const bf16* __restrict__ X, bf16* __restrict__ X_open, int* n_open,
+                                    int* n_proxy, int L, int P, int d, int m, int r) {
   const int pz = pdl_enter();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x + pz;
-  if (b < B) {
+  const int b = blockIdx.x + pz;
+  if (blockIdx.y == 0 && threadIdx.x == 0) {
     n_proxy[b] = m;
     n_open[b] = r;
   }
+  const long i = ((long)blockIdx.y * blockDim.x + threadIdx.x) * 8;
+  if (i < (long)r * d)
+    *reinterpret_cast<uint4*>(X_open + (long)b * P * d + i) =
+        *reinterpret_cast<const uint4*>(X + ((long)b * L + L - r) * d + i);
 }
 
-cudaError_t prefill_counts(int* n_open, int* n_proxy, int B, int m, int r, cudaStream_t st) {
-  LaunchTimer lt("prefill_counts", st, 0.0, 8.0 * B);
-  return launch_kernel(prefill_counts_kernel, (B + 127) / 128, 128, 0, st, n_open, n_proxy, B, m,
+cudaError_t prefill_tail(const bf16* X, bf16* X_open, int* n_open, int* n_proxy, int B, int L, int P,
+                         int d, int m, int r, cudaStream_t st) {
+  LaunchTimer lt("prefill_tail", st, 0.0, 4.0 * B * r * d);
+  const dim3 grid(B, (unsigned)std::max(1L, ((long)r * d / 8 + 255) / 256));
+  return launch_kernel(prefill_tail_kernel, grid, 256, 0, st, X, X_open, n_open, n_proxy, L, P, d, m,
                        r);
+}
+
+cudaError_t kv_rows(int M, int d, const bf16* x, const bf16* W, bf16* K, bf16* V, const int* n_open,
+                    const int* n_proxy, int P, int cap, const char* tag, cudaStream_t st) {
+  if (M > KV_GEMV_ROWS) {
+    EpiAppendArgs e{K, V, n_open, n_proxy, d, P, cap};
+    set_gemm_tag(tag, (double)M * 2 * d * 2.0);
+    return gemm_append_kv(M, 2 * d, d, {x, d, 0}, {W, d, 0}, e, st);
+  }
+  for (int b0 = 0; b0 < M; b0 += GEMV_MAXB) {
+    GemvArgs g{};
+    const long o = (long)b0 * d * (n_proxy ? cap : 1);
+    g.W = W;
+    g.x = x + (long)b0 * d;
+    g.B = std::min(GEMV_MAXB, M - b0);
+    g.N = 2 * d;
+    g.K = g.d = d;
+    g.K_open = K + o;
+    g.V_open = V + o;
+    g.n_open = n_proxy ? n_open + b0 : nullptr;
+    g.n_proxy = n_proxy ? n_proxy + b0 : nullptr;
+    g.P = P;
+    g.cap = cap;
+    LaunchTimer lt(tag, st, 4.0 * g.B * d * (double)d, 4.0 * d * (double)d + 6.0 * g.B * d);
+    const cudaError_t e = launch_kernel(gemv_kernel<EPI_KV>, (2 * d + 15) / 16, GEMV_WARPS * 32, 0,
+                                        st, g);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t append_finish(int* n_open, int* n_proxy, int B, int P, int cap, cudaStream_t st) {

@@ -257,6 +257,7 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ part, int S, int 
   const long row = i / N;
   const int col = (int)(i % N);
   float4 v = *reinterpret_cast<const float4*>(part + i);
+#pragma unroll 8
   for (int s = 1; s < S; ++s) {
     const float4 w = *reinterpret_cast<const float4*>(part + (long)s * M * N + i);
     v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;

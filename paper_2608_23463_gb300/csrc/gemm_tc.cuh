@@ -913,7 +913,8 @@ struct EpiDX1D : EpiRowsBase {
 
 // KV append (Sec. 3.8): rows are sequences b, columns [0, 2d) the proxy's key
 // and value rows W_kh H and W_vh H, written as bf16 at cache row n_proxy[b] of
-// the sequences whose open block is full and whose cache has room.
+// the sequences whose open block is full and whose cache has room; without n_proxy,
+// row by row.
 struct EpiAppendKV : EpiBase {
   struct Row {
     bool ok;
@@ -925,7 +926,10 @@ struct EpiAppendKV : EpiBase {
   int d, P, cap;
   __device__ __forceinline__ Row row_info(int row, int) const {
     Row r{false, 0};
-    if (row < M) {
+    if (row < M && !n_proxy) {
+      r.ok = true;
+      r.off = (long)row * d;
+    } else if (row < M) {
       const int np = n_proxy[row];
       r.ok = n_open[row] == P && np >= 0 && np < cap;
       r.off = ((long)row * cap + (r.ok ? np : 0)) * d;

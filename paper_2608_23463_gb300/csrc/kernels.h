@@ -227,7 +227,12 @@ int decode_splits(int B, int nh, int cap);
 cudaError_t decode_step_launch(const DecodeLaunch& L, cudaStream_t st);
 cudaError_t append_finish(int* n_open, int* n_proxy, int B, int P, int cap, cudaStream_t st);
 // n_proxy[b] = m, n_open[b] = r for every sequence (bulk prefill)
-cudaError_t prefill_counts(int* n_open, int* n_proxy, int B, int m, int r, cudaStream_t st);
+cudaError_t prefill_tail(const bf16* X, bf16* X_open, int* n_open, int* n_proxy, int B, int L, int P,
+                         int d, int m, int r, cudaStream_t st);
+// [K | V] rows = x [M, d] W^T, W [2d, d]: to rows 0..M-1 of K and V or, given n_proxy
+// (and n_open, P, cap), to cache row n_proxy[b] of each sequence b whose block is full.
+cudaError_t kv_rows(int M, int d, const bf16* x, const bf16* W, bf16* K, bf16* V, const int* n_open,
+                    const int* n_proxy, int P, int cap, const char* tag, cudaStream_t st);
 
 // 2D bf16 TMA map over a row-major [outer, inner] matrix (ld elements per
 // row), 128-byte swizzle, zero fill outside; box box_inner x box_outer.
