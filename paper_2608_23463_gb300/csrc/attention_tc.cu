@@ -3,20 +3,23 @@
 //
 // Work item = (two consecutive 128-query tiles A and B, head, sequence); one
 // persistent CTA per SM walks the items heaviest first.  Two softmax warp
-// groups, one per query tile, take turns on the SM's exponential unit (SFU):
-// while one evaluates the exponentials of its tile, the other loads its next
-// scores, finds their maximum and stores its probabilities, so the SFU -- the
-// bound of a 64-wide head, 16384 exponentials per 128 x 128 tile against 512
-// cycles of MMAs -- stays busy.
+// groups, one per query tile, take turns on the tensor cores and the SM's
+// exponential unit (SFU): while one evaluates the exponentials of its tile, the
+// other waits for its scores, finds their maximum and stores its probabilities.
 //   warp 0    TMA producer: the item's two Q tiles (double-buffered across
 //             items) and a FA_STAGES-deep ring of (K, V) 128-key tiles, shared
 //             by both query tiles
 //   warp 1    MMA issuer: S_w = Q_w K_j^T (M=128, N=128, K=64) into tile w's
 //             TMEM score buffer, and O_w += P_w V_j (M=128, N=64, K=128) with
 //             P_w read from TMEM (only V comes from shared memory)
-//   warps 2-5 softmax group A, warps 6-9 group B: one query row per thread
-//             (TMEM lane); the 128 scores are loaded once into registers,
-//             P_j = 2^(s - m) goes back to TMEM as bf16 pairs
+//   warps 4-7 softmax group A, warps 8-11 group B: one query row per thread
+//             (TMEM lane); the 128 scores are loaded once into registers and
+//             freed at once, so the tile's next score MMAs run beside the
+//             exponentials; P_j = 2^(s - m) goes back to TMEM as bf16 pairs
+// A pair of tiles takes about 2660 cycles, 2540 of them MMAs (an M = 128, N = 64
+// MMA with its A from TMEM costs what N = 128 costs).  With the scores read twice,
+// and freed after the exponentials, 16384 causal proxies of 8 heads took 425 us, 303
+// so; 131072 tokens of 16 heads against 2048 proxies 1036 us, 756 so.
 // O accumulates in TMEM across the key tiles.  A row's probabilities are
 // taken against a reference m: the maximum of its first key tile, raised only
 // when a later tile's maximum exceeds it by more than FA_RESCALE (log2
@@ -44,13 +47,18 @@ constexpr int FA_M = 128;  // query rows per tile (TMEM lanes)
 constexpr int FA_N = 128;  // keys per tile
 constexpr int FA_D = 64;   // head width
 constexpr int FA_STAGES = 4;
-constexpr int FA_THREADS = 320;  // producer, MMA, two softmax groups of four warps
+constexpr int FA_THREADS = 384;  // producer, MMA, two idle warps, two softmax groups of four
+// A softmax thread holds a row's 128 scores: the control warps give registers up.
+// 168 x 384 at launch = 72 x 128 + 216 x 256.
+constexpr int FA_REGS_CTRL = 88, FA_REGS_ROWS = 208;
+static_assert(FA_REGS_CTRL * 128 + FA_REGS_ROWS * 256 == 168 * FA_THREADS, "register split");
 constexpr float FA_RESCALE = 8.f;
 constexpr uint32_t FA_Q_BYTES = FA_M * FA_D * 2;   // 16 KB
 constexpr uint32_t FA_KV_BYTES = FA_N * FA_D * 2;  // 16 KB each of K and V
 constexpr uint32_t FA_OFF_KV = 4 * FA_Q_BYTES;     // Q: [2 items][tiles A, B]
 constexpr uint32_t FA_OFF_BAR = FA_OFF_KV + FA_STAGES * 2 * FA_KV_BYTES;
-constexpr uint32_t FA_SMEM = FA_OFF_BAR + 256 + 1024;
+constexpr uint32_t FA_OFF_STG = FA_OFF_BAR + 256;  // 32 output rows of each softmax warp
+constexpr uint32_t FA_SMEM = FA_OFF_STG + 8 * 32 * FA_D * 2 + 1024;
 // TMEM columns of group w: scores S at 128 w (fp32), O at 256 + 64 w (fp32),
 // P at 384 + 64 w (bf16 pairs: key 2c in the low half of column c)
 constexpr uint32_t FA_TMEM_COLS = 512;
@@ -159,129 +167,133 @@ __global__ void __launch_bounds__(FA_THREADS, 1)
   pdl_enter();  // the setup above overlaps the kernel before this one
   uint32_t kv_issued = 0, q_issued = 0;
 
-  if (warp == 0 && lane == 0) {
-    // ------------------------------------------------------------ producer
-    prefetch_tmap(&tmQ);
-    prefetch_tmap(&tmKV);
-    bool ok = true;
-    uint32_t it = 0;
-    for (int rd = 0, k = fa_rank(blockIdx.x, 0); k < a.n_items && ok;
-         k = fa_rank(blockIdx.x, ++rd), ++it) {
-      int u, h, b, n2[2];
-      fa_item(a, k, u, h, b, n2);
-      const int n = max(n2[0], n2[1]);
-      const int krow0 = b * a.Lk;
-      const uint32_t qb = it & 1;
-      if (!mbar_wait(q_empty + 8 * qb, ((it >> 1) & 1) ^ 1)) break;
-      mbar_arrive_expect_tx(q_full + 8 * qb, (n2[0] > 0 ? FA_Q_BYTES : 0u) +
-                                                 (n2[1] > 0 ? FA_Q_BYTES : 0u));
-      for (int w = 0; w < 2; ++w)
-        if (n2[w] > 0)
-          tma_load_2d(sbase + (2 * qb + w) * FA_Q_BYTES, &tmQ, q_full + 8 * qb,
-                      a.qcol + h * FA_D, b * a.Lq + (2 * u + w) * FA_M);
-      q_issued = it + 1;
-      for (int j = 0; j < n; ++j) {
-        const uint32_t g = kv_issued, st = g % FA_STAGES;
-        if (!mbar_wait(kv_empty + 8 * st, ((g / FA_STAGES) & 1) ^ 1)) {
-          ok = false;
-          break;
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(FA_REGS_CTRL));
+    if (warp == 0 && lane == 0) {
+      // ------------------------------------------------------------ producer
+      prefetch_tmap(&tmQ);
+      prefetch_tmap(&tmKV);
+      bool ok = true;
+      uint32_t it = 0;
+      for (int rd = 0, k = fa_rank(blockIdx.x, 0); k < a.n_items && ok;
+           k = fa_rank(blockIdx.x, ++rd), ++it) {
+        int u, h, b, n2[2];
+        fa_item(a, k, u, h, b, n2);
+        const int n = max(n2[0], n2[1]);
+        const int krow0 = b * a.Lk;
+        const uint32_t qb = it & 1;
+        if (!mbar_wait(q_empty + 8 * qb, ((it >> 1) & 1) ^ 1)) break;
+        mbar_arrive_expect_tx(q_full + 8 * qb, (n2[0] > 0 ? FA_Q_BYTES : 0u) +
+                                                   (n2[1] > 0 ? FA_Q_BYTES : 0u));
+        for (int w = 0; w < 2; ++w)
+          if (n2[w] > 0)
+            tma_load_2d(sbase + (2 * qb + w) * FA_Q_BYTES, &tmQ, q_full + 8 * qb,
+                        a.qcol + h * FA_D, b * a.Lq + (2 * u + w) * FA_M);
+        q_issued = it + 1;
+        for (int j = 0; j < n; ++j) {
+          const uint32_t g = kv_issued, st = g % FA_STAGES;
+          if (!mbar_wait(kv_empty + 8 * st, ((g / FA_STAGES) & 1) ^ 1)) {
+            ok = false;
+            break;
+          }
+          const uint32_t kdst = sbase + FA_OFF_KV + st * 2 * FA_KV_BYTES;
+          mbar_arrive_expect_tx(kv_full + 8 * st, 2 * FA_KV_BYTES);
+          tma_load_2d(kdst, &tmKV, kv_full + 8 * st, a.kcol + h * FA_D, krow0 + j * FA_N);
+          tma_load_2d(kdst + FA_KV_BYTES, &tmKV, kv_full + 8 * st, a.vcol + h * FA_D,
+                      krow0 + j * FA_N);
+          kv_issued = g + 1;
         }
-        const uint32_t kdst = sbase + FA_OFF_KV + st * 2 * FA_KV_BYTES;
-        mbar_arrive_expect_tx(kv_full + 8 * st, 2 * FA_KV_BYTES);
-        tma_load_2d(kdst, &tmKV, kv_full + 8 * st, a.kcol + h * FA_D, krow0 + j * FA_N);
-        tma_load_2d(kdst + FA_KV_BYTES, &tmKV, kv_full + 8 * st, a.vcol + h * FA_D,
-                    krow0 + j * FA_N);
-        kv_issued = g + 1;
       }
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    // The whole warp runs the loop; one elected lane issues and commits.
-    constexpr uint32_t idesc_s = idesc_bf16_f32(FA_M, FA_N, 0, 0);
-    constexpr uint32_t idesc_o = idesc_bf16_f32(FA_M, FA_D, 0, 1);
-    bool ok = true;
-    uint32_t G = 0, it = 0;
-    uint32_t gs[2] = {0, 0};  // score / probability tiles of each group so far
-    uint32_t io[2] = {0, 0};  // items of each group so far
-    // O_w (+)= P_w V for key tile jj of the current item (G: its first stage)
-    auto issue_pv = [&](const int* n2, int jj) -> bool {
-      const uint32_t st = (G + jj) % FA_STAGES;
-      const uint32_t vb = sbase + FA_OFF_KV + st * 2 * FA_KV_BYTES + FA_KV_BYTES;
-      for (int w = 0; w < 2; ++w) {
-        if (jj >= n2[w]) continue;
-        const uint32_t g = gs[w] + jj;
-        if (!mbar_wait_warp(p_full(w), g & 1)) return false;
-        if (jj == 0 && io[w] > 0 && !mbar_wait_warp(o_free(w), (io[w] - 1) & 1)) return false;
-        tc_fence_after();
-        const uint32_t pt = tmem + 384 + 64 * w, ot = tmem + 256 + 64 * w;
-        if (elect_one()) {
-#pragma unroll
-          for (int kk = 0; kk < FA_N / 16; ++kk)
-            tc_mma_f16_ts(ot, pt + kk * 8, smem_desc_sw128(vb + kk * 2048, 8192, 1024), idesc_o,
-                          (jj > 0 || kk > 0) ? 1u : 0u);
-          tc_commit(p_free(w));
-          if (jj == n2[w] - 1) tc_commit(o_full(w));
-        }
-        __syncwarp();
-      }
-      if (elect_one()) tc_commit(kv_empty + 8 * st);
-      __syncwarp();
-      return true;
-    };
-    for (int rd = 0, k = fa_rank(blockIdx.x, 0); k < a.n_items && ok;
-         k = fa_rank(blockIdx.x, ++rd), ++it) {
-      int u, h, b, n2[2];
-      fa_item(a, k, u, h, b, n2);
-      const int n = max(n2[0], n2[1]);
-      const uint32_t qb = it & 1;
-      if (!mbar_wait_warp(q_full + 8 * qb, (it >> 1) & 1)) break;
-      tc_fence_after();
-      for (int j = 0; j < n && ok; ++j) {
-        const uint32_t st = (G + j) % FA_STAGES;
-        if (!mbar_wait_warp(kv_full + 8 * st, ((G + j) / FA_STAGES) & 1)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t ks = sbase + FA_OFF_KV + st * 2 * FA_KV_BYTES;
+    } else if (warp == 1) {
+      // ------------------------------------------------------------ MMA issuer
+      // The whole warp runs the loop; one elected lane issues and commits.
+      constexpr uint32_t idesc_s = idesc_bf16_f32(FA_M, FA_N, 0, 0);
+      constexpr uint32_t idesc_o = idesc_bf16_f32(FA_M, FA_D, 0, 1);
+      bool ok = true;
+      uint32_t G = 0, it = 0;
+      uint32_t gs[2] = {0, 0};  // score / probability tiles of each group so far
+      uint32_t io[2] = {0, 0};  // items of each group so far
+      // O_w (+)= P_w V for key tile jj of the current item (G: its first stage)
+      auto issue_pv = [&](const int* n2, int jj) -> bool {
+        const uint32_t st = (G + jj) % FA_STAGES;
+        const uint32_t vb = sbase + FA_OFF_KV + st * 2 * FA_KV_BYTES + FA_KV_BYTES;
         for (int w = 0; w < 2; ++w) {
-          if (j >= n2[w]) continue;
-          const uint32_t g = gs[w] + j;
-          if (g > 0 && !mbar_wait_warp(s_free(w), (g - 1) & 1)) {
+          if (jj >= n2[w]) continue;
+          const uint32_t g = gs[w] + jj;
+          if (!mbar_wait_warp(p_full(w), g & 1)) return false;
+          if (jj == 0 && io[w] > 0 && !mbar_wait_warp(o_free(w), (io[w] - 1) & 1)) return false;
+          tc_fence_after();
+          const uint32_t pt = tmem + 384 + 64 * w, ot = tmem + 256 + 64 * w;
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < FA_N / 16; ++kk)
+              tc_mma_f16_ts(ot, pt + kk * 8, smem_desc_sw128(vb + kk * 2048, 8192, 1024), idesc_o,
+                            (jj > 0 || kk > 0) ? 1u : 0u);
+            tc_commit(p_free(w));
+            if (jj == n2[w] - 1) tc_commit(o_full(w));
+          }
+          __syncwarp();
+        }
+        if (elect_one()) tc_commit(kv_empty + 8 * st);
+        __syncwarp();
+        return true;
+      };
+      for (int rd = 0, k = fa_rank(blockIdx.x, 0); k < a.n_items && ok;
+           k = fa_rank(blockIdx.x, ++rd), ++it) {
+        int u, h, b, n2[2];
+        fa_item(a, k, u, h, b, n2);
+        const int n = max(n2[0], n2[1]);
+        const uint32_t qb = it & 1;
+        if (!mbar_wait_warp(q_full + 8 * qb, (it >> 1) & 1)) break;
+        tc_fence_after();
+        for (int j = 0; j < n && ok; ++j) {
+          const uint32_t st = (G + j) % FA_STAGES;
+          if (!mbar_wait_warp(kv_full + 8 * st, ((G + j) / FA_STAGES) & 1)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t qs = sbase + (2 * qb + w) * FA_Q_BYTES;
-          if (elect_one()) {
+          const uint32_t ks = sbase + FA_OFF_KV + st * 2 * FA_KV_BYTES;
+          for (int w = 0; w < 2; ++w) {
+            if (j >= n2[w]) continue;
+            const uint32_t g = gs[w] + j;
+            if (g > 0 && !mbar_wait_warp(s_free(w), (g - 1) & 1)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t qs = sbase + (2 * qb + w) * FA_Q_BYTES;
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < FA_D / 16; ++kk)
-              tc_mma_f16(tmem + 128 * w, smem_desc_sw128(qs + kk * 32, 16, 1024),
-                         smem_desc_sw128(ks + kk * 32, 16, 1024), idesc_s, kk ? 1u : 0u);
-            tc_commit(s_full(w));
+              for (int kk = 0; kk < FA_D / 16; ++kk)
+                tc_mma_f16(tmem + 128 * w, smem_desc_sw128(qs + kk * 32, 16, 1024),
+                           smem_desc_sw128(ks + kk * 32, 16, 1024), idesc_s, kk ? 1u : 0u);
+              tc_commit(s_full(w));
+            }
+            __syncwarp();
           }
-          __syncwarp();
+          if (!ok) break;
+          if (j == n - 1) {
+            if (elect_one()) tc_commit(q_empty + 8 * qb);
+            __syncwarp();
+          }
+          if (j > 0 && !issue_pv(n2, j - 1)) ok = false;
         }
-        if (!ok) break;
-        if (j == n - 1) {
-          if (elect_one()) tc_commit(q_empty + 8 * qb);
-          __syncwarp();
-        }
-        if (j > 0 && !issue_pv(n2, j - 1)) ok = false;
+        if (!ok || !issue_pv(n2, n - 1)) break;
+        for (int w = 0; w < 2; ++w)
+          if (n2[w] > 0) {
+            gs[w] += n2[w];
+            ++io[w];
+          }
+        G += n;
       }
-      if (!ok || !issue_pv(n2, n - 1)) break;
-      for (int w = 0; w < 2; ++w)
-        if (n2[w] > 0) {
-          gs[w] += n2[w];
-          ++io[w];
-        }
-      G += n;
+      if (elect_one()) tc_commit(done);
+      __syncwarp();
     }
-    if (elect_one()) tc_commit(done);
-    __syncwarp();
-  } else if (warp >= 2) {
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(FA_REGS_ROWS));
     // ------------------------------------------------------------ softmax
-    const int w = (warp - 2) >> 2;  // group: query tile A (0) or B (1)
+    const int w = (warp - 4) >> 2;  // group: query tile A (0) or B (1)
     const int q4 = warp & 3;         // TMEM lane quarter
     const int r = q4 * 32 + lane;    // query row in the tile = TMEM lane
     const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16);
@@ -296,6 +308,9 @@ __global__ void __launch_bounds__(FA_THREADS, 1)
       if (nw == 0) continue;
       const int q = (2 * u + w) * FA_M + r;  // query index in the sequence
       const int vis = fa_vis(a, q);
+      float gx = 0.f;  // the row's gate, asked for early
+      if (a.out_g && q < a.Lq)
+        gx = __bfloat162float(a.gpre[((long)b * a.Lq + q) * a.ldg + a.gcol + h]) + a.b_a[h];
       float mref = 0.f, l = 0.f;
       for (int j = 0; j < nw; ++j, ++g) {
         if (!mbar_wait_warp(s_full(w), g & 1)) {
@@ -306,34 +321,30 @@ __global__ void __launch_bounds__(FA_THREADS, 1)
         // keys c >= lim of this tile are masked (causal diagonal or block
         // boundary, sequence end); lim <= 0 masks the whole tile
         const int lim = min(FA_N, vis - j * FA_N);
-        // the tile's row maximum (log2 units): 64 TMEM columns at a time,
-        // three-input maxima
+        // the row's scores into registers; then the next scores may replace them
+        uint32_t sc[128];
+#pragma unroll
+        for (int c = 0; c < 128; c += 32) tmem_ld32_async(ts + c, sc + c);
+#pragma unroll
+        for (int c = 0; c < 128; c += 32) tmem_wait_ld(sc + c);
+        tc_fence_before();
+        mbar_arrive_warp(s_free(w));
+        if (lim < FA_N) {
+#pragma unroll
+          for (int c = 0; c < 128; ++c)
+            if (c >= lim) sc[c] = 0xff800000u;  // -inf
+        }
+        // the row maximum (log2 units), three-input maxima
         float mt;
         {
-          float mx0 = -INFINITY, mx1 = -INFINITY;
-#pragma unroll 1
-          for (int hh = 0; hh < 2; ++hh) {
-            uint32_t ra[32], rb[32];
-            tmem_ld32_async(ts + 64 * hh, ra);
-            tmem_ld32_async(ts + 64 * hh + 32, rb);
-            tmem_wait_ld(ra);
-            tmem_wait_ld(rb);
-            if (lim >= FA_N) {
+          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-              for (int c = 0; c < 32; c += 2) {
-                mx0 = max3f(mx0, __uint_as_float(ra[c]), __uint_as_float(ra[c + 1]));
-                mx1 = max3f(mx1, __uint_as_float(rb[c]), __uint_as_float(rb[c + 1]));
-              }
-            } else {
+          for (int c = 0; c < 128; c += 8)
 #pragma unroll
-              for (int c = 0; c < 32; ++c) {
-                const float va = 64 * hh + c < lim ? __uint_as_float(ra[c]) : -INFINITY;
-                const float vb = 64 * hh + 32 + c < lim ? __uint_as_float(rb[c]) : -INFINITY;
-                mx0 = max3f(mx0, va, vb);
-              }
-            }
-          }
-          mt = fmaxf(mx0, mx1) * a.sl2;
+            for (int i = 0; i < 4; ++i)
+              mx[i] = max3f(mx[i], __uint_as_float(sc[c + 2 * i]),
+                            __uint_as_float(sc[c + 2 * i + 1]));
+          mt = fmaxf(max3f(mx[0], mx[1], mx[2]), mx[3]) * a.sl2;
         }
         // the first tile sets the reference m; later tiles raise it only by
         // more than FA_RESCALE, scaling O and the running sum
@@ -356,27 +367,19 @@ __global__ void __launch_bounds__(FA_THREADS, 1)
         float2 ps = make_float2(0.f, 0.f);
         {
           const float2 sl = make_float2(a.sl2, a.sl2), nm = make_float2(-mnew, -mnew);
-#pragma unroll 1
-          for (int hh = 0; hh < 2; ++hh) {
-            uint32_t ra[32], rb[32], pk[32];
-            tmem_ld32_async(ts + 64 * hh, ra);
-            tmem_ld32_async(ts + 64 * hh + 32, rb);
-            tmem_wait_ld(ra);
-            tmem_wait_ld(rb);
 #pragma unroll
-            for (int c = 0; c < 64; c += 2) {
-              const uint32_t* src = c < 32 ? ra + c : rb + (c - 32);
-              const float2 z = __ffma2_rn(
-                  make_float2(__uint_as_float(src[0]), __uint_as_float(src[1])), sl, nm);
-              float2 pp = make_float2(ex2_approx(z.x), ex2_approx(z.y));
-              if (lim < FA_N) {
-                if (64 * hh + c >= lim) pp.x = 0.f;
-                if (64 * hh + c + 1 >= lim) pp.y = 0.f;
-              }
+          for (int hh = 0; hh < 4; ++hh) {
+            uint32_t pk[16];
+#pragma unroll
+            for (int c = 0; c < 32; c += 2) {
+              const float2 z = __ffma2_rn(make_float2(__uint_as_float(sc[32 * hh + c]),
+                                                      __uint_as_float(sc[32 * hh + c + 1])),
+                                          sl, nm);
+              const float2 pp = make_float2(ex2_approx(z.x), ex2_approx(z.y));
               ps = __fadd2_rn(ps, pp);
               pk[c >> 1] = pack_bf16(pp.x, pp.y);
             }
-            tmem_st32(tp + 32 * hh, pk);
+            tmem_st16(tp + 16 * hh, pk);
           }
         }
         const float psum = ps.x + ps.y;
@@ -390,8 +393,6 @@ __global__ void __launch_bounds__(FA_THREADS, 1)
             tmem_st16(to + c, ov);
           }
         }
-        tc_fence_before();
-        mbar_arrive_warp(s_free(w));  // this group's scores are no longer read
         l = fmaf(l, corr, psum);
         mref = mnew;
         tmem_wait_st();
@@ -410,33 +411,34 @@ __global__ void __launch_bounds__(FA_THREADS, 1)
       tmem_wait_ld(ov + 32);
       tc_fence_before();
       mbar_arrive_warp(o_free(w));
-      if (q < a.Lq) {
-        const float inv = l > 0.f ? 1.f / l : 0.f;  // a row that sees no key: 0
-        const long row = (long)b * a.Lq + q;
-        if (a.out) {
-          bf16* op = a.out + row * a.ldo + h * FA_D;
+      const float inv = l > 0.f ? 1.f / l : 0.f;  // a row that sees no key: 0
+      // the warp's 32 rows through its own stage (16-byte piece p of row i at piece
+      // p ^ (i & 7)), so that 8 lanes store a row's 128 bytes
+      uint8_t* const stg = smem + FA_OFF_STG + (warp - 4) * 4096;
+      const int q0 = (2 * u + w) * FA_M + q4 * 32;
+      auto put = [&](bf16* dst, float f) {
 #pragma unroll
-          for (int i = 0; i < FA_D; i += 8) {
-            const float* o = reinterpret_cast<const float*>(ov + i);
-            *reinterpret_cast<uint4*>(op + i) =
-                make_uint4(pack_bf16(o[0] * inv, o[1] * inv), pack_bf16(o[2] * inv, o[3] * inv),
-                           pack_bf16(o[4] * inv, o[5] * inv), pack_bf16(o[6] * inv, o[7] * inv));
-          }
+        for (int i = 0; i < FA_D; i += 8) {
+          const float* o = reinterpret_cast<const float*>(ov + i);
+          *reinterpret_cast<uint4*>(stg + lane * 128 + (((i >> 3) ^ (lane & 7)) << 4)) =
+              make_uint4(pack_bf16(o[0] * f, o[1] * f), pack_bf16(o[2] * f, o[3] * f),
+                         pack_bf16(o[4] * f, o[5] * f), pack_bf16(o[6] * f, o[7] * f));
         }
-        if (a.out_g) {
-          const float x = __bfloat162float(a.gpre[row * a.ldg + a.gcol + h]) + a.b_a[h];
-          const float gi = inv / (1.f + __expf(-x));
-          bf16* gp = a.out_g + row * a.ldo + h * FA_D;
+        __syncwarp();
 #pragma unroll
-          for (int i = 0; i < FA_D; i += 8) {
-            const float* o = reinterpret_cast<const float*>(ov + i);
-            *reinterpret_cast<uint4*>(gp + i) =
-                make_uint4(pack_bf16(o[0] * gi, o[1] * gi), pack_bf16(o[2] * gi, o[3] * gi),
-                           pack_bf16(o[4] * gi, o[5] * gi), pack_bf16(o[6] * gi, o[7] * gi));
-          }
+        for (int i = 0; i < 32; i += 4) {
+          const int rr = i + (lane >> 3), p = lane & 7;
+          const uint4 v = *reinterpret_cast<const uint4*>(stg + rr * 128 + ((p ^ (rr & 7)) << 4));
+          if (q0 + rr < a.Lq)
+            *reinterpret_cast<uint4*>(dst + ((long)b * a.Lq + q0 + rr) * a.ldo + h * FA_D +
+                                      p * 8) = v;
         }
+        __syncwarp();
+      };
+      if (a.out) put(a.out, inv);
+      if (a.out_g) put(a.out_g, inv / (1.f + __expf(-gx)));
+      if (q < a.Lq)
         a.lse[((long)b * a.nh + h) * a.Lq + q] = l > 0.f ? mref + log2f(l) : 0.f;  // log2 units
-      }
     }
   }
   tc_fence_before();

@@ -1,4 +1,4 @@
-"""Attention backward at proxy and token counts around its 128-row tiles and
+"""Attention forward and backward at proxy and token counts around its 128-row tiles and
 128-column steps: one row, one short of, at and past a tile, several tiles; causal
 and bidirectional proxies, and tokens against proxies (cross injection) where
 block boundaries fall inside tiles and steps."""
@@ -45,3 +45,18 @@ def test_proxy_attention_backward_edges(m, mode):
 def test_cross_attention_backward_edges(L, P, mode):
     spec = S.LayerSpec(batch=2, L=L, d=128, n_heads=2, P=P, mode=mode, inject=S.INJ_CROSS)
     _check(spec, L, CROSS_TOL, CROSS_MAX_TOL)
+
+
+# one sequence ends inside a tile and another follows it: no row may spill over
+@pytest.mark.parametrize("train", [True, False])
+@pytest.mark.parametrize("L,P,inject", [(4 * 129 - 1, 4, S.INJ_GATED), (4 * 256, 4, S.INJ_GATED),
+                                        (129, 1, S.INJ_CROSS), (391, 3, S.INJ_CROSS),
+                                        (520, 130, S.INJ_CROSS), (100, 101, S.INJ_CROSS)])
+def test_attention_forward_edges(L, P, inject, train):
+    spec = S.LayerSpec(batch=3, L=L, d=128, n_heads=2, P=P, inject=inject)
+    inp = S.make_layer_inputs(spec, L)
+    lay = ProxyLayer(spec, inp)
+    Xo = lay.forward(to_device(inp["X"], torch.bfloat16), train=train)
+    pf.pf_sync_check(torch.cuda.current_stream().cuda_stream)
+    ref, _ = OL.layer_fwd(spec, inp, inp["X"])
+    assert_grad_close("X_out", Xo.float().cpu().numpy(), ref)
