@@ -361,14 +361,14 @@ cudaError_t gemm_linear(int M, int N, int K, Operand A, Operand B, const EpiLine
 cudaError_t gemm_inject1d(int M, int N, int K, Operand A, Operand B, const EpiInjectArgs& e,
                           cudaStream_t st) {
   EpiInject1D epi{{}, M, N, e.bias, e.D_save, e.X, e.X_out, e.w_x, e.w_dlt, e.b_g,
-                  e.d, e.k1, e.k2, e.m, e.L, e.shift, e.gated};
+                  e.d, e.k1, e.k2, e.m, e.L, e.shift, e.gated, FastDiv(e.k2), FastDiv(e.m), FastDiv(e.d)};
   if (A.mn || B.mn || e.d % 32 != 0) return cudaErrorInvalidValue;
   return gemm_dispatch(M, N, K, A, B, epi, st);
 }
 
 cudaError_t gemm_dx1d(int M, int N, int K, Operand A, Operand B, const EpiDXArgs& e,
                       cudaStream_t st) {
-  EpiDX1D epi{{}, M, N, e.dX, e.d, e.k1, e.k2, e.m, e.L};
+  EpiDX1D epi{{}, M, N, e.dX, e.d, e.k1, e.L, FastDiv(e.m * e.k2)};
   if (A.mn || !B.mn || e.d % 8 != 0) return cudaErrorInvalidValue;
   return gemm_dispatch(M, N, K, A, B, epi, st);
 }
@@ -382,14 +382,17 @@ cudaError_t gemm_append_kv(int M, int N, int K, Operand A, Operand B, const EpiA
 
 cudaError_t gemm_affine2d(int M, int N, int K, Operand A, Operand B, const EpiAffine2DArgs& e,
                           cudaStream_t st) {
-  EpiAffine2D epi{{}, M, e.bias, e.S_save, e.X, e.X_out, e.stats, e.d, e.patch, e.gh, e.gw, e.m};
+  EpiAffine2D epi{{}, M, e.bias, e.S_save, e.X, e.X_out, e.stats, e.d, e.patch, e.gh, e.gw, e.m,
+                  FastDiv(e.m), FastDiv(e.gw / e.patch), FastDiv(e.patch), FastDiv(e.d >> 7)};
   if (A.mn || B.mn || e.d % 128 != 0) return cudaErrorInvalidValue;
   return gemm_dispatch(M, N, K, A, B, epi, st);
 }
 
 cudaError_t gemm_dx2d(int M, int N, int K, Operand A, Operand B, const EpiDX2DArgs& e,
                       cudaStream_t st) {
-  EpiDX2D epi{{}, M, N, e.dXd, e.dX, e.d, e.patch, e.gh, e.gw, e.m};
+  EpiDX2D epi{{},   M,     N,    e.dXd,        e.dX,
+              e.d,  e.patch, e.gh, e.gw,         e.m,
+              FastDiv(e.m), FastDiv(e.gw / e.patch), FastDiv(e.patch), FastDiv(e.d)};
   if (A.mn || !B.mn || e.d % 32 != 0) return cudaErrorInvalidValue;
   return gemm_dispatch(M, N, K, A, B, epi, st);
 }

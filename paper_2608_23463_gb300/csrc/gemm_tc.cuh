@@ -145,8 +145,13 @@ constexpr int gemm_xd(bool pair) {
   return pair ? Epi::kPairDepth : 2;
 }
 template <class Epi>
+constexpr uint32_t gemm_slot_bytes() {
+  return 2048 + Epi::kParBytes;
+}
+template <class Epi>
 constexpr uint32_t gemm_stage_bytes(bool pair) {
-  return Epi::kRows ? (uint32_t)(GEMM_EPI_WARPS * gemm_xd<Epi>(pair) * 2048) : Epi::kStageBytes;
+  return Epi::kRows ? (uint32_t)(GEMM_EPI_WARPS * gemm_xd<Epi>(pair)) * gemm_slot_bytes<Epi>()
+                    : Epi::kStageBytes;
 }
 
 template <int BN, bool A_MN, bool B_MN, class Epi, bool PAIR = false>
@@ -393,7 +398,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       // pieces sp (16 bytes) of rows sr + 8 it to `mine`.  Fragments: row r's piece
       // p sits at piece p ^ (r / 2 % 4), so that neither a matrix's eight rows nor
       // the lanes' pieces meet in a bank; lane names row lane % 8 of matrix lane / 8.
-      uint8_t* const slots = epi_smem + (warp - 2) * (XD * 2048);
+      constexpr uint32_t SLOT = gemm_slot_bytes<Epi>();
+      uint8_t* const slots = epi_smem + (warp - 2) * (XD * SLOT);
       const uint32_t slots0 = smem_u32(slots);
       const uint32_t mine = Epi::kDirect ? lane * 16 : sr * 64 + ((sp ^ ((sr >> 1) & 3)) << 4);
       const uint32_t mrow = (lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4);
@@ -425,8 +431,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         if (n0 + c < N) {  // uniform
 #pragma unroll
           for (int it = 0; it < 4; ++it)
-            cp_async16(slots0 + (put % XD) * 2048 + it * 512 + mine,
+            cp_async16(slots0 + (put % XD) * SLOT + it * 512 + mine,
                        epi.src(r, it, n0, c + 8 * sp));
+          if constexpr (Epi::kParBytes > 0)
+            if (lane * 16 < (int)Epi::kParBytes)
+              cp_async16(slots0 + (put % XD) * SLOT + 2048 + lane * 16, epi.par_src(r, c, lane));
         }
       };
       int n0 = 0, nn0 = 0;
@@ -452,7 +461,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           const int c = cb + 32 * ci;
           const bool live = n0 + c < N;  // uniform
           typename Epi::Par par;
-          if (live) epi.params(par, n0, c + (Epi::kDirect ? 8 : 2) * sp);
+          if constexpr (Epi::kParBytes > 0) {
+            __syncwarp();  // the slot's last reader is done
+          } else {
+            if (live) epi.params(par, n0, c + (Epi::kDirect ? 8 : 2) * sp);
+          }
           // the pieces of the chunk AHEAD of this one
           if (ci + AHEAD < NCH)
             fetch(rows, n0, ci + AHEAD);
@@ -461,7 +474,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           cp_async_commit();
           // r[16 h + 4 g + 2 k + e]: row sr + 16 h + 8 k, column 8 g + 2 sp + e (direct:
           // column 8 sp + 2 g + e)
-          const uint32_t slot = (get % XD) * 2048;
+          const uint32_t slot = (get % XD) * SLOT;
           uint32_t r[32];
           load(trow, c, r);
           if constexpr (Epi::kDirect) {
@@ -469,6 +482,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             if (Epi::kPaired) load(trow, c + BN / 2, r2);  // belong to columns c..
             if (ci == NCH - 1) release(buf);
             cp_async_wait<AHEAD>();  // this chunk's pieces have landed
+            if constexpr (Epi::kParBytes > 0) {
+              __syncwarp();
+              if (live) epi.params(par, slots + slot + 2048, sp);
+            }
             if (live) {
 #pragma unroll
               for (int it = 0; it < 4; ++it) {
@@ -610,6 +627,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 // row of B (K-major) loaded for 128-row box j of the tile starting at output
 // column n0.  N is a multiple of 32.
 struct EpiBase {
+  static constexpr uint32_t kParBytes = 0;  // kRows: parameters of a 32-column chunk, beside its X
   static constexpr bool kRows = false;
   static constexpr bool kDirect = false;
   static constexpr int kPairDepth = 0;
@@ -619,6 +637,23 @@ struct EpiBase {
   static constexpr uint32_t kStageBytes = 0;
   __device__ __forceinline__ int b_row(int n0, int j) const { return n0 + 128 * j; }
 };
+// n / d and n % d for 0 <= n < 2^31 by a multiplication with ceil(2^(31 + l) / d), l =
+// ceil(log2 d) (Granlund and Montgomery, 1994): a tile's rows take eight divisions a lane.
+struct FastDiv {
+  uint32_t d, mul, sh;
+  explicit FastDiv(int dv) : d((uint32_t)dv), mul(0), sh(0) {
+    uint32_t l = 0;
+    while ((1ull << l) < d) ++l;
+    if (l > 0) {
+      mul = (uint32_t)(((1ull << (31 + l)) + d - 1) / d);
+      sh = l - 1;
+    }
+  }
+  __device__ __forceinline__ int div(int n) const {
+    return d == 1 ? n : (int)(__umulhi((uint32_t)n, mul) >> sh);
+  }
+};
+
 struct EpiRowsBase : EpiBase {
   static constexpr bool kRows = true;
   static constexpr int kPairDepth = 2;  // gemm_xd of a CTA pair
@@ -812,14 +847,15 @@ struct EpiInject1D : EpiRowsBase {
   bf16* X_out;
   const float *w_x, *w_dlt, *b_g;
   int d, k1, k2, m, L, shift, gated;
+  FastDiv dk2, dm, dd;  // by k2, m, d
   __device__ __forceinline__ void rows_info(Rows& r, int row, int) const {
     r.row = row;
     r.copy = 0;
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       const int rr = row + 8 * it;
-      const int a = rr % k2, prox = rr / k2;
-      const int b = prox / m, i = prox % m;
+      const int prox = dk2.div(rr), a = rr - prox * k2;
+      const int b = dm.div(prox), i = prox - b * m;
       int blk = i + shift;
       if (blk >= m) {
         blk = 0;
@@ -838,7 +874,7 @@ struct EpiInject1D : EpiRowsBase {
     const int col = n0 + c;
     ld8_f32(bias + col, p.b);
     if (gated) {
-      const int ch = col % d;
+      const int ch = col - dd.div(col) * d;
       ld8_f32(w_x + ch, p.wx);
       ld8_f32(w_dlt + ch, p.wd);
       ld8_f32(b_g + ch, p.bg);
@@ -892,13 +928,13 @@ struct EpiDX1D : EpiRowsBase {
   };
   int M, N;
   bf16* dX;
-  int d, k1, k2, m, L;
+  int d, k1, L;
+  FastDiv dper;  // by the rows of a sequence, m k2
   __device__ __forceinline__ void rows_info(Rows& r, int row, int) const {
-    const int per_seq = m * k2;
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
-      const int rr = row + 8 * it, b = rr / per_seq;
-      const long tok0 = (long)(rr % per_seq) * k1, lim = (L - tok0) * d;
+      const int rr = row + 8 * it, b = dper.div(rr);
+      const long tok0 = (long)(rr - b * (int)dper.d) * k1, lim = (L - tok0) * d;
       r.off[it] = ((long)b * L + tok0) * d;
       r.lim[it] = rr < M && lim > 0 ? (lim < N ? (int)lim : N) : 0;
     }
@@ -956,12 +992,16 @@ struct EpiAppendKV : EpiBase {
 struct EpiAffine2D : EpiRowsBase {
   static constexpr bool kDirect = true;
   static constexpr bool kPaired = true;
-  // two chunks ahead of X (K = d <= 512: the epilogue, not the ring, bounds it)
-  static constexpr int kPairDepth = 4;
+  // two chunks ahead of X (K = d <= 512: the epilogue, not the ring, bounds it), the
+  // chunk's biases with it: 16384 patches of 64 tokens, d = 512, take 989 us, with
+  // their loads in the open and eight divisions a row 1110
+  static constexpr int kPairDepth = 3;
+  static constexpr uint32_t kParBytes = 256;
   struct Rows {
     long off[4];  // element offset of (token, channel cb) in X and X_out
     float2 st[4];
     int row;
+    int pcol, pbias;  // p d + cb and 2 p d + cb
   };
   struct Par {
     float bs[8], bt[8];
@@ -973,21 +1013,26 @@ struct EpiAffine2D : EpiRowsBase {
   bf16* X_out;
   const float* stats;
   int d, patch, gh, gw, m;
-  __device__ __forceinline__ int ptok(int n0) const { return n0 / (2 * d); }
-  __device__ __forceinline__ int cbase(int n0) const { return ((n0 >> 8) % (d >> 7)) << 7; }
+  FastDiv dm, dnpw, dpatch, dch;  // by m, patches per row, patch, 128-channel slices of d
+  __device__ __forceinline__ int ptok(int n0) const { return dch.div(n0 >> 8); }
+  __device__ __forceinline__ int cbase(int n0) const {
+    return ((n0 >> 8) - ptok(n0) * (int)dch.d) << 7;
+  }
   __device__ __forceinline__ int b_row(int n0, int j) const {
     return ptok(n0) * 2 * d + j * d + cbase(n0);
   }
   __device__ __forceinline__ void rows_info(Rows& r, int row, int n0) const {
-    const int npw = gw / patch, p = ptok(n0), py = p / patch, px = p % patch, cb = cbase(n0);
+    const int p = ptok(n0), py = dpatch.div(p), px = p - py * patch, cb = cbase(n0);
     r.row = row;
+    r.pcol = p * d + cb;
+    r.pbias = r.pcol + p * d;
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       const int rr = row + 8 * it;
       r.off[it] = 0;
       r.st[it] = make_float2(0.f, 0.f);
       if (rr < M) {
-        const int b = rr / m, pr = rr % m, by = pr / npw, bx = pr % npw;
+        const int b = dm.div(rr), pr = rr - b * m, by = dnpw.div(pr), bx = pr - by * (int)dnpw.d;
         const long tok = (long)b * gh * gw + (long)(by * patch + py) * gw + bx * patch + px;
         r.off[it] = tok * d + cb;
         r.st[it] = __ldg(reinterpret_cast<const float2*>(stats) + tok);
@@ -997,12 +1042,20 @@ struct EpiAffine2D : EpiRowsBase {
   __device__ __forceinline__ const bf16* src(const Rows& r, int it, int, int c) const {
     return X + (r.row + 8 * it < M ? r.off[it] + c : 0);
   }
-  __device__ __forceinline__ void params(Par& p, int n0, int c) const {
-    const float* bs = bias + (long)ptok(n0) * 2 * d + cbase(n0) + c;
-    ld8_f32(bs, p.bs);
-    ld8_f32(bs + d, p.bt);
+  // piece `lane` of a chunk's 32 biases of s, then 32 of t; a lane's columns of it
+  __device__ __forceinline__ const float* par_src(const Rows& r, int c, int lane) const {
+    return bias + r.pbias + (lane & 8 ? d : 0) + c + 4 * (lane & 7);
   }
-  __device__ __forceinline__ void apply(const Rows& r, const Par& p, int it, int n0, int c, float* fs,
+  __device__ __forceinline__ void params(Par& p, const uint8_t* par, int sp) const {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      *reinterpret_cast<float4*>(p.bs + 4 * i) =
+          *reinterpret_cast<const float4*>(par + sp * 32 + 16 * i);
+      *reinterpret_cast<float4*>(p.bt + 4 * i) =
+          *reinterpret_cast<const float4*>(par + 128 + sp * 32 + 16 * i);
+    }
+  }
+  __device__ __forceinline__ void apply(const Rows& r, const Par& p, int it, int, int c, float* fs,
                                         const float* ft, uint4 x) const {
     const int row = r.row + 8 * it;
     if (row >= M) return;
@@ -1018,8 +1071,7 @@ struct EpiAffine2D : EpiRowsBase {
     }
     *reinterpret_cast<uint4*>(X_out + r.off[it] + c) = pack8_bf16(o);
     const long pd = (long)patch * patch * d;
-    *reinterpret_cast<uint4*>(S_save + (long)row * pd + (long)ptok(n0) * d + cbase(n0) + c) =
-        pack8_bf16(fs);
+    *reinterpret_cast<uint4*>(S_save + (long)row * pd + r.pcol + c) = pack8_bf16(fs);
   }
 };
 
@@ -1036,13 +1088,13 @@ struct EpiDX2D : EpiRowsBase {
   const bf16* dXd;
   bf16* dX;
   int d, patch, gh, gw, m;
+  FastDiv dm, dnpw, dpatch, dd;  // by m, patches per row, patch, d
   __device__ __forceinline__ void rows_info(Rows& r, int row, int) const {
-    const int npw = gw / patch;
     r.row = row;
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       const int rr = row + 8 * it;
-      const int b = rr / m, pr = rr % m, by = pr / npw, bx = pr % npw;
+      const int b = dm.div(rr), pr = rr - b * m, by = dnpw.div(pr), bx = pr - by * (int)dnpw.d;
       r.base[it] = ((long)b * gh * gw + (long)by * patch * gw + bx * patch) * d;
     }
   }
@@ -1051,7 +1103,7 @@ struct EpiDX2D : EpiRowsBase {
     return dXd + (row < M ? (long)row * N + n0 + c : 0);
   }
   __device__ __forceinline__ bf16* dst(const Rows& r, int it, int n0, int c) const {
-    const int col = n0 + c, p = col / d, py = p / patch;
+    const int col = n0 + c, p = dd.div(col), py = dpatch.div(p);
     const long ofs = ((long)py * gw + (p - py * patch)) * d + (col - p * d);
     return r.row + 8 * it < M ? dX + r.base[it] + ofs : nullptr;
   }
