@@ -393,45 +393,6 @@ __global__ void __launch_bounds__(256) attn_f32_kernel(const float* __restrict__
   }
 }
 
-// Routing + injection (Eq. inj-gate / inj-add) in fp32, four channels per
-// thread.  D is [B*m*k2, k1*d] in proxy order; token t of block i reads the
-// row of proxy i - shift.
-__global__ void inject_f32_kernel(const float* __restrict__ X, const float* __restrict__ D,
-                                  float* __restrict__ Xo, const float* __restrict__ w_x,
-                                  const float* __restrict__ w_dlt, const float* __restrict__ b_g,
-                                  long L, int d, int P, int k1, int k2, int m, int shift, int gated,
-                                  long total4) {
-  const int pz = pdl_enter();
-  const long e4 = (long)blockIdx.x * blockDim.x + threadIdx.x + pz;
-  if (e4 >= total4) return;
-  const int d4 = d >> 2;
-  const long tokg = e4 / d4;  // global token (b * L + t)
-  const int ch = (int)(e4 - tokg * d4) * 4;
-  const long b = tokg / L, t = tokg - b * L;
-  const long i = t / P, p = t - i * P;
-  const float4 x = *reinterpret_cast<const float4*>(X + e4 * 4);
-  if (i < shift) {
-    *reinterpret_cast<float4*>(Xo + e4 * 4) = x;
-    return;
-  }
-  const long prox = b * m + (i - shift);
-  const long row = prox * k2 + p / k1;
-  const float4 dv = *reinterpret_cast<const float4*>(D + row * ((long)k1 * d) + (p % k1) * d + ch);
-  float4 o;
-  if (gated) {
-    const float4 wx = *reinterpret_cast<const float4*>(w_x + ch);
-    const float4 wd = *reinterpret_cast<const float4*>(w_dlt + ch);
-    const float4 bg = *reinterpret_cast<const float4*>(b_g + ch);
-    o.x = x.x + dv.x / (1.f + expf(-(wx.x * x.x + wd.x * dv.x + bg.x)));
-    o.y = x.y + dv.y / (1.f + expf(-(wx.y * x.y + wd.y * dv.y + bg.y)));
-    o.z = x.z + dv.z / (1.f + expf(-(wx.z * x.z + wd.z * dv.z + bg.z)));
-    o.w = x.w + dv.w / (1.f + expf(-(wx.w * x.w + wd.w * dv.w + bg.w)));
-  } else {
-    o = make_float4(x.x + dv.x, x.y + dv.y, x.z + dv.z, x.w + dv.w);
-  }
-  *reinterpret_cast<float4*>(Xo + e4 * 4) = o;
-}
-
 __global__ void pad_f32_kernel(const float* __restrict__ src, float* __restrict__ dst, long L,
                                long Lp, int d, long total) {
   const int pz = pdl_enter();
@@ -585,15 +546,6 @@ cudaError_t attn_f32(const float* qkv, float* out, int B, int m, int d, int nh, 
   dim3 grid((m + ATT_Q - 1) / ATT_Q, nh, B);
   return launch_kernel(attn_f32_kernel, grid, 256, 0, st, qkv, out, m, d, causal ? 1 : 0,
                        1.0f / sqrtf(64.0f));
-}
-
-cudaError_t inject_f32(const float* X, const float* D, float* Xo, const float* w_x,
-                       const float* w_dlt, const float* b_g, int B, long L, int d, int P, int k1,
-                       int k2, int m, int shift, int gated, cudaStream_t st) {
-  const long total4 = (long)B * L * d / 4;
-  LaunchTimer lt("inject_f32", st, 0.0, 48.0 * total4);
-  return launch_kernel(inject_f32_kernel, (unsigned)((total4 + 255) / 256), 256, 0, st, X, D, Xo,
-                       w_x, w_dlt, b_g, L, d, P, k1, k2, m, shift, gated, total4);
 }
 
 cudaError_t pad_f32(const float* src, float* dst, int B, long L, long Lp, int d, cudaStream_t st) {

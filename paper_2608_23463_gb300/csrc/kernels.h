@@ -204,9 +204,6 @@ cudaError_t gemm_f32_inject(int M, int N, int K, const float* A, long lda, const
                             int k1, int k2, int m, int shift, int gated, cudaStream_t st);
 cudaError_t attn_f32(const float* qkv, float* out, int B, int m, int d, int nh, bool causal,
                      cudaStream_t st);
-cudaError_t inject_f32(const float* X, const float* D, float* Xo, const float* w_x,
-                       const float* w_dlt, const float* b_g, int B, long L, int d, int P, int k1,
-                       int k2, int m, int shift, int gated, cudaStream_t st);
 cudaError_t pad_f32(const float* src, float* dst, int B, long L, long Lp, int d, cudaStream_t st);
 
 // ---------------------------------------------------------------- decode
