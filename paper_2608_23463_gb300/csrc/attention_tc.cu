@@ -36,6 +36,7 @@
 // optional second output applies the per-head gate sigmoid(a + b_a) (the
 // ungated output is optional too, for inference).
 #include <algorithm>
+#include <atomic>
 
 #include "kernels.h"
 
@@ -468,6 +469,21 @@ int set_wait_limit_attention_tc(unsigned long long ns) { return set_wait_limit_t
 
 namespace {
 
+// The registers that the softmax warps ask for (setmaxnreg) must be in the block's
+// pool, which holds what it was launched with: else they would wait for ever.
+cudaError_t fa_registers_ok() {
+  static std::atomic<int> regs{0};  // a constant of the binary
+  int n = regs.load(std::memory_order_relaxed);
+  if (n == 0) {
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, attn_fwd_tc_kernel);
+    if (e != cudaSuccess) return e;
+    regs.store(n = at.numRegs, std::memory_order_relaxed);
+  }
+  return n * FA_THREADS >= FA_REGS_CTRL * 128 + FA_REGS_ROWS * 256 ? cudaSuccess
+                                                                    : cudaErrorInvalidConfiguration;
+}
+
 cudaError_t fa_launch(const CUtensorMap& tq, const CUtensorMap& tkv, FaArgs& a, const char* label,
                       double pairs, double bytes, cudaStream_t st) {
   a.n_qt = (a.Lq + FA_M - 1) / FA_M;
@@ -478,7 +494,9 @@ cudaError_t fa_launch(const CUtensorMap& tq, const CUtensorMap& tkv, FaArgs& a, 
   a.n_items = qt_min >= a.n_qt ? 0 : (a.n_st - a.st_min) * a.nh * a.B;
   a.sl2 = 1.4426950408889634f / sqrtf((float)FA_D);
   auto kern = attn_fwd_tc_kernel;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FA_SMEM);
+  cudaError_t e = fa_registers_ok();
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FA_SMEM);
   if (e != cudaSuccess) return e;
   LaunchTimer lt(label, st, 4.0 * FA_D * pairs, bytes);
   if (qt_min > 0) {  // query tiles that see no key: zero rows, LSE 0
