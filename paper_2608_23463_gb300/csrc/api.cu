@@ -114,6 +114,7 @@ size_t splitk_need(const pf_layer_desc& s, const Dims& g, bool bwd,
   }
   size_t m = 0;
   for (const S3& x : v) m = std::max(m, bytes(x.M, x.N, x.K));
+  if (!bwd && s.levels == 1) m = std::max(m, splitk_scratch_bytes(R, d, N1, 1));
   return m;
 }
 
@@ -492,6 +493,7 @@ pf_status layer_fwd_2d(const pf_layer_desc& s, const Dims& g, const pf_layer_par
     e.ld_add = d;
     e.out_f32 = Hf;
     e.ld_f32 = d;
+    e.exact_in = 1;
     set_gemm_tag("compress_c1", (double)g.R * d * 8.0);
     PF_CUDA(gemm_linear((int)g.R, d, N1, {sv.Xp, N1, 0}, {static_cast<const bf16*>(p.W_c1), N1, 0}, with_sk(e, sk, skb), cs));
   }
@@ -716,6 +718,7 @@ pf_status proxy_layer_fwd(const pf_layer_desc* desc, const pf_layer_params* prm,
       e.ld_f32 = d;
       e.out_bf16 = sv.Hb;
       e.ld_bf16 = d;
+      e.exact_in = 1;
       set_gemm_tag("compress_c1", (double)g.R * d * 6.0);
       PF_CUDA(gemm_linear((int)g.R, d, (int)g.N1, Xop,
                           {static_cast<const bf16*>(prm->W_c1), g.N1, 0}, with_sk(e, sk, skb), cs));

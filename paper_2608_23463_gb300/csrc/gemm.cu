@@ -154,13 +154,38 @@ double plan_cost(int M, int N, int K, int bn, bool pair, int S) {
   return waves * (kb * c + 1200.) + red;
 }
 
-// The cheapest plan whose slices' partial sums fit `bytes`: slices are at least
-// 16 K blocks deep and must promise a tenth, since a last wave that is partly
+// K slices of at least 16 blocks that fill the SMs with 128 x 128 tiles (1: the tiles
+// alone do).
+int fill_slices(int M, int N, int K) {
+  const long tiles = (long)((N + 127) / 128) * ((M + GEMM_BM - 1) / GEMM_BM);
+  const int num_k = (K + GEMM_BK - 1) / GEMM_BK;
+  if (tiles >= kPlanSms || num_k < 32) return 1;
+  int best = 1;
+  double best_eff = (double)tiles / kPlanSms;
+  for (int S = 2; S <= 16 && num_k / S >= 16; ++S) {
+    const long t = tiles * S;
+    const double eff = (double)t / (((t + kPlanSms - 1) / kPlanSms) * kPlanSms);
+    if (eff > best_eff + 1e-9) {
+      best = S;
+      best_eff = eff;
+    }
+  }
+  return best;
+}
+
+// The cheapest plan of at least min_S slices whose partial sums fit `bytes`: slices are
+// at least 16 K blocks deep and must promise a tenth, since a last wave that is partly
 // empty costs less than the model says (weight gradients of the 262144-token
 // layer, 128 pair tiles in two waves: 320 us, on four slices 321 + 33).
-Plan gemm_plan(int M, int N, int K, size_t bytes) {
+// Why min_S: each MMA cuts its 16 products' sum off at the accumulator's last bit, so a
+// slice's error grows with its depth (2-norm, about 2^-26 of the result an MMA).  Where
+// inputs are rounded to bf16 or the result is, that is lost beside 1e-3; in the proxies
+// of a one-level compression nothing else is: 2565 patches of 24576 values, d = 384, are
+// 8.9e-6 off float64 on three slices, 2.0e-6 on twelve or more.
+Plan gemm_plan(int M, int N, int K, size_t bytes, int min_S) {
   Plan best;
   const long nk = (K + GEMM_BK - 1) / GEMM_BK;
+  while (min_S > 1 && (N % 4 != 0 || (size_t)min_S * M * N * sizeof(float) > bytes)) --min_S;
   double cost = 1e300;
   for (int v = 0; v < 3; ++v) {
     const int bn = v == 0 ? 128 : 256;
@@ -168,6 +193,7 @@ Plan gemm_plan(int M, int N, int K, size_t bytes) {
     if (v > 0 && N < 256) continue;
     for (int S = 1; S <= 32 && (S == 1 || (nk / S >= 16 && v != 1)); ++S) {
       if (S > 1 && (N % 4 != 0 || (size_t)S * M * N * sizeof(float) > bytes)) break;
+      if (S < min_S) continue;
       const double c = plan_cost(M, N, K, bn, pair, S) * (S > 1 ? 1.0 / 0.9 : 1.0);
       if (c < cost) {
         cost = c;
@@ -238,7 +264,7 @@ cudaError_t gemm_dispatch(int M, int N, int K, Operand A, Operand B, const Epi& 
   if (!make_maps(&tm, Epi::kDirect, M, N, K, A, B)) return cudaErrorInvalidValue;
   LaunchTimer lt(gemm_tag_label(), st, 2.0 * M * N * (double)K,
                  2.0 * ((double)M * K + (double)N * K) + gemm_tag_bytes());
-  Plan plan = gemm_plan(M, N, K, 0);
+  Plan plan = gemm_plan(M, N, K, 0, 1);
   if constexpr (Epi::kPaired) {
     plan.bn = 256;
     plan.pair = plan_cost(M, N, K, 256, true, 1) <= plan_cost(M, N, K, 256, false, 1);
@@ -288,33 +314,22 @@ bool tmap_bf16_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t out
   return make_map(m, base, inner, outer, ld, box_inner, box_outer);
 }
 
-size_t splitk_scratch_bytes(int M, int N, int K) {
-  const int S = gemm_plan(M, N, K, ~size_t(0)).S;
+size_t splitk_scratch_bytes(int M, int N, int K, int exact_in) {
+  const int S = gemm_plan(M, N, K, ~size_t(0), exact_in ? fill_slices(M, N, K) : 1).S;
   return S > 1 ? (size_t)S * M * N * sizeof(float) : 0;
 }
+size_t splitk_scratch_bytes(int M, int N, int K) { return splitk_scratch_bytes(M, N, K, 0); }
 
 size_t splitk_scratch_least(int M, int N, int K) {
-  const long tiles = (long)((N + 127) / 128) * ((M + GEMM_BM - 1) / GEMM_BM);
-  const int num_k = (K + GEMM_BK - 1) / GEMM_BK;
-  if (tiles >= kPlanSms || num_k < 32) return 0;
-  int best = 1;
-  double best_eff = (double)tiles / kPlanSms;
-  for (int S = 2; S <= 16 && num_k / S >= 16; ++S) {
-    const long t = tiles * S;
-    const double eff = (double)t / (((t + kPlanSms - 1) / kPlanSms) * kPlanSms);
-    if (eff > best_eff + 1e-9) {
-      best = S;
-      best_eff = eff;
-    }
-  }
-  return best > 1 ? (size_t)best * M * N * sizeof(float) : 0;
+  const int S = fill_slices(M, N, K);
+  return S > 1 ? (size_t)S * M * N * sizeof(float) : 0;
 }
 
 cudaError_t gemm_linear(int M, int N, int K, Operand A, Operand B, const EpiLinearArgs& e,
                         cudaStream_t st) {
   Plan plan;
   if (e.splitk_scratch && !e.act_silu && !e.pre_bf16 && !e.dsilu_of)
-    plan = gemm_plan(M, N, K, e.splitk_bytes);
+    plan = gemm_plan(M, N, K, e.splitk_bytes, e.exact_in ? fill_slices(M, N, K) : 1);
   const int S = plan.S;
   if (S > 1) {
     // deterministic split-K: raw partials, then one reduce applying the epilogue

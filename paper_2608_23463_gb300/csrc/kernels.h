@@ -75,11 +75,15 @@ struct EpiLinearArgs {
   // alone cannot fill the GPU and splitk_scratch_bytes() bytes are given)
   float* splitk_scratch = nullptr;
   size_t splitk_bytes = 0;
+  // A and B are inputs as given and the fp32 result is an output, so that nothing but
+  // the sums over K rounds: at least fill_slices() slices
+  int exact_in = 0;
 };
 // fp32 scratch of an M x N x K linear GEMM's split-K (0: it is not split) at the
 // tiling it takes when given enough, and the least that a caller short of memory
 // should give (it splits as far as that goes); independent of the device.
-size_t splitk_scratch_bytes(int M, int N, int K);
+size_t splitk_scratch_bytes(int M, int N, int K, int exact_in);
+size_t splitk_scratch_bytes(int M, int N, int K);  // exact_in = 0
 size_t splitk_scratch_least(int M, int N, int K);
 
 struct EpiInjectArgs {
