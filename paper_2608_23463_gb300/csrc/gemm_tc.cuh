@@ -229,7 +229,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   if (PAIR) cluster_sync_all();  // both CTAs' barriers exist before any remote arrival
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  pdl_enter();  // the setup above overlaps the kernel before this one
+  // the setup above overlaps the kernel before this one; every address that is read
+  // follows from the tile, and with it from the wait
+  const int first = unit + pdl_enter();
   uint32_t issued = 0;
 
   if (warp == 0 && lane == 0) {
@@ -241,7 +243,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     const bool skip_loads = *(volatile int*)&g_debug_skip_loads != 0;
     uint32_t it = 0;
     bool ok = true;
-    for (int tile = unit; tile < tiles && ok; tile += n_units) {
+    for (int tile = first; tile < tiles && ok; tile += n_units) {
       PF_TILE_DECODE(tile)
       (void)sp;
       for (int kt = kb; kt < ke; ++kt, ++it) {
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     constexpr uint32_t idesc = idesc_bf16_f32(TILE_M, BN, A_MN ? 1 : 0, B_MN ? 1 : 0);
     uint32_t it = 0, lt = 0;
     bool ok = true;
-    for (int tile = unit; tile < tiles && ok; tile += n_units, ++lt) {
+    for (int tile = first; tile < tiles && ok; tile += n_units, ++lt) {
       const uint32_t buf = lt & 1, use = lt >> 1;
       if (!mbar_wait_warp(tempty0 + 8 * buf, (use & 1) ^ 1)) break;
       tc_fence_after();
@@ -442,15 +444,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         }
       };
       int n0 = 0, nn0 = 0;
-      if (unit < tiles) {
-        n0 = info(unit, rows);
+      if (first < tiles) {
+        n0 = info(first, rows);
 #pragma unroll
         for (int ci = 0; ci < AHEAD; ++ci, ++put) {
           fetch(rows, n0, ci);
           cp_async_commit();
         }
       }
-      for (int tile = unit; tile < tiles; tile += n_units, ++lt) {
+      for (int tile = first; tile < tiles; tile += n_units, ++lt) {
         const uint32_t buf = lt & 1, use = lt >> 1;
         const bool more = tile + n_units < tiles;
         if (more) {
@@ -539,7 +541,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       }
       cp_async_wait<0>();
     } else {
-      for (int tile = unit; tile < tiles; tile += n_units, ++lt) {
+      for (int tile = first; tile < tiles; tile += n_units, ++lt) {
         PF_TILE_DECODE(tile)
         const bool no_k = ke <= kb;
         const uint32_t buf = lt & 1, use = lt >> 1;
