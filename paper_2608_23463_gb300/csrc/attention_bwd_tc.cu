@@ -21,6 +21,8 @@
 // the tensor pipe always has one or the other.  E stays in TMEM as the A operand
 // of the accumulating MMAs, so those read only their B tile from shared memory.
 // Every wait is bounded.
+// A tile's rows past the end of its sequence read as zero: a masked column has P = 0, and
+// 0 times another sequence's infinity or NaN would reach this sequence's gradients.
 // What bounds it and why 128 streamed columns a step: an M=128 K=16 MMA takes
 // ~107 cycles at N=128 and hardly less at N=64, and the hand-offs of a step
 // (barriers, TMEM round trips) cost the same.  Steps of 64 with T and E double-
@@ -202,14 +204,13 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
     for (int rd = 0; k < a.n_items && ok; k = bw_rank(blockIdx.x, ++rd), ++it) {
       int t, h, b, j0, n;
       bw_item<DKDV>(a, k, t, h, b, j0, n);
-      const int row0 = b * a.Lx;
       const uint32_t xb = it & 1;
       if (!mbar_wait_warp(x_empty + 8 * xb, ((it >> 1) & 1) ^ 1)) break;
       if (lane == 0) {
         const uint32_t xdst = sbase + xb * 2 * BW_X_BYTES;
         mbar_arrive_expect_tx(x_full + 8 * xb, 2 * BW_X_BYTES);
-        tma_load_2d(xdst, &tmX1, x_full + 8 * xb, x1c + h * BW_D, row0 + t * BW_M);
-        tma_load_2d(xdst + BW_X_BYTES, &tmX2, x_full + 8 * xb, x2c + h * BW_D, row0 + t * BW_M);
+        tma_load_3d(xdst, &tmX1, x_full + 8 * xb, x1c + h * BW_D, t * BW_M, b);
+        tma_load_3d(xdst + BW_X_BYTES, &tmX2, x_full + 8 * xb, x2c + h * BW_D, t * BW_M, b);
       }
       x_issued = it + 1;
       for (int j = 0; j < n; ++j) {
@@ -225,10 +226,10 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
         }
         if (lane == 0) {
           const uint32_t ydst = sbase + BW_OFF_Y + st * 2 * BW_Y_BYTES;
-          const int yrow = b * a.Ly + (j0 + j) * BW_N;
+          const int yrow = (j0 + j) * BW_N;
           mbar_arrive_expect_tx(y_full + 8 * st, 2 * BW_Y_BYTES);
-          tma_load_2d(ydst, &tmY1, y_full + 8 * st, y1c + h * BW_D, yrow);
-          tma_load_2d(ydst + BW_Y_BYTES, &tmY2, y_full + 8 * st, y2c + h * BW_D, yrow);
+          tma_load_3d(ydst, &tmY1, y_full + 8 * st, y1c + h * BW_D, yrow, b);
+          tma_load_3d(ydst + BW_Y_BYTES, &tmY2, y_full + 8 * st, y2c + h * BW_D, yrow, b);
         }
         y_issued = G + 1;
         if (DKDV) {  // the pairs of the next step (this item's or the next item's first)
@@ -523,11 +524,10 @@ cudaError_t attn_bwd_tc(const bf16* qkv, const bf16* dO, const float* lse, const
                         bf16* dqkv, int B, int m, int d, int nh, bool causal, cudaStream_t st) {
   if (d != nh * BW_D || ((uintptr_t)qkv & 15) || ((uintptr_t)dO & 15) || ((uintptr_t)dqkv & 15))
     return cudaErrorInvalidValue;
-  const uint64_t rows = (uint64_t)B * m;
   static_assert(BW_M == BW_N, "one tensor map serves stationary and streamed tiles");
   CUtensorMap tqkv, tdo;
-  if (!tmap_bf16_2d(&tqkv, qkv, 3ull * d, rows, 3ull * d, 64, BW_M) ||
-      !tmap_bf16_2d(&tdo, dO, (uint64_t)d, rows, (uint64_t)d, 64, BW_M))
+  if (!tmap_bf16_seq(&tqkv, qkv, 3ull * d, m, B, 3ull * d, 64, BW_M) ||
+      !tmap_bf16_seq(&tdo, dO, (uint64_t)d, m, B, (uint64_t)d, 64, BW_M))
     return cudaErrorInvalidValue;
   BwArgs a{};
   a.lse = lse;
@@ -560,11 +560,10 @@ cudaError_t attn_cross_bwd(const bf16* qa, long ldq, const bf16* kv, const bf16*
   if (d != nh * BW_D || P < 1 || ldq < d || ((uintptr_t)qa & 15) || ((uintptr_t)kv & 15) ||
       ((uintptr_t)dO & 15) || ((uintptr_t)dqa & 15) || ((uintptr_t)dkv & 15) || (ldq * 2) % 16)
     return cudaErrorInvalidValue;
-  const uint64_t rq = (uint64_t)B * Lq, rk = (uint64_t)B * Lk;
   CUtensorMap tqa, tkv, tdo;
-  if (!tmap_bf16_2d(&tqa, qa, (uint64_t)ldq, rq, (uint64_t)ldq, 64, BW_M) ||
-      !tmap_bf16_2d(&tkv, kv, 2ull * d, rk, 2ull * d, 64, BW_M) ||
-      !tmap_bf16_2d(&tdo, dO, (uint64_t)d, rq, (uint64_t)d, 64, BW_M))
+  if (!tmap_bf16_seq(&tqa, qa, (uint64_t)ldq, Lq, B, (uint64_t)ldq, 64, BW_M) ||
+      !tmap_bf16_seq(&tkv, kv, 2ull * d, Lk, B, 2ull * d, 64, BW_M) ||
+      !tmap_bf16_seq(&tdo, dO, (uint64_t)d, Lq, B, (uint64_t)d, 64, BW_M))
     return cudaErrorInvalidValue;
   BwArgs a{};
   a.lse = lse;

@@ -314,6 +314,19 @@ bool tmap_bf16_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t out
   return make_map(m, base, inner, outer, ld, box_inner, box_outer);
 }
 
+bool tmap_bf16_seq(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint64_t n_seq,
+                   uint64_t ld, uint32_t box_inner, uint32_t box_outer) {
+  auto fn = encode_fn();
+  if (fn == nullptr) return false;
+  cuuint64_t dims[3] = {inner, outer, n_seq};
+  cuuint64_t strides[2] = {ld * 2, outer * ld * 2};
+  cuuint32_t box[3] = {box_inner, box_outer, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 size_t splitk_scratch_bytes(int M, int N, int K, int exact_in) {
   const int S = gemm_plan(M, N, K, ~size_t(0), exact_in ? fill_slices(M, N, K) : 1).S;
   return S > 1 ? (size_t)S * M * N * sizeof(float) : 0;

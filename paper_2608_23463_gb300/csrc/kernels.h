@@ -239,6 +239,11 @@ cudaError_t kv_rows(int M, int d, const bf16* x, const bf16* W, bf16* K, bf16* V
 // row), 128-byte swizzle, zero fill outside; box box_inner x box_outer.
 bool tmap_bf16_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint64_t ld,
                   uint32_t box_inner, uint32_t box_outer);
+// The same for n_seq matrices of `outer` rows that follow one another, with the matrix
+// as the third coordinate: rows past the end of a matrix read as zero, not as the next
+// one's.
+bool tmap_bf16_seq(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint64_t n_seq,
+                   uint64_t ld, uint32_t box_inner, uint32_t box_outer);
 
 // ------------------------------------------------------------- attention
 cudaError_t attn_fwd(const bf16* qkv, bf16* out, float* lse, int B, int m, int d, int nh,

@@ -60,3 +60,25 @@ def test_attention_forward_edges(L, P, inject, train):
     pf.pf_sync_check(torch.cuda.current_stream().cuda_stream)
     ref, _ = OL.layer_fwd(spec, inp, inp["X"])
     assert_grad_close("X_out", Xo.float().cpu().numpy(), ref)
+
+
+# 64 proxies and 192 tokens: a 128-row step ends in the sequence that follows
+@pytest.mark.parametrize("mode", [S.CAUSAL_1D, S.BIDIR_1D])
+@pytest.mark.parametrize("L,P,inject", [(256, 4, S.INJ_GATED), (192, 3, S.INJ_CROSS)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_a_sequence_keeps_its_gradients_beside_a_bad_one(L, P, inject, mode, bad):
+    spec = S.LayerSpec(batch=2, L=L, d=128, n_heads=2, P=P, mode=mode, inject=inject)
+    inp = S.make_layer_inputs(spec, 31)
+    lay = ProxyLayer(spec, inp)
+    X, G = to_device(inp["X"], torch.bfloat16), to_device(inp["G"], torch.bfloat16)
+    lay.forward(X)
+    got = []
+    for fill in (None, bad):
+        if fill is not None:
+            G[1] = fill
+        dH = lay.empty_proxy()
+        got.append((lay.backward(X, G, dH_in=dH), dH))
+    pf.pf_sync_check(torch.cuda.current_stream().cuda_stream)
+    for clean, dirty in zip(*got):
+        assert torch.equal(clean[0], dirty[0])
+        assert not torch.isfinite(dirty[1]).all()
