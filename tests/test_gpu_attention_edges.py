@@ -9,7 +9,7 @@ import paper_2608_23463_gb300 as pf
 import pf_synth as S
 from oracle import layer as OL
 from paper_2608_23463_gb300.layer import ProxyLayer, to_device
-from tests._util import CROSS_MAX_TOL, CROSS_TOL, assert_grad_close
+from tests._util import BF16_MAX_TOL, BF16_TOL, CROSS_MAX_TOL, CROSS_TOL, assert_grad_close
 
 pytestmark = pytest.mark.gpu
 
@@ -33,10 +33,14 @@ def _check(spec, seed, tol, max_tol):
 @pytest.mark.parametrize("mode", [S.CAUSAL_1D, S.BIDIR_1D])
 @pytest.mark.parametrize("m", [2, 127, 128, 129, 300])
 def test_proxy_attention_backward_edges(m, mode):
-    # four-token blocks: the gradients are held to the cross injection's bar, whose bf16
-    # floor is as high
+    # two proxies: rounding the oracle's intermediates to bf16 moves the gradient of W_qkv by
+    # 1.0e-2 (RMS) and 1.1e-1 (max), past the layer's bars' margin; the cross injection's are
+    # about twice that.  From 127 proxies on it is 8.5e-3 and 7.5e-2 in any gradient.
     spec = S.LayerSpec(batch=2, L=4 * m - 1, d=128, n_heads=2, P=4, mode=mode)
-    _check(spec, m, CROSS_TOL, CROSS_MAX_TOL)
+    if m == 2:
+        _check(spec, m, CROSS_TOL, CROSS_MAX_TOL)
+    else:
+        _check(spec, m, BF16_TOL, BF16_MAX_TOL)
 
 
 @pytest.mark.parametrize("L,P,mode", [(129, 1, S.CAUSAL_1D), (257, 3, S.CAUSAL_1D),

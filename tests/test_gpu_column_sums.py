@@ -16,8 +16,11 @@ pytestmark = pytest.mark.gpu
 ROWS = [1, 16, 17, 33, 256, 257, 1100]
 
 
-# 2048 columns: by registers | streamed, 64 rows to each of 304 chunks, then ragged
-@pytest.mark.parametrize("rows,P", [(r, 8) for r in ROWS] + [(19455, 32), (19456, 32), (19500, 32)])
+# 2048 columns: by registers | streamed, 64 rows to each of 304 chunks, then ragged.  Slices
+# of 2048 columns: 64 fill 256 of 304 places, by registers; 76 fill all, streamed
+@pytest.mark.parametrize("rows,P", [(r, 8) for r in ROWS] +
+                         [(19455, 32), (19456, 32), (19500, 32), (257, 2048), (255, 2432),
+                          (256, 2432), (257, 2432)])
 def test_bias_gradient_is_the_exact_sum(rows, P):
     """Add injection: the gradient of b_d1 at token t of a block is the sum of G over
     the blocks.  G holds whole numbers of at most 8, so the sum is exact."""

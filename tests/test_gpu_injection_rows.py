@@ -19,12 +19,17 @@ SPECS = {
     "one_block": S.LayerSpec(batch=1, L=16, d=64, n_heads=1, P=16),
     "b3_ragged_k1_8": S.LayerSpec(batch=3, L=333, d=64, n_heads=1, P=32, levels=2, k1=8, k2=4),
     "b5_last_block_one_token": S.LayerSpec(batch=5, L=8 * 13 + 1, d=128, n_heads=2, P=8),
-    # 96-column output: the 128-column tile ends inside a warp's half
+    # 192 columns: of the second 128-column tile only one half of the warps has any
     "narrow_tokens": S.LayerSpec(batch=2, L=77, d=128, n_heads=2, P=3, d_fine=64),
     # 256-wide tiles on CTA pairs, two ragged sequences, the row count not a multiple of 256
     "pairs_b2_ragged": S.LayerSpec(batch=2, L=9001, d=1024, n_heads=16, P=64, levels=2, k1=8, k2=8),
     "pairs_add_bidir": S.LayerSpec(batch=1, L=12000, d=1024, n_heads=16, P=64, levels=2, k1=8, k2=8,
                                    mode=S.BIDIR_1D, inject=S.INJ_ADD),
+    # 320 and 448 columns of 256-wide tiles: the last tile's warps find 64 columns of 256, or
+    # one half whole and the other half of theirs, and fetch the next tile's rows past that
+    "pairs_last_64": S.LayerSpec(batch=1, L=99998, d=64, n_heads=1, P=5, interact=S.F_IDENTITY),
+    "pairs_last_192": S.LayerSpec(batch=2, L=70000, d=64, n_heads=1, P=7, mode=S.BIDIR_1D,
+                                  inject=S.INJ_ADD, interact=S.F_IDENTITY),
 }
 
 
