@@ -39,9 +39,12 @@ constexpr int GEMV_MAXB = 8;      // batch rows handled per launch (the MMA's N)
 constexpr int SPLIT_STAGES = 3;  // depth of the split kernel's copy ring
 constexpr int SPLIT_STAGE_BYTES = 32768;  // K + V rows of one stage
 constexpr int MAX_SPLITS = 1024;
-// Rows up to which a K/V projection runs as matrix-vector products, 8 rows to a pass
-// over the weights: 8 rows of 2048 take 11.9 us, on 128-row tiles 16.4; 56 rows of
-// 1024 take 55 in seven passes, 13.7 on tiles.
+// Rows up to which a K/V projection runs as matrix-vector products, all its groups of 8
+// rows in one launch (a launch a group: appends of 9 to 16 sequences of 256 took 16.4 us,
+// 13.8 so, and longer than on tiles, 31 us against 28, where the host launches them).
+// Whole appends, so and on 128-row tiles: 16 rows of 256 14.4 and 16.9 us, of 2048 41.6 and
+// 46.4, of 4096 55.5 and 54.7; 24 rows of 1024 19.3 and 23.1, of 2048 42.3 and 44.9, of
+// 4096 63 and 55.
 constexpr int KV_GEMV_ROWS = 16;
 
 enum { EPI_QKV = 0, EPI_OUT = 1, EPI_KV = 2 };
@@ -54,7 +57,7 @@ __device__ __forceinline__ void load8f(const float* p, float* v) {
 struct GemvArgs {
   const bf16* W;  // [N, K]
   const bf16* x;  // [B, K]
-  int B, N, K;    // B <= 8, K % 32 == 0
+  int B, N, K;    // B <= 8 (EPI_KV: 8 rows to a blockIdx.y), K % 32 == 0
   // EPI_QKV: q (fp32 [B, d]), the open-slot X/K/V rows, and the alpha tiles
   float* q;
   bf16 *X_open, *K_open, *V_open;
@@ -96,10 +99,12 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_kernel(GemvArgs a) {
   const bf16* W = second ? a.W2 : a.W;
   const int N = second ? a.N2 : a.N;
   const int n0 = (second ? blockIdx.x - nt1 : blockIdx.x) * 16;
-  const bool ra = n0 + g < N, rb = n0 + g + 8 < N, xb = g < a.B;
+  const int b0 = EPI == EPI_KV ? (int)blockIdx.y * GEMV_MAXB : 0;  // first row, and rows
+  const int nb = EPI == EPI_KV ? min(a.B - b0, GEMV_MAXB) : a.B;
+  const bool ra = n0 + g < N, rb = n0 + g + 8 < N, xb = g < nb;
   const bf16* wa = W + (long)(ra ? n0 + g : 0) * a.K + 8 * t;
   const bf16* wb = W + (long)(rb ? n0 + g + 8 : 0) * a.K + 8 * t;
-  const bf16* xr = a.x + (long)(xb ? g : 0) * a.K + 8 * t;
+  const bf16* xr = a.x + (long)(b0 + (xb ? g : 0)) * a.K + 8 * t;
   if (EPI == EPI_QKV && !second && (int)blockIdx.x < a.B) {
     // CTA b: x -> X_open[b, n_o] (or flag a full / invalid open block)
     const int b = blockIdx.x, slot = a.n_open[b];
@@ -160,7 +165,7 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_kernel(GemvArgs a) {
   __syncthreads();
   if (tid >= 16 * GEMV_MAXB) return;
   const int r = tid / GEMV_MAXB, b = tid % GEMV_MAXB, n = n0 + r;
-  if (n >= N || b >= a.B) return;
+  if (n >= N || b >= nb) return;
   float v = 0.f;
 #pragma unroll
   for (int w = 0; w < GEMV_WARPS; ++w) v += red[w][r][b];
@@ -178,11 +183,11 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_kernel(GemvArgs a) {
       a.V_open[((long)b * a.P + slot) * a.d + (n - 2 * a.d)] = __float2bfloat16(v);
     }
   } else if (EPI == EPI_KV) {
-    long row = b;
+    long row = b0 + b;
     if (a.n_proxy) {
-      const int np = a.n_proxy[b];
-      if (a.n_open[b] != a.P || np < 0 || np >= a.cap) return;  // flagged by append_finish
-      row = (long)b * a.cap + np;
+      const int np = a.n_proxy[row];
+      if (a.n_open[row] != a.P || np < 0 || np >= a.cap) return;  // flagged by append_finish
+      row = row * a.cap + np;
     }
     (n < a.d ? a.K_open : a.V_open)[row * a.d + (n < a.d ? n : n - a.d)] = __float2bfloat16(v);
   } else {
@@ -620,26 +625,21 @@ cudaError_t kv_rows(int M, int d, const bf16* x, const bf16* W, bf16* K, bf16* V
     set_gemm_tag(tag, (double)M * 2 * d * 2.0);
     return gemm_append_kv(M, 2 * d, d, {x, d, 0}, {W, d, 0}, e, st);
   }
-  for (int b0 = 0; b0 < M; b0 += GEMV_MAXB) {
-    GemvArgs g{};
-    const long o = (long)b0 * d * (n_proxy ? cap : 1);
-    g.W = W;
-    g.x = x + (long)b0 * d;
-    g.B = std::min(GEMV_MAXB, M - b0);
-    g.N = 2 * d;
-    g.K = g.d = d;
-    g.K_open = K + o;
-    g.V_open = V + o;
-    g.n_open = n_proxy ? n_open + b0 : nullptr;
-    g.n_proxy = n_proxy ? n_proxy + b0 : nullptr;
-    g.P = P;
-    g.cap = cap;
-    LaunchTimer lt(tag, st, 4.0 * g.B * d * (double)d, 4.0 * d * (double)d + 6.0 * g.B * d);
-    const cudaError_t e = launch_kernel(gemv_kernel<EPI_KV>, (2 * d + 15) / 16, GEMV_WARPS * 32, 0,
-                                        st, g);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  GemvArgs g{};
+  g.W = W;
+  g.x = x;
+  g.B = M;
+  g.N = 2 * d;
+  g.K = g.d = d;
+  g.K_open = K;
+  g.V_open = V;
+  g.n_open = n_open;
+  g.n_proxy = n_proxy;
+  g.P = P;
+  g.cap = cap;
+  LaunchTimer lt(tag, st, 4.0 * M * d * (double)d, 4.0 * d * (double)d + 6.0 * M * d);
+  const dim3 grid((2 * d + 15) / 16, (M + GEMV_MAXB - 1) / GEMV_MAXB);
+  return launch_kernel(gemv_kernel<EPI_KV>, grid, GEMV_WARPS * 32, 0, st, g);
 }
 
 cudaError_t append_finish(int* n_open, int* n_proxy, int B, int P, int cap, cudaStream_t st) {

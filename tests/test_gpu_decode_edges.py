@@ -72,3 +72,19 @@ def test_prefill_open_rows(r):
         assert_close(k, cache.s[k][:, :r].float().cpu().numpy(), ref[k][:, :r])
         assert torch.equal(before[k], cache.s[k][:, r:])
     assert cache.s["n_open"].tolist() == [r, r] and cache.s["n_proxy"].tolist() == [0, 0]
+
+
+@pytest.mark.parametrize("batch", [1, 8, 9, 16, 17])
+def test_append_kv_is_one_launch(batch):
+    """However many rows it has: a short append is bound by its launches."""
+    spec = S.DecodeSpec(batch=batch, d=192, n_heads=3, P=4, capacity=5)
+    cache = ProxyKVCache(spec, S.make_decode_params(spec, 13),
+                         S.make_decode_state(spec, 14, [0] * batch, [4] * batch))
+    pf.pf_timing_enable(True)
+    try:
+        cache.append()
+        pf.pf_sync_check(torch.cuda.current_stream().cuda_stream)
+        launches = pf.pf_timing_collect()["append_kv"]["launches"]
+    finally:
+        pf.pf_timing_enable(False)
+    assert launches == 1
