@@ -484,8 +484,6 @@ pf_status layer_fwd_2d(const pf_layer_desc& s, const Dims& g, const pf_layer_par
   const int patch = s.patch, gh = s.grid_h, gw = s.grid_w;
   float* Hf = H_out ? H_out : Hws;
   PF_CUDA(patch_gather_stats(X, sv.Xp, sv.stats, (int)g.B, d, patch, gh, gw, cs));
-  // the patch matrix (Eq. partition): X itself through the patch view, else the gathered copy
-
   {
     EpiLinearArgs e;
     e.bias = p.b_c1;
@@ -1904,7 +1902,7 @@ pf_status proxy_segments_bwd(const pf_layer_desc* desc, int32_t n_seg, const pf_
       e.out_f32 = sg[i].W_c1;
       e.ld_f32 = N1;
       set_gemm_tag("seg_bwd_dW_c1", (double)d * N1 * 4.0);
-      PF_CUDA(gemm_linear(d, N1, r1, {dYsrc, d, 1}, 
+      PF_CUDA(gemm_linear(d, N1, r1, {dYsrc, d, 1},
                           token_rows(Xb + g.off * d, g.L, N1, d, 1), with_sk(e, w.sk, w.skb), cs));
     }
     EpiDXArgs e{dXb + g.off * d, d, (int)g.k1, (int)g.k2, (int)g.m, (int)g.L};

@@ -17,20 +17,22 @@
 // 2-17 the row warps: four per TMEM lane quarter, each thread one row (TMEM
 // lane) and one quarter of the 128 streamed columns.  A thread takes its 32
 // scores and 32 dP into registers first and frees T1/T2, so the score MMAs of
-// step j+1 and the accumulating MMAs of step j-1 run while it works on step j:
-// the tensor pipe always has one or the other.  E stays in TMEM as the A operand
+// step j+1 and the accumulating MMAs of step j-1 can run while it works on step j.  E stays in TMEM as the A operand
 // of the accumulating MMAs, so those read only their B tile from shared memory.
 // Every wait is bounded.
 // A tile's rows past the end of its sequence read as zero: a masked column has P = 0, and
 // 0 times another sequence's infinity or NaN would reach this sequence's gradients.
-// What bounds it and why 128 streamed columns a step: an M=128 K=16 MMA takes
-// ~107 cycles at N=128 and hardly less at N=64, and the hand-offs of a step
-// (barriers, TMEM round trips) cost the same.  Steps of 64 with T and E double-
-// buffered took 1620 (DKDV) and 1475 (DQ) cycles each, steps of 128 take 2550 and
-// 1690, about the time of their 24 and 16 MMAs.  16384 proxies of 8 heads, causal:
-// 706 -> 555 and 642 -> 367 us; 131072 tokens against 2048 proxies, 16 heads: 1676
-// -> 1341 and 1380 -> 896.  With eight row warps (64 columns a thread) DKDV takes
-// 572 and DQ 367; scalar instead of packed arithmetic there 556 and 408.
+// What bounds it and why 128 streamed columns a step: the chain score MMAs -> row warps
+// -> accumulating MMAs, whose hand-offs (barriers, TMEM round trips) cost a step of 64
+// columns what they cost one of 128.  Steps of 64 with T and E double-buffered took 1620
+// (DKDV) and 1475 (DQ) cycles each, steps of 128 take 2550 and 1690, of which the 24 and 16
+// MMAs alone are 1244 and 989.  16384 proxies of 8 heads, causal: 706 -> 555 and 642 ->
+// 367 us; 131072 tokens against 2048 proxies, 16 heads: 1676 -> 1341 and 1380 -> 896.
+// Timed with parts left out (the former): one in eight of the accumulating MMAs 512 and
+// 322, one in four of the score MMAs 519 and 293, both 482 and 273, no arithmetic in the
+// row warps 445 and 350, no stores of E 472 and 358.
+// With eight row warps (64 columns a thread) DKDV takes 572 and DQ 367; scalar instead of
+// packed arithmetic there 556 and 408.
 //
 // The cross-attention of the injection (Eq. inj-cross) runs on the same
 // kernels: queries are tokens, keys / values proxies (separate matrices, Lq

@@ -16,10 +16,13 @@
 //             (TMEM lane); the 128 scores are loaded once into registers and
 //             freed at once, so the tile's next score MMAs run beside the
 //             exponentials; P_j = 2^(s - m) goes back to TMEM as bf16 pairs
-// A pair of tiles takes about 2660 cycles, 2540 of them MMAs (an M = 128, N = 64
-// MMA with its A from TMEM costs what N = 128 costs).  With the scores read twice,
-// and freed after the exponentials, 16384 causal proxies of 8 heads took 425 us, 303
-// so; 131072 tokens of 16 heads against 2048 proxies 1036 us, 756 so.
+// What bounds it: the chain score MMAs -> softmax -> P V MMAs of a key tile with its
+// hand-offs.  A pair of tiles takes about 2660 cycles; its 24 MMAs alone take 1242.
+// 16384 causal proxies of 8 heads, timed with parts left out: 301 us as it is, 257 with
+// one in four of the score MMAs, 266 with one in eight of the P V ones, 258 with both, 271
+// without maxima, exponentials and sums, 289 without the P stores, 304 without the
+// exponentials alone.  With the scores read twice, and freed after the exponentials, it
+// took 425 us; 131072 tokens of 16 heads against 2048 proxies 1036 us, 756 so.
 // O accumulates in TMEM across the key tiles.  A row's probabilities are
 // taken against a reference m: the maximum of its first key tile, raised only
 // when a later tile's maximum exceeds it by more than FA_RESCALE (log2
@@ -49,8 +52,8 @@ constexpr int FA_N = 128;  // keys per tile
 constexpr int FA_D = 64;   // head width
 constexpr int FA_STAGES = 4;
 constexpr int FA_THREADS = 384;  // producer, MMA, two idle warps, two softmax groups of four
-// A softmax thread holds a row's 128 scores: the control warps give registers up.
-// 168 x 384 at launch = 72 x 128 + 216 x 256.
+// A softmax thread holds a row's 128 scores: the control warps give registers up, of the
+// 168 that each thread has at launch.
 constexpr int FA_REGS_CTRL = 88, FA_REGS_ROWS = 208;
 static_assert(FA_REGS_CTRL * 128 + FA_REGS_ROWS * 256 == 168 * FA_THREADS, "register split");
 constexpr float FA_RESCALE = 8.f;

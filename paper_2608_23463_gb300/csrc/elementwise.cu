@@ -1,5 +1,6 @@
 // Bandwidth-bound kernels of the layer: injection backward with its column
-// reductions, deterministic column sums (bias gradients) and zero padding.  All accesses are 16-byte vectors over contiguous rows.
+// reductions, deterministic column sums (bias gradients) and zero padding.  All
+// accesses are 16-byte vectors over contiguous rows.
 #include <algorithm>
 
 #include "kernels.h"
@@ -538,6 +539,11 @@ cudaError_t pad_rows(const bf16* src, bf16* dst, int B, long L, long Lp, int d, 
 // ring: one wave of at most 304 CTAs (two per SM of a 152-SM part) that leaves few
 // SMs idle, at least 64 rows each.  1024 x 65536: 9 chunks, 118 us; 10 chunks, 16
 // CTAs into a second wave, 166; by registers 139.
+// The line at 272 CTAs, the sums over the chunks included, streamed and by registers: 270
+// CTAs (90 slices) 2048 rows 675 and 680 us; 256 CTAs (64 slices) 512 rows 144 and 153,
+// 1024 266 and 266, 4096 998 and 954; 256 slices 512 rows 520 and 558; 240 CTAs (120
+// slices) 256 rows 149 and 153, 2048 1001 and 931; 220 CTAs 1024 rows 515 and 429.  Fewer
+// rows a CTA would stream well too: 43 (512 x 65536) 74 and 95 us.
 long ib_stream_chunks(long M, int N) {
   if (N % IB_W != 0) return 0;
   const long slices = N / IB_W, c = 304 / slices;

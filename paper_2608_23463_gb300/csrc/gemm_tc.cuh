@@ -9,12 +9,12 @@
 // Persistent: one CTA per SM walks the 128 x BN output tiles tile = blockIdx.x
 // + k * gridDim.x (N fastest, so co-running CTAs share A panels and all of B
 // in L2; M fastest when A has at most 16 row tiles and B is wider than the
-// grid, so co-running CTAs share B tiles).  With BN = 256 and enough tiles the
-// kernel runs on CTA pairs (clusters of two): a pair owns a 256 x 256 tile,
+// grid, so co-running CTAs share B tiles).  With BN = 256 the kernel also runs
+// on CTA pairs (clusters of two; gemm_plan chooses): a pair owns a 256 x 256 tile,
 // rank 0 issues tcgen05.mma.cta_group::2 (M = 256) and each CTA stages its 128
-// rows of A and half of B, so a stage is 32 KB instead of 48 and 7 (4-5 with an
-// X tile) fit where 4 (3) did: the deeper ring hides the HBM latency of the
-// streamed operand (a mainloop measured at ~680 cycles per 64-deep K block
+// rows of A and half of B, so a stage is 32 KB instead of 48 and 7 fit where 4 did (6
+// beside a fused epilogue's X, 5 beside the affine one's): the deeper ring hides the HBM
+// latency of the streamed operand (a mainloop measured at ~680 cycles per 64-deep K block
 // with 4 stages runs at ~525 with 6, the MMAs' own time being 512).  Roles:
 //   warp 0   : TMA producer (one thread): STAGES-deep ring of 128B-swizzled
 //              64-wide K slices of A and B, continuing across tiles
@@ -624,11 +624,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 // kRows epilogues: rows_info(r, row, n0) describes a lane's rows row, row + 8,
 // row + 16, row + 24 of the tile that starts at output column n0; src(r, it, n0,
 // c) is the address of the 16 bytes that its it-th row needs for columns n0 + c
-// .. + 7 (where there are none: of any 16 bytes that can be read, so that the
-// copies need no branch).  kDirect: params(par, n0, c) reads the parameters of
-// columns n0 + c .. + 7 and apply(r, par, it, n0, c, f, x) stores them (kPaired:
-// with columns c + BN/2 in ft).  Else apply(f, x) gives an output pair and dst
-// the address of 8 output columns of a row, or null.  b_row(n0, j) is the first
+// .. + 7, or null for a row or token past the end: nothing is copied then, x is what the
+// slot held before, and what is made of it must not be stored.  kDirect: params(par,
+// n0, c) reads the parameters of columns n0 + c .. + 7 and apply(r, par, it, n0, c, f, x)
+// stores them (kPaired: with columns c + BN/2 in ft).  Else apply(f, x) gives an output
+// pair and dst the address of 8 output columns of a row, or null.  b_row(n0, j) is the first
 // row of B (K-major) loaded for 128-row box j of the tile starting at output
 // column n0.  N is a multiple of 32.
 struct EpiBase {

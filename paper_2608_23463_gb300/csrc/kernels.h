@@ -71,8 +71,7 @@ struct EpiLinearArgs {
   long ld_f32 = 0;
   bf16* out_bf16 = nullptr;
   long ld_bf16 = 0;
-  // optional scratch for deterministic split-K (used when the output tiles
-  // alone cannot fill the GPU and splitk_scratch_bytes() bytes are given)
+  // optional scratch for deterministic split-K: the plan takes the slices that fit
   float* splitk_scratch = nullptr;
   size_t splitk_bytes = 0;
   // A and B are inputs as given and the fp32 result is an output, so that nothing but
@@ -227,7 +226,7 @@ size_t decode_workspace_bytes(int B, int d, int nh, int splits);
 int decode_splits(int B, int nh, int cap);
 cudaError_t decode_step_launch(const DecodeLaunch& L, cudaStream_t st);
 cudaError_t append_finish(int* n_open, int* n_proxy, int B, int P, int cap, cudaStream_t st);
-// n_proxy[b] = m, n_open[b] = r for every sequence (bulk prefill)
+// Every sequence's last r of L tokens to X_open; n_proxy[b] = m, n_open[b] = r.
 cudaError_t prefill_tail(const bf16* X, bf16* X_open, int* n_open, int* n_proxy, int B, int L, int P,
                          int d, int m, int r, cudaStream_t st);
 // [K | V] rows = x [M, d] W^T, W [2d, d]: to rows 0..M-1 of K and V or, given n_proxy
