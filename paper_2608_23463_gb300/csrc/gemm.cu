@@ -173,19 +173,22 @@ int fill_slices(int M, int N, int K) {
   return best;
 }
 
-// The cheapest plan of at least min_S slices whose partial sums fit `bytes`: slices are
-// at least 16 K blocks deep and must promise a tenth, since a last wave that is partly
+// The cheapest plan whose slices' partial sums fit `bytes`: slices are at least
+// 16 K blocks deep and must promise a tenth, since a last wave that is partly
 // empty costs less than the model says (weight gradients of the 262144-token
-// layer, 128 pair tiles in two waves: 320 us, on four slices 321 + 33).
+// layer, 128 pair tiles in two waves: 320 us, on four slices 321 + 33).  If it has fewer
+// than min_S slices, min_S on 128 x 128 tiles.
 // Why min_S: each MMA cuts its 16 products' sum off at the accumulator's last bit, so a
 // slice's error grows with its depth (2-norm, about 2^-26 of the result an MMA).  Where
 // inputs are rounded to bf16 or the result is, that is lost beside 1e-3; in the proxies
 // of a one-level compression nothing else is: 2565 patches of 24576 values, d = 384, are
-// 8.9e-6 off float64 on three slices, 1.8e-6 on thirteen.
+// 8.9e-6 off float64 on three slices, 2.0e-6 on twelve.  Why 128 x 128 tiles then: the
+// model leaves out the partial sums' stores, which short slices of wider tiles do not hide
+// (product and sum, M 3624, N 512, K 16384: thirteen slices of 128-wide tiles 92 us, fifteen
+// of a pair's 101).
 Plan gemm_plan(int M, int N, int K, size_t bytes, int min_S) {
   Plan best;
   const long nk = (K + GEMM_BK - 1) / GEMM_BK;
-  while (min_S > 1 && (N % 4 != 0 || (size_t)min_S * M * N * sizeof(float) > bytes)) --min_S;
   double cost = 1e300;
   for (int v = 0; v < 3; ++v) {
     const int bn = v == 0 ? 128 : 256;
@@ -193,7 +196,6 @@ Plan gemm_plan(int M, int N, int K, size_t bytes, int min_S) {
     if (v > 0 && N < 256) continue;
     for (int S = 1; S <= 32 && (S == 1 || (nk / S >= 16 && v != 1)); ++S) {
       if (S > 1 && (N % 4 != 0 || (size_t)S * M * N * sizeof(float) > bytes)) break;
-      if (S < min_S) continue;
       const double c = plan_cost(M, N, K, bn, pair, S) * (S > 1 ? 1.0 / 0.9 : 1.0);
       if (c < cost) {
         cost = c;
@@ -202,6 +204,12 @@ Plan gemm_plan(int M, int N, int K, size_t bytes, int min_S) {
         best.S = S;
       }
     }
+  }
+  while (min_S > 1 && (N % 4 != 0 || (size_t)min_S * M * N * sizeof(float) > bytes)) --min_S;
+  if (best.S < min_S) {
+    best.bn = 128;
+    best.pair = false;
+    best.S = min_S;
   }
   return best;
 }
