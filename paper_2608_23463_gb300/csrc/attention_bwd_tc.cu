@@ -20,8 +20,9 @@
 // step j+1 and the accumulating MMAs of step j-1 can run while it works on step j.  E stays in TMEM as the A operand
 // of the accumulating MMAs, so those read only their B tile from shared memory.
 // Every wait is bounded.
-// A tile's rows past the end of its sequence read as zero: a masked column has P = 0, and
-// 0 times another sequence's infinity or NaN would reach this sequence's gradients.
+// A masked column has P = 0, and 0 times an infinity or NaN would reach the gradients: a
+// tile's rows past the end of its sequence read as zero, and DKDV streams from the first
+// query that sees its keys on, not from the step that holds it.
 // What bounds it and why 128 streamed columns a step: the chain score MMAs -> row warps
 // -> accumulating MMAs, whose hand-offs (barriers, TMEM round trips) cost a step of 64
 // columns what they cost one of 128.  Steps of 64 with T and E double-buffered took 1620
@@ -75,7 +76,7 @@ struct BwArgs {
   const float* Di;    // [B, nh, Lq]
   int B, Lq, Lk, d, nh, causal, P;  // P > 0: cross-attention with block size P
   int Lx, Ly;         // stationary / streamed rows per sequence
-  int n_tiles, n_steps_total, n_items;
+  int n_tiles, n_items;
   float sl2, scale;
 };
 
@@ -100,7 +101,7 @@ __device__ __forceinline__ int bw_rank(int c, int round) {
   return round * (int)gridDim.x + ((round & 1) ? (int)gridDim.x - 1 - c : c);
 }
 
-// Item k -> stationary tile t (128 rows), head, sequence, first streamed tile
+// Item k -> stationary tile t (128 rows), head, sequence, first streamed row
 // j0 and step count n.  DKDV: the keys of tile t are seen by the queries from
 // bw_first_q on, so the heaviest items have the smallest t; DQ: the largest t.
 // The host sizes n_items so that every item has n >= 1.
@@ -113,12 +114,12 @@ __device__ __forceinline__ void bw_item(const BwArgs& a, int k, int& t, int& h, 
   b = r / a.nh;
   if (DKDV) {
     t = rnk;
-    j0 = bw_first_q(a, t * BW_M) / BW_N;
-    n = a.n_steps_total - j0;
+    j0 = bw_first_q(a, t * BW_M);
+    n = (a.Ly - j0 + BW_N - 1) / BW_N;
   } else {
     t = a.n_tiles - 1 - rnk;
     j0 = 0;
-    n = min((bw_vis(a, min(t * BW_M + BW_M - 1, a.Lq - 1)) + BW_N - 1) / BW_N, a.n_steps_total);
+    n = (bw_vis(a, min(t * BW_M + BW_M - 1, a.Lq - 1)) + BW_N - 1) / BW_N;
   }
 }
 
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
     if (DKDV && k < a.n_items) {
       int t, h, b, j0, n;
       bw_item<DKDV>(a, k, t, h, b, j0, n);
-      fetch_step(b, h, j0 * BW_N);
+      fetch_step(b, h, j0);
     }
     bool ok = true;
     uint32_t it = 0;
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
         }
         if (lane == 0) {
           const uint32_t ydst = sbase + BW_OFF_Y + st * 2 * BW_Y_BYTES;
-          const int yrow = (j0 + j) * BW_N;
+          const int yrow = j0 + j * BW_N;
           mbar_arrive_expect_tx(y_full + 8 * st, 2 * BW_Y_BYTES);
           tma_load_3d(ydst, &tmY1, y_full + 8 * st, y1c + h * BW_D, yrow, b);
           tma_load_3d(ydst + BW_Y_BYTES, &tmY2, y_full + 8 * st, y2c + h * BW_D, yrow, b);
@@ -236,13 +237,13 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
         y_issued = G + 1;
         if (DKDV) {  // the pairs of the next step (this item's or the next item's first)
           if (j + 1 < n) {
-            fetch_step(b, h, (j0 + j + 1) * BW_N);
+            fetch_step(b, h, j0 + (j + 1) * BW_N);
           } else {
             const int k2 = bw_rank(blockIdx.x, rd + 1);
             if (k2 < a.n_items) {
               int t2, h2, b2, j02, n2;
               bw_item<DKDV>(a, k2, t2, h2, b2, j02, n2);
-              fetch_step(b2, h2, j02 * BW_N);
+              fetch_step(b2, h2, j02);
             }
           }
         }
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(BW_THREADS, 1)
       }
       for (int j = 0; j < n; ++j) {
         const uint32_t Gj = G + j;
-        const int c0 = (j0 + j) * BW_N;  // first streamed index of this step
+        const int c0 = j0 + j * BW_N;  // first streamed index of this step
         // DKDV: the step's (lse, Di) pairs, staged by the producer before the
         // stage's full barrier (already complete: the step's scores used it;
         // the slot is refilled only after this step's E has been consumed)
@@ -497,7 +498,6 @@ cudaError_t bw_launch(const CUtensorMap& x1, const CUtensorMap& x2, const CUtens
   a.Lx = DKDV ? a.Lk : a.Lq;
   a.Ly = DKDV ? a.Lq : a.Lk;
   a.n_tiles = (a.Lx + BW_M - 1) / BW_M;
-  a.n_steps_total = (a.Ly + BW_N - 1) / BW_N;
   a.scale = 1.0f / sqrtf((float)BW_D);
   a.sl2 = a.scale * 1.4426950408889634f;
   // stationary tiles with work: DKDV [0, hi), DQ [lo, n_tiles)

@@ -86,3 +86,25 @@ def test_a_sequence_keeps_its_gradients_beside_a_bad_one(L, P, inject, mode, bad
     for clean, dirty in zip(*got):
         assert torch.equal(clean[0], dirty[0])
         assert not torch.isfinite(dirty[1]).all()
+
+
+# token tau sees none of the proxies from block n on: block 0 sees none (n = 0), block 128 those of
+# the first 128-key tile only
+@pytest.mark.parametrize("L,P,tau,n", [(1144, 200, 0, 0), (1144, 200, 130, 0), (1144, 200, 199, 0),
+                                       (14000, 100, 12810, 128), (14000, 100, 12899, 128)])
+def test_a_bad_token_leaves_the_proxies_it_does_not_see(L, P, tau, n):
+    spec = S.LayerSpec(batch=1, L=L, d=128, n_heads=2, P=P, inject=S.INJ_CROSS,
+                       interact=S.F_IDENTITY)
+    inp = S.make_layer_inputs(spec, 37)
+    lay = ProxyLayer(spec, inp)
+    X, G = to_device(inp["X"], torch.bfloat16), to_device(inp["G"], torch.bfloat16)
+    lay.forward(X)
+    got = []
+    for bad in (False, True):
+        if bad:
+            G[0, tau] = float("nan")
+        dH = lay.empty_proxy()
+        lay.backward(X, G, dH_in=dH)
+        got.append(dH[0, n:])
+    pf.pf_sync_check(torch.cuda.current_stream().cuda_stream)
+    assert torch.equal(*got)
